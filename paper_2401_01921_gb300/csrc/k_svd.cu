@@ -24,7 +24,8 @@
 //    x_p / sigma_p on one side and the rows of J on the other.
 // Blocks of 16 or more vectors go through a column-pivoted Householder QR
 // first and the sweeps run on the rows of its triangular factor (see the QR
-// preconditioning section below); the output has the same form.
+// preconditioning section below), the sweeps there by the kernel of k_jacobi.cu
+// (jacobi_coop_kernel when a block is too long for it); the output has the same form.
 // All arithmetic is FP64.  Block reductions use a fixed order (deterministic).
 #include "tnx_internal.h"
 
@@ -463,22 +464,26 @@ __global__ void __launch_bounds__(CJT) qr_coop_kernel(const SvdQr* __restrict__ 
   }
 }
 
-// Xr[p][j] = R[p][j] = X[perm[j]][p] for j >= p (0 below the diagonal), Jr = I
+// Xr[p][j] = R[p][j] = X[perm[j]][p] for p <= j < c (0 elsewhere in the row), Jr = I
 __global__ void qr_gather_r_kernel(const SvdQr* __restrict__ qs, int nq) {
   tnx_grid_dependency();
   for (int gi = blockIdx.y; gi < nq; gi += gridDim.y) {
     const SvdQr q = qs[gi];
-    const int64_t n = (int64_t)q.c * q.c;
+    const int64_t n = (int64_t)q.c * q.ldr;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-      const int p = (int)(e / q.c), j = (int)(e % q.c);
-      q.Xr[e] = j >= p ? q.X[(int64_t)q.perm[j] * q.r + p] : 0.0;
+      const int p = (int)(e / q.ldr), j = (int)(e % q.ldr);
+      q.Xr[e] = j >= p && j < q.c ? q.X[(int64_t)q.perm[j] * q.r + p] : 0.0;
       q.Jr[e] = p == j ? 1.0 : 0.0;
+      if (j == 0) {
+        q.D[4 * p] = q.D[4 * p + 1] = 1.0;
+        q.D[4 * p + 2] = q.D[4 * p + 3] = 0.0;
+      }
     }
   }
 }
 
-// One warp per (block, vector p), after the Jacobi on the rows of R:
-// sigma_p = |Xr[p,:]|; J[p][perm[i]] = Xr[p][i] / sigma_p (the right singular
+// One warp per (block, vector p), after the Jacobi on the rows of R (both rows
+// count times the vector's factor D[4 p]): sigma_p = |Xr[p,:]|; J[p][perm[i]] = Xr[p][i] / sigma_p (the right singular
 // vector of A, 0 when sigma_p = 0); Xf[p,:] = sigma_p Q Jr[p,:]^T, with Q
 // applied as H_0 H_1 ... H_{c-1} to (Jr[p,:], 0, ..., 0).  Lane l keeps the
 // entries e = l (mod 32) of z throughout, in registers when r <= 32 VB.
@@ -490,21 +495,21 @@ __global__ void qr_apply_kernel(const SvdQr* __restrict__ qs, const int2* __rest
     const int2 gv = vecs[vi];
     const SvdQr q = qs[gv.x];
     const int p = gv.y, c = q.c, r = q.r;
-    const double* xr = q.Xr + (int64_t)p * c;
+    const double* xr = q.Xr + (int64_t)p * q.ldr;
     double s = 0.0;
     for (int i = lane; i < c; i += 32) s = fma(xr[i], xr[i], s);
     s = warp_sum(s);
-    const double sg = sqrt(s), inv = sg > 0.0 ? 1.0 / sg : 0.0;
+    const double dp = q.D[4 * p], nx = sqrt(s), sg = nx * dp, inv = nx > 0.0 ? 1.0 / nx : 0.0;
     for (int i = lane; i < c; i += 32) q.J[(int64_t)p * c + q.perm[i]] = xr[i] * inv;
     if (lane == 0) q.sigma[p] = sg;
-    const double* jr = q.Jr + (int64_t)p * c;
+    const double* jr = q.Jr + (int64_t)p * q.ldr;
     double* xf = q.Xf + (int64_t)p * r;
     if (r <= 32 * VB) {
       double z[VB];
 #pragma unroll
       for (int m = 0; m < VB; ++m) {
         const int e = lane + 32 * m;
-        z[m] = e < c ? jr[e] : 0.0;
+        z[m] = e < c ? jr[e] * dp : 0.0;
       }
       for (int k = c - 1; k >= 0; --k) {
         const double tk = q.tau[k];
@@ -529,7 +534,7 @@ __global__ void qr_apply_kernel(const SvdQr* __restrict__ qs, const int2* __rest
         if (e < r) xf[e] = sg * z[m];
       }
     } else {
-      for (int e = lane; e < r; e += 32) xf[e] = e < c ? jr[e] : 0.0;
+      for (int e = lane; e < r; e += 32) xf[e] = e < c ? jr[e] * dp : 0.0;
       for (int k = c - 1; k >= 0; --k) {
         const double tk = q.tau[k];
         if (tk == 0.0) continue;

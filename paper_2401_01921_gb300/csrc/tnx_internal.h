@@ -335,13 +335,37 @@ struct SvdQr {
   int32_t* perm;    // [c] vector at pivot position k
   double* nrm;      // [2][c] squared norms of the trailing parts, by position
   int32_t* pos;     // [2][c] vector at each position
-  double* Xr;       // c x c
-  double* Jr;       // c x c
+  double* Xr;       // c x ldr
+  double* Jr;       // c x ldr
   double* Xf;       // c x r
   double* J;        // c x c
   double* sigma;    // [c]
   int32_t c, r;
+  int32_t ldr, pad0;   // row stride of Xr and Jr (>= c)
+  double* D;        // [c][4] factor of each row of Xr and Jr, and more (JbGroup::D)
 };
+// One charge block of the block Jacobi sweeps (k_jacobi.cu): c vectors of c
+// entries (rows of X, and of the accumulator J; row stride ld even, rows 16-byte
+// aligned, entries c .. ld zero), cut into nb column blocks (nb even) of at
+// most wmax vectors: block b holds the vectors [b c / nb, (b + 1) c / nb).
+struct JbGroup {
+  double* X;
+  double* J;
+  double* D;   // [c][4]: the factor of vector v (its rows of X and J count times it; 1 at first), its
+               // reciprocal, |x_v|^2, unused
+  unsigned* ver;   // [nb]: rounds that each column block has been through, zeroed by the caller
+  int32_t c, ld, nb, wmax;
+};
+#define TNX_JB_MAXSLOTS 1024   // slots per CTA at most
+// Vectors per column block for a block of c vectors (8 at most; 0: too long for
+// shared memory, the sweeps then run on jacobi_coop_kernel).
+int tnx_jacobi_block_width(int c);
+// every sweep of every block in one cooperative launch over slots (group, slot
+// < nb / 2; every slot of every group listed once); met[ngroups * max_sweeps],
+// cnt[ngroups], *status and *sweeps_out zeroed by the caller
+cudaError_t tnx_launch_jacobi_block(const JbGroup* groups, const JbGroup* host_groups, int ngroups, const int2* slots,
+                                    int nslots, int max_sweeps, double tol, int* met, unsigned* cnt, int* status,
+                                    int* sweeps_out, cudaStream_t st);
 cudaError_t tnx_launch_jacobi_init(const SvdGroup* groups, int ngroups, cudaStream_t st);
 // the pivoted QR of every block in one cooperative launch over slots (block,
 // position); *bar and *status zeroed by the caller; cudaErrorNotSupported

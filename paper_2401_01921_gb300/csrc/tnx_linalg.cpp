@@ -178,29 +178,35 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
   // pivoted QR and the sweeps on R each in one cooperative launch
   int maxc = 0;
   int64_t nC = 0, nC2 = 0, nCR = 0;
+  for (Group* G : groups) maxc = std::max(maxc, G->c);
+  // the sweeps on column blocks in shared memory (k_jacobi.cu) want even row
+  // strides; a block too large for them keeps the rows of jacobi_coop_kernel
+  const int jw = tnx_jacobi_block_width(maxc);
+  auto row_stride = [&](const Group* G) { return jw ? G->c + (G->c & 1) : G->c; };
   for (Group* G : groups) {
-    maxc = std::max(maxc, G->c);
     nC += (G->c + 31) / 32 * 32;
-    nC2 += ((int64_t)G->c * G->c + 31) / 32 * 32;
+    nC2 += ((int64_t)G->c * row_stride(G) + 31) / 32 * 32;
     nCR += ((int64_t)G->c * G->r + 31) / 32 * 32;
   }
   std::unique_ptr<DevBuf> QD, QI, QXf;
   if (!done && maxc >= 16) {
-    QD.reset(new DevBuf(ctx, (size_t)(3 * nC + 2 * nC2) * 8));   // tau, nrm[2], Xr, Jr
+    QD.reset(new DevBuf(ctx, (size_t)(7 * nC + 2 * nC2) * 8));   // tau, nrm[2], D[4], Xr, Jr
     QI.reset(new DevBuf(ctx, (size_t)(3 * nC) * 4));             // perm, pos[2]
     QXf.reset(new DevBuf(ctx, (size_t)std::max<int64_t>(nCR, 1) * 8));
     std::vector<SvdQr> hq(ngr);
     std::vector<SvdGroup> hr(ngr);
-    std::vector<int2> qslots;
-    int64_t oc = 0, oc2 = 0, ocr = 0;
+    std::vector<JbGroup> hj(ngr);
+    std::vector<int2> qslots, jslots;
+    int64_t oc = 0, oc2 = 0, ocr = 0, nver = 0;
     for (int i = 0; i < ngr; ++i) {
       Group* G = groups[i];
       SvdQr& q = hq[i];
       q.X = dX + G->offX;
       q.tau = (double*)QD->p + oc;
       q.nrm = (double*)QD->p + nC + 2 * oc;
-      q.Xr = (double*)QD->p + 3 * nC + oc2;
-      q.Jr = (double*)QD->p + 3 * nC + nC2 + oc2;
+      q.D = (double*)QD->p + 3 * nC + 4 * oc;
+      q.Xr = (double*)QD->p + 7 * nC + oc2;
+      q.Jr = (double*)QD->p + 7 * nC + nC2 + oc2;
       q.perm = (int32_t*)QI->p + oc;
       q.pos = (int32_t*)QI->p + nC + 2 * oc;
       q.Xf = (double*)QXf->p + ocr;
@@ -208,15 +214,40 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
       q.sigma = dS + G->offS;
       q.c = G->c;
       q.r = G->r;
+      q.ldr = row_stride(G);
+      q.pad0 = 0;
+      JbGroup& b = hj[i];
+      b = JbGroup{q.Xr, q.Jr, q.D, nullptr, q.c, q.ldr, 0, 0};
+      if (jw && q.c >= 2) {
+        const int w = tnx_jacobi_block_width(q.c);
+        b.nb = 2 * ((q.c + 2 * w - 1) / (2 * w));
+        b.wmax = (q.c + b.nb - 1) / b.nb;
+        for (int s = 0; s < b.nb / 2; ++s) jslots.push_back(make_int2(i, s));
+        nver += b.nb;
+      }
       hr[i] = SvdGroup{q.Xr, q.Jr, q.sigma, G->c, G->c};
       for (int j = 0; j < G->c; ++j) qslots.push_back(make_int2(i, j));
       oc += (G->c + 31) / 32 * 32;
-      oc2 += ((int64_t)G->c * G->c + 31) / 32 * 32;
+      oc2 += ((int64_t)G->c * q.ldr + 31) / 32 * 32;
       ocr += ((int64_t)G->c * G->r + 31) / 32 * 32;
     }
     const SvdQr* dq = (const SvdQr*)up(hq.data(), hq.size() * sizeof(SvdQr));
     const SvdGroup* dr = (const SvdGroup*)up(hr.data(), hr.size() * sizeof(SvdGroup));
     const int2* dqs = (const int2*)up(qslots.data(), qslots.size() * sizeof(int2));
+    // slots of the largest blocks first, so that they land on SMs of their own;
+    // past one per SM the smallest come first, beside the largest
+    std::stable_sort(jslots.begin(), jslots.end(), [&](const int2& a, const int2& b) { return hj[a.x].c > hj[b.x].c; });
+    if (jslots.size() > 152) std::reverse(jslots.begin() + 152, jslots.end());
+    // block sweeps: [pairs above tol met, per block and sweep | arrivals per block | versions of the column blocks]
+    std::vector<int32_t> jzero(jw ? (size_t)ngr * (MAX_SWEEPS + 1) + (size_t)nver : 0, 0);
+    int* jmet = (int*)up(jzero.data(), jzero.size() * 4);
+    unsigned* ver = (unsigned*)jmet + (size_t)ngr * (MAX_SWEEPS + 1);
+    for (JbGroup& b : hj) {
+      b.ver = ver;
+      ver += b.nb;
+    }
+    const JbGroup* dj = (const JbGroup*)up(hj.data(), hj.size() * sizeof(JbGroup));
+    const int2* djs = (const int2*)up(jslots.data(), jslots.size() * sizeof(int2));
     // [QR barrier count | QR status, pad | offmax per sweep | Jacobi barrier count | Jacobi status, sweeps]
     std::vector<uint64_t> zero(MAX_SWEEPS + 4, 0);
     unsigned long long* w = (unsigned long long*)up(zero.data(), zero.size() * 8);
@@ -226,8 +257,12 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
     if (ce == cudaSuccess) {
       CUDA_CHECK(tnx_launch_qr_gather_r(dq, ngr, maxc, st));
       // the sweeps run on R: vectors of c entries
-      CUDA_CHECK(tnx_launch_jacobi_coop(dr, dslots, (int)slots.size(), maxcp, maxc, MAX_SWEEPS, 1e-13, w + 2,
-                                        w + MAX_SWEEPS + 2, jstat, jstat + 1, st));
+      if (jw)
+        CUDA_CHECK(tnx_launch_jacobi_block(dj, hj.data(), ngr, djs, (int)jslots.size(), MAX_SWEEPS, 1e-13, jmet,
+                                           (unsigned*)(jmet + (size_t)ngr * MAX_SWEEPS), jstat, jstat + 1, st));
+      else
+        CUDA_CHECK(tnx_launch_jacobi_coop(dr, dslots, (int)slots.size(), maxcp, maxc, MAX_SWEEPS, 1e-13, w + 2,
+                                          w + MAX_SWEEPS + 2, jstat, jstat + 1, st));
       CUDA_CHECK(tnx_launch_qr_apply(dq, dvecs, (int)vecs.size(), maxr, st));
       int hs[4] = {0, 0, 0, 0};
       CUDA_CHECK(cudaMemcpyAsync(hs, qstat, 4, cudaMemcpyDeviceToHost, st));
