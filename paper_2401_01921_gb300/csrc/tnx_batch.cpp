@@ -26,6 +26,7 @@ struct BStep {
   GemmGroup* dG = nullptr;
   GemmTile *dT = nullptr, *dTs = nullptr;
   int nt = 0, nts = 0;
+  int edge = 64;                // of the FP64 tiles
   StepPlan::Jobs jobs;
   KexpJob* dKJ = nullptr;       // K balancing of the split steps (every launch: all operands are new)
   int nkj = 0;
@@ -116,7 +117,7 @@ void enqueue_batch(tnx_batch& B, cudaStream_t st) {
     }
     if (B.prec == TNX_PREC_F64 || B.prec == TNX_PREC_F32) {
       ProfScope ps(c, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
-      if (B.prec == TNX_PREC_F64) CUDA_CHECK(tnx_launch_gemm_f64(s.dG, s.dT, s.nt, B.d_slots, st));
+      if (B.prec == TNX_PREC_F64) CUDA_CHECK(tnx_launch_gemm_f64(s.dG, s.dT, s.nt, s.edge, B.d_slots, st));
       else CUDA_CHECK(tnx_launch_gemm_f32(s.dG, s.dT, s.nt, B.d_slots, st));
     } else if (B.prec == TNX_PREC_TF32) {
       if (s.jobs.n) {
@@ -203,7 +204,7 @@ extern "C" tnx_status tnx_batch_create(tnx_ctx* ctx, int n, tnx_network* const* 
       bs.A = merge_tasks(*B, pa);
       bs.B = merge_tasks(*B, pb);
       std::vector<GemmGroup> gg;
-      std::vector<GemmTile> tt, ts;
+      std::vector<int> dense_g, skinny_g;
       std::vector<SliceJob> jobs;
       std::vector<KexpJob> kjobs;
       std::vector<SplitGroup> sg;
@@ -234,9 +235,9 @@ extern "C" tnx_status tnx_batch_create(tnx_ctx* ctx, int n, tnx_network* const* 
           g.c_slot = shift_slot(g.c_slot, b);
           gg.push_back(g);
         }
-        for (GemmTile t : sp.hT) { t.group += goff; tt.push_back(t); }
-        if (!sp.nftiles)   // a fused instance's skinny tiles run inside its fused tiles
-          for (GemmTile t : sp.hTs) { t.group += goff; ts.push_back(t); }
+        for (int g : sp.dense_g) dense_g.push_back(goff + g);
+        if (!sp.nftiles)   // a fused instance's skinny groups run inside its fused tiles
+          for (int g : sp.skinny_g) skinny_g.push_back(goff + g);
         bs.flops += sp.flops;
         bs.flops_skinny += sp.flops_skinny;
         if (split) {
@@ -266,6 +267,9 @@ extern "C" tnx_status tnx_batch_create(tnx_ctx* ctx, int n, tnx_network* const* 
           for (GemmTile t : sp.hST) { t.group += soff; st.push_back(t); }
         }
       }
+      // the merged launch is larger than any instance's: its tiles are chosen afresh
+      if (B->prec == TNX_PREC_F64) bs.edge = tnx_f64_edge(gg, dense_g);
+      const std::vector<GemmTile> tt = tnx_gemm_tiles(gg, dense_g, bs.edge), ts = tnx_skinny_tiles(gg, skinny_g);
       bs.dG = B->upload(gg);
       bs.dT = B->upload(tt);
       bs.nt = (int)tt.size();

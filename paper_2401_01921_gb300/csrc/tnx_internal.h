@@ -252,9 +252,10 @@ struct FusedTile {
 cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, const FusedCol* cols,
                                     int kp, int np, double* const* slots, cudaStream_t st);
 size_t tnx_fused_smem_bytes(int kp, int np);
-cudaError_t tnx_launch_gemm_f64(const GemmGroup* groups, const GemmTile* tiles, int ntiles,
+// edge: rows and columns of a tile (8 or 16; FP32: 64)
+cudaError_t tnx_launch_gemm_f64(const GemmGroup* groups, const GemmTile* tiles, int ntiles, int edge,
                                 double* const* slots, cudaStream_t st);
-// K <= 16 products, tiles of 128 rows x 64 columns (FP64)
+// K <= 16 products (FP64), tiles of 128 rows by GemmTile::pad0 columns (64 at most)
 cudaError_t tnx_launch_gemm_skinny(const GemmGroup* groups, const GemmTile* tiles, int ntiles, double* const* slots,
                                    cudaStream_t st);
 cudaError_t tnx_launch_gemm_f32(const GemmGroup* groups, const GemmTile* tiles, int ntiles,

@@ -718,6 +718,46 @@ std::vector<CopyTask> tnx_unband_tasks(const std::vector<CopyTask>& tasks) {
   return out;
 }
 
+// Edge of the FP64 product's tiles (k_gemm64.cu): 8, or 16 for launches of more than
+// 2^16 such tiles, whose list would take longer to build and copy than the smaller
+// tiles save.  One FP64 apply of the Heisenberg H_eff with tiles of 64 / 32 / 16 / 8:
+// bond dimension 150 235 / 103 / 62 / 54 us, 500 604 / 292 / 222 / 206, 1024 1419 /
+// 1169 / 1017 / 950, 2048 (1.2e5 tiles of 8 in its largest product) 5793 / 5359 /
+// 5184 / 5116.
+int tnx_f64_edge(const std::vector<GemmGroup>& groups, const std::vector<int>& which) {
+  int64_t n = 0;
+  for (int g : which) n += (int64_t)((groups[g].M + 7) / 8) * ((groups[g].N + 7) / 8);
+  return n > 65536 ? 16 : 8;
+}
+
+// Longest K first: the last tiles to start are the short ones.
+std::vector<GemmTile> tnx_gemm_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which, int edge) {
+  std::vector<int> order = which;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return groups[a].K > groups[b].K; });
+  std::vector<GemmTile> tiles;
+  for (int g : order)
+    for (int m0 = 0; m0 < groups[g].M; m0 += edge)
+      for (int n0 = 0; n0 < groups[g].N; n0 += edge) tiles.push_back(GemmTile{g, m0, n0, 0});
+  return tiles;
+}
+
+// Columns per skinny tile: 64, or fewer while that leaves SMs without a few tiles
+// (each tile stages its rows of A again).
+std::vector<GemmTile> tnx_skinny_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which) {
+  int width = 64;
+  auto count = [&](int w) {
+    int64_t n = 0;
+    for (int g : which) n += (int64_t)((groups[g].M + 127) / 128) * ((groups[g].N + w - 1) / w);
+    return n;
+  };
+  while (width > 8 && count(width) < 4 * 152) width /= 2;
+  std::vector<GemmTile> tiles;
+  for (int g : which)
+    for (int m0 = 0; m0 < groups[g].M; m0 += 128)
+      for (int n0 = 0; n0 < groups[g].N; n0 += width) tiles.push_back(GemmTile{g, m0, n0, width});
+  return tiles;
+}
+
 // Chunks of the relayout kernel (see k_copy.cu): large tasks cut into pieces of
 // TNX_COPY_CHUNK elements, consecutive small tasks packed together, transposing
 // tasks cut into 32 x 32 tiles, bands into their tiles.
@@ -1065,7 +1105,6 @@ void build_step(Plan& p, StepPlan& s) {
 
   // grouped GEMM
   std::vector<GemmGroup> gg(G);
-  std::vector<GemmTile> tiles, stiles;
   s.skinny.assign(G, 0);
   // Groups with K <= 16 run on the skinny FP64 kernel.  Under split precision
   // that holds only when every group of the step is that small: otherwise the
@@ -1090,21 +1129,19 @@ void build_step(Plan& p, StepPlan& s) {
     x.ldc = x.N;
     if (x.K <= 16 && (!split_prec || all_small)) {
       s.skinny[g] = 1;
-      for (int m0 = 0; m0 < x.M; m0 += 128)
-        for (int n0 = 0; n0 < x.N; n0 += 64) stiles.push_back(GemmTile{g, m0, n0, 0});
+      s.skinny_g.push_back(g);
     } else {
-      for (int m0 = 0; m0 < x.M; m0 += 64)
-        for (int n0 = 0; n0 < x.N; n0 += 64) tiles.push_back(GemmTile{g, m0, n0, 0});
+      s.dense_g.push_back(g);
     }
   }
+  if (p.prec == TNX_PREC_F64) s.edge = tnx_f64_edge(gg, s.dense_g);
+  const std::vector<GemmTile> tiles = tnx_gemm_tiles(gg, s.dense_g, s.edge), stiles = tnx_skinny_tiles(gg, s.skinny_g);
   s.dG = p.upload(gg);
   s.dT = p.upload(tiles);
   s.ntiles = (int)tiles.size();
   s.dTs = p.upload(stiles);
   s.nstiles_skinny = (int)stiles.size();
   s.hG = gg;
-  s.hT = tiles;
-  s.hTs = stiles;
 
   // useful flops: matched block pairs share (group, K offset)
   std::map<std::pair<int64_t, int64_t>, std::pair<double, double>> acc;
@@ -1672,7 +1709,7 @@ void enqueue_plan(Plan& p, cudaStream_t st, uint64_t fixed = 0, int skip_slot = 
     switch (p.prec) {
       case TNX_PREC_F64: {
         ProfScope ps(c, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
-        CUDA_CHECK(tnx_launch_gemm_f64(s.dG, s.dT, s.ntiles, p.d_slots, st));
+        CUDA_CHECK(tnx_launch_gemm_f64(s.dG, s.dT, s.ntiles, s.edge, p.d_slots, st));
         break;
       }
       case TNX_PREC_F32: {

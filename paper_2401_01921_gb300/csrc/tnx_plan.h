@@ -59,10 +59,11 @@ struct StepPlan {
   GemmGroup* dG = nullptr;
   GemmTile* dT = nullptr;
   int ntiles = 0;
+  int edge = 64;                // rows and columns of those tiles
   GemmTile* dTs = nullptr;      // skinny (K <= 16) tiles, FP64 in every precision
   int nstiles_skinny = 0;
   std::vector<GemmGroup> hG;    // host copies
-  std::vector<GemmTile> hT, hTs;
+  std::vector<int> dense_g, skinny_g;   // the groups of either kind
   std::vector<char> skinny;     // per group
   double flops_skinny = 0;      // useful flops of the skinny groups
   // split precision
@@ -198,6 +199,12 @@ std::vector<int4> tnx_kexp_items(const std::vector<KexpJob>& jobs);
 void tnx_enqueue_split(Plan& p, StepPlan& s, cudaStream_t st, bool needA, bool needB, bool balance);
 std::vector<int2> tnx_slice_schedule(std::vector<SliceJob>& jobs);
 std::vector<int2> tnx_tf32_schedule(std::vector<SliceJob>& jobs);
+
+// tiles of the FP64 / FP32 products and of the skinny (K <= 16) ones (tnx_network.cpp): over
+// the groups listed, a launch's tile edge or width chosen for all of them
+int tnx_f64_edge(const std::vector<GemmGroup>& groups, const std::vector<int>& which);
+std::vector<GemmTile> tnx_gemm_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which, int edge);
+std::vector<GemmTile> tnx_skinny_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which);
 
 // relayout chunks (tnx_network.cpp)
 void tnx_make_copy_chunks(const std::vector<CopyTask>& tasks, std::vector<int4>& chunks);
