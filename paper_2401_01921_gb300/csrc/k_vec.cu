@@ -137,11 +137,12 @@ constexpr int MD_BLOCKS_MAX = 608;
 
 // Blocks of the multidot kernel: about 416 vector entries per block (an
 // L2-resident basis is bound by FP64 issue, where fewer partial sums help),
-// rounded to a multiple of the SM count, at least 1 and at most 4 per SM (a
-// basis in HBM needs the loads of that many blocks in flight).
+// at least 1; above one per SM rounded to a multiple of the SM count, at most 4 per
+// SM (a basis in HBM needs the loads of that many blocks in flight).
 int multidot_blocks(int64_t n) {
-  int64_t b = (n / 416 + 151) / 152 * 152;
-  if (b < 152) b = 152;
+  int64_t b = n / 416;
+  if (b < 1) b = 1;
+  if (b > 152) b = (b + 151) / 152 * 152;
   if (b > MD_BLOCKS_MAX) b = MD_BLOCKS_MAX;
   return (int)b;
 }
@@ -199,6 +200,16 @@ __device__ void block_multidot(const LanczosDev& L, int m, int64_t c0, int64_t c
       case 15: multidot_group<15>(L, r0, c0, c1, sh); break;
       default: multidot_group<16>(L, r0, c0, c1, sh); break;
     }
+    if (ng == 1) {   // a single vector: warp sums (the row sums below would chain 16 additions)
+      const double v = warp_sum(sh[0][threadIdx.x]);
+      __syncthreads();
+      if ((threadIdx.x & 31) == 0) sh[0][threadIdx.x >> 5] = v;
+      __syncthreads();
+      if (threadIdx.x == 0)
+        L.partial[(int64_t)blockIdx.x * m + g0] = (sh[0][0] + sh[0][1]) + (sh[0][2] + sh[0][3]);
+      __syncthreads();
+      continue;
+    }
     __syncthreads();
     // thread t sums 16 consecutive entries of row t/8, then 8 partners combine
     const int row = threadIdx.x >> 3, part = threadIdx.x & 7;
@@ -221,7 +232,7 @@ __device__ void finalize_coefs(const LanczosDev& L, int m, int nb, int alpha_i, 
   for (int i = 0; i < m; ++i) {
     double acc = 0.0;
     for (int b = threadIdx.x; b < nb; b += blockDim.x) acc += __ldcg(L.partial + (int64_t)b * m + i);
-    acc = block_sum(acc, sh);
+    acc = nb > 32 ? block_sum(acc, sh) : warp_sum(acc);   // up to 32 partials lie in one warp
     if (threadIdx.x == 0) {
       L.coef[i] = acc;
       if (i == alpha_i) L.alpha[alpha_j] = acc;
@@ -334,69 +345,105 @@ __global__ void __launch_bounds__(RT) gs_update_kernel(LanczosDev L, int m, int 
 // test, the next input slot); with one, the gated launches after it do.
 constexpr int PRO_MAX = 514;   // rows of at most 500 steps + 2
 
+// What a step waits for here is FP64 latency: an FP64 instruction takes its SM
+// quarter 64 cycles however few lanes need it (a root ten of them, a division
+// nine), so roots and divisions are taken once, by one warp, maxima of
+// non-negative numbers are formed on their bit patterns, and eps1 comes from the
+// host.  Dense bond dimension 32 (4096 entries): the three-term launch 11.4 -> 9.0 us
+// (ncu, cold caches).
+__device__ __forceinline__ unsigned long long bits_abs(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// max(|alpha_i|, beta_i) and max(|alpha_i| + beta_i + beta_{i+1}) over i <= j (beta_{j+1}
+// left out), as bit patterns; one warp.
+__device__ __forceinline__ void tridiag_scale(const LanczosDev& L, int j, int lane, unsigned long long& amax,
+                                              unsigned long long& an) {
+  amax = an = 0;
+  for (int i = lane; i <= j; i += 32) {
+    const double a = fabs(L.alpha[i]), b = L.beta[i];
+    amax = max(amax, max(bits_abs(a), bits_abs(b)));
+    an = max(an, bits_abs(a + b + (i < j ? L.beta[i + 1] : 0.0)));
+  }
+  amax = warp_max(amax);
+  an = warp_max(an);
+}
+
+// Sum of the nb partials, in a fixed order; valid in thread 0.
+__device__ double partial_sum(const double* partial, int nb, double* sh) {
+  double acc = 0.0;
+  for (int b = threadIdx.x; b < nb; b += RT) acc += __ldcg(partial + b);
+  if (nb > 32) return block_sum(acc, sh);   // else the other warps hold zeros
+  return warp_sum(acc);
+}
+
 // Run by one block of RT threads over the nb norm partials.
-__device__ void pro_decide(const LanczosDev& L, int j, int nb, int last, double** next_slot, double tau) {
+__device__ void pro_decide(const LanczosDev& L, int j, int nb, int last, double** next_slot, double tau,
+                           double eps1) {
   __shared__ double sh[32];
   __shared__ double s_om[PRO_MAX];
-  __shared__ double s_b, s_amax, s_anorm, s_mx[RT / 32];
+  __shared__ double s_b, s_inv;
+  __shared__ unsigned long long s_amax, s_an, s_mx[4];
   __shared__ int s_pass;
-  double acc = 0.0;
-  for (int b = threadIdx.x; b < nb; b += RT) acc += __ldcg(L.partial + b);
-  if (threadIdx.x < 32) {
-    double amax = 0.0, an = 0.0;
-    for (int i = threadIdx.x; i <= j; i += 32) {
-      amax = fmax(amax, fmax(fabs(L.alpha[i]), L.beta[i]));
-      an = fmax(an, fabs(L.alpha[i]) + L.beta[i] + (i < j ? L.beta[i + 1] : 0.0));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-      an = fmax(an, __shfl_xor_sync(0xffffffffu, an, o));
-    }
-    if (threadIdx.x == 0) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (wid == 1) {
+    unsigned long long amax, an;
+    tridiag_scale(L, j, lane, amax, an);
+    if (lane == 0) {
       s_amax = amax;
-      s_anorm = an;
+      s_an = an;
     }
   }
-  acc = block_sum(acc, sh);
-  if (threadIdx.x == 0) s_b = sqrt(acc);
+  const double acc = partial_sum(L.partial, nb, sh);
+  if (threadIdx.x == 0) {
+    s_b = sqrt(acc);
+    s_inv = 1.0 / s_b;
+  }
   __syncthreads();
-  const double bn = s_b;
-  const double anorm = fmax(s_anorm, fabs(L.alpha[j]) + (j > 0 ? L.beta[j] : 0.0) + bn);
-  const double eps1 = sqrt((double)L.n) * 0.5 * 2.220446049250313e-16;
-  const double* om = L.omega;                  // row j: k = 0..j
-  const double* omp = L.omega + (L.nmax + 2);  // row j-1: k = 0..j-1
-  double mx = 0.0;
-  for (int k = threadIdx.x; k <= j; k += RT) {
-    double e;
-    if (k < j) {
-      double t = L.beta[k + 1] * om[k + 1] + (L.alpha[k] - L.alpha[j]) * om[k] - L.beta[j] * omp[k];
-      if (k > 0) t += L.beta[k] * om[k - 1];
-      e = (t + copysign(eps1 * anorm, t)) / bn;
-    } else {
-      e = eps1 * anorm / bn;
+  const double bn = s_b, inv = s_inv;
+  // one warp per SM quarter covers the j + 1 estimates
+  if (threadIdx.x < 128) {
+    const double* om = L.omega;                  // row j: k = 0..j
+    const double* omp = L.omega + (L.nmax + 2);  // row j-1: k = 0..j-1
+    const double aj = L.alpha[j], bj = j > 0 ? L.beta[j] : 0.0;
+    const double an = __longlong_as_double((long long)max(s_an, bits_abs(fabs(aj) + bj + bn)));
+    const double round = eps1 * an;
+    unsigned long long mx = 0;
+    for (int k = threadIdx.x; k <= j; k += 128) {
+      double e;
+      if (k < j) {
+        double t = L.beta[k + 1] * om[k + 1] + (L.alpha[k] - aj) * om[k] - bj * omp[k];
+        if (k > 0) t += L.beta[k] * om[k - 1];
+        e = (t + copysign(round, t)) * inv;
+      } else {
+        e = round * inv;
+      }
+      s_om[k] = e;
+      // beta_{j+1} = 0 or an overflowing estimate (its bit pattern lies above every
+      // finite one's) counts as lost orthogonality
+      mx = max(mx, bits_abs(e));
     }
-    s_om[k] = e;
-    // beta_{j+1} = 0 or an overflowing estimate counts as lost orthogonality
-    mx = (fabs(e) <= 1e300) ? fmax(mx, fabs(e)) : INFINITY;
+    mx = warp_max(mx);
+    if (lane == 0) s_mx[wid] = mx;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) s_mx[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int w = 0; w < RT / 32; ++w) m = fmax(m, s_mx[w]);
+    const unsigned long long m = max(max(s_mx[0], s_mx[1]), max(s_mx[2], s_mx[3]));
     const int forced = L.state[3];
-    const int pass = forced || !(m <= tau);
+    const int pass = forced || !(tau >= 0.0 && m <= bits_abs(tau));
     s_pass = pass;
     L.state[2] = pass;
     L.state[3] = pass && !forced;
     if (!pass) {
       L.beta[j + 1] = bn;
-      L.scratch[3 * L.nmax + 3] = 1.0 / bn;   // for the normalising kernel
+      L.scratch[3 * L.nmax + 3] = inv;   // for the normalising kernel
       L.state[0] = j + 1;
-      if (last || bn < 1e-14 * s_amax) L.state[1] = 1;
+      if (last || bn < 1e-14 * __longlong_as_double((long long)s_amax)) L.state[1] = 1;
       else *next_slot = L.V + (int64_t)(j + 1) * L.n;
     }
   }
@@ -414,7 +461,7 @@ __device__ void pro_decide(const LanczosDev& L, int j, int nb, int last, double*
 // The three-term step w <- (w - alpha_j v_j) - beta_j v_{j-1} (beta_0 = 0), with
 // partial[b] = this block's share of the new |w|^2 (fixed order).
 __global__ void __launch_bounds__(RT) three_term_norm_kernel(LanczosDev L, int j, int last, double** next_slot,
-                                                              double tau) {
+                                                              double tau, double eps1) {
   tnx_grid_dependency();
   __shared__ double sh[32];
   if (stopped(L.state)) return;
@@ -442,7 +489,7 @@ __global__ void __launch_bounds__(RT) three_term_norm_kernel(LanczosDev L, int j
   nrm = block_sum(nrm, sh);
   if (threadIdx.x == 0) L.partial[blockIdx.x] = nrm;
   if (last_block(L.state + 4)) {
-    pro_decide(L, j, gridDim.x, last, next_slot, tau);
+    pro_decide(L, j, gridDim.x, last, next_slot, tau, eps1);
     if (threadIdx.x == 0) L.state[4] = 0;
   }
 }
@@ -465,126 +512,169 @@ __device__ __forceinline__ double dfromkey(long long key) {
   return __longlong_as_double(key >= 0 ? key : (long long)(0x8000000000000000ull - (unsigned long long)key));
 }
 
-// Sturm count on the shared-memory copy of T: number of negative pivots of the
-// LDL^T factorisation of T - xI (b2[j] = beta_j^2, b2[0] unused).
-__device__ int sturm_count(const double* a, const double* b2, int k, double x) {
-  int cnt = 0;
-  double d = 1.0;
-  for (int j = 0; j < k; ++j) {
-    d = (a[j] - x) - (j > 0 ? b2[j] / d : 0.0);
-    if (d == 0.0) d = -1e-300;
-    if (d < 0) ++cnt;
-  }
-  return cnt;
+// Doubles between lo and hi >= lo (unsigned: keys of both signs lie up to 2^64 apart).
+__device__ __forceinline__ unsigned long long doubles_between(double lo, double hi) {
+  return (unsigned long long)dkey(hi) - (unsigned long long)dkey(lo);
 }
 
-// Lowest eigenvalue of T by Sturm-sequence multisection: each of the RT
-// threads counts the eigenvalues below its own point of the current bracket,
-// and the bracket shrinks to the one sub-interval where the count first
-// reaches 1 (the same test as bisection, RT points per round), until it stops
-// shrinking.  Then inverse iteration (Thomas algorithm, 3 sweeps) for the
-// eigenvector y on thread 0.  beta[j] couples rows j-1 and j (beta[0] unused).
-// T is copied to shared memory first: the sequential parts run on thread 0,
-// where every global-memory access would be a dependent trip to L2; the LU
-// factors of T - shift I are the same in every sweep and computed once.
-constexpr int TD_MAX = 512;   // Lanczos steps are limited to 500
+// Whether T - xI has an eigenvalue <= 0, i.e. whether its leading minors p_j are not
+// all positive: p_{j+1} = (a_j - x) p_j - b_j^2 p_{j-1} (b2[j] = beta_j^2, b2[0] = 0).
+// The pivots of the LDL^T factorisation are p_{j+1} / p_j, so this is Sturm's count
+// >= 1 without a division per row (three FP64 instructions instead of twelve).
+// The pair is rescaled by exponents when it leaves the middle of the range.
+__device__ bool eigenvalue_below(const double* a, const double* b2, int k, double x) {
+  double pm = 0.0, p = 1.0;
+  for (int j = 0; j < k; ++j) {
+    const double r = fma(a[j] - x, p, -(b2[j] * pm));
+    pm = p;
+    p = r;
+    const int hi = __double2hiint(p);
+    if (hi < 0 || (hi | __double2loint(p)) == 0) return true;   // negative, or zero (counted as negative)
+    const int ex = hi >> 20;
+    if (ex < 600 || (ex > 1450 && ex < 2047)) {
+      const int sh = (ex < 600 ? 500 : -500) << 20, hm = __double2hiint(pm);
+      p = __hiloint2double(hi + (ex > 0 ? sh : 0), __double2loint(p));
+      const int em = (hm >> 20) + (sh >> 20);
+      pm = hm >> 20 > 0 && em > 0 && em < 2047 ? __hiloint2double(hm + sh, __double2loint(pm)) : 0.0;
+    }
+  }
+  return false;
+}
 
-__global__ void __launch_bounds__(RT) tridiag_kernel(LanczosDev L) {
+// Lowest eigenvalue of T by multisection: each of the TT threads tests its own
+// point of the current bracket, and the bracket shrinks to the one sub-interval
+// where the test first holds (the same test as bisection, TT points per round),
+// until at most TT doubles are left, which the threads test one by one: the
+// result is the smallest double of the bracket for which the test holds, as
+// bisection to adjacent doubles finds it.  Then inverse iteration (Thomas
+// algorithm, 3 sweeps) for the eigenvector y, by one warp (its serial parts by all
+// lanes alike).  beta[j] couples rows j-1 and j (beta[0] unused).  T is copied to
+// shared memory first; the LU factors of T - shift I are the same in every sweep
+// and computed once.  Four warps, one per SM quarter: more would queue for the
+// quarters' FP64 units (an instruction takes one 64 cycles).  172 -> 54 us for
+// 20 steps (with 256 threads and a division per row and point before).
+constexpr int TD_MAX = 512;   // Lanczos steps are limited to 500
+constexpr int TT = 128;
+
+__global__ void __launch_bounds__(TT) tridiag_kernel(LanczosDev L) {
   tnx_grid_dependency();
   __shared__ double sa[TD_MAX], sb[TD_MAX], sb2[TD_MAX], sl[TD_MAX], sy[TD_MAX];
-  __shared__ double s_lo, s_hi;
-  __shared__ int s_first;
+  __shared__ double s_x[TT];
+  __shared__ long long s_key[2][TT / 32];
+  __shared__ int s_first[TT / 32];
   const int k = L.state[0];
-  for (int j = threadIdx.x; j < k; j += RT) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int j = threadIdx.x; j < k; j += TT) {
     sa[j] = L.alpha[j];
     sb[j] = L.beta[j];
     sb2[j] = j > 0 ? sb[j] * sb[j] : 0.0;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double lo = 0.0, hi = 0.0;
-    for (int j = 0; j < k; ++j) {
-      const double r = (j > 0 ? fabs(sb[j]) : 0.0) + (j + 1 < k ? fabs(sb[j + 1]) : 0.0);
-      if (j == 0 || sa[j] - r < lo) lo = sa[j] - r;
-      if (j == 0 || sa[j] + r > hi) hi = sa[j] + r;
-    }
-    s_lo = lo;
-    s_hi = hi;
+  // Gershgorin bracket, compared as ordered integers
+  long long klo = INT64_MAX, khi = INT64_MIN;
+  for (int j = threadIdx.x; j < k; j += TT) {
+    const double r = (j > 0 ? fabs(sb[j]) : 0.0) + (j + 1 < k ? fabs(sb[j + 1]) : 0.0);
+    klo = min(klo, dkey(sa[j] - r));
+    khi = max(khi, dkey(sa[j] + r));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    klo = min(klo, __shfl_xor_sync(0xffffffffu, klo, o));
+    khi = max(khi, __shfl_xor_sync(0xffffffffu, khi, o));
+  }
+  if (lane == 0) {
+    s_key[0][wid] = klo;
+    s_key[1][wid] = khi;
   }
   __syncthreads();
-  const double frac = (double)(threadIdx.x + 1) / (double)(RT + 1);
-  for (int round = 0; round < 64; ++round) {
-    const double lo = s_lo, hi = s_hi;
+  for (int w = 0; w < TT / 32; ++w) {
+    klo = min(klo, s_key[0][w]);
+    khi = max(khi, s_key[1][w]);
+  }
+  double lo = dfromkey(klo), hi = dfromkey(khi);
+  // index of the first thread whose test holds (TT: none); every thread gets it
+  auto first = [&](bool holds) {
+    const unsigned m = __ballot_sync(0xffffffffu, holds);
+    if (lane == 0) s_first[wid] = m ? __ffs(m) - 1 + 32 * wid : TT;
+    __syncthreads();
+    int f = TT;
+    for (int w = TT / 32 - 1; w >= 0; --w)
+      if (s_first[w] < TT) f = s_first[w];
+    __syncthreads();
+    return f;
+  };
+  const double frac = (double)(threadIdx.x + 1) / (double)(TT + 1);
+  for (int round = 0; round < 96 && doubles_between(lo, hi) > TT; ++round) {
     const double x = lo + (hi - lo) * frac;
-    if (threadIdx.x == 0) s_first = RT;
-    __syncthreads();
-    if (x > lo && x < hi && sturm_count(sa, sb2, k, x) >= 1) atomicMin(&s_first, (int)threadIdx.x);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const int f = s_first;
-      const double nlo = f == 0 ? lo : lo + (hi - lo) * ((double)f / (double)(RT + 1));
-      const double nhi = f == RT ? hi : lo + (hi - lo) * ((double)(f + 1) / (double)(RT + 1));
-      s_lo = nlo > lo ? nlo : lo;
-      s_hi = nhi < hi ? nhi : hi;
-    }
-    __syncthreads();
-    if (!(s_lo < s_hi) || (s_lo == lo && s_hi == hi)) break;
+    s_x[threadIdx.x] = x;
+    const int f = first(dkey(x) > dkey(lo) && dkey(x) < dkey(hi) && eigenvalue_below(sa, sb2, k, x));
+    const double nlo = f == 0 ? lo : s_x[f - 1], nhi = f == TT ? hi : s_x[f];
+    __syncthreads();   // s_x is rewritten in the next round
+    const bool same = nlo <= lo && nhi >= hi;
+    if (nlo > lo) lo = nlo;
+    if (nhi < hi) hi = nhi;
+    if (same) break;
   }
-  // Finish on the (tiny) bracket: the oracle bisects until lo and hi are
-  // adjacent doubles, which leaves hi = the smallest double of (lo, hi] whose
-  // count reaches 1.  Here the RT threads test the doubles lo+1, lo+2, ... ulps
-  // at once (a key that orders doubles like integers), after serial halving
-  // while more than RT of them remain.
-  __shared__ int s_t;
-  double lo = s_lo, hi = s_hi;
-  if (threadIdx.x == 0) {
-    for (int it = 0; it < 200 && dkey(hi) - dkey(lo) > RT; ++it) {
-      const double mid = 0.5 * (lo + hi);
-      if (mid <= lo || mid >= hi) break;
-      if (sturm_count(sa, sb2, k, mid) >= 1) hi = mid; else lo = mid;
-    }
-    s_lo = lo;
-    s_hi = hi;
-    s_t = RT;
+  for (int it = 0; it < 200 && doubles_between(lo, hi) > TT; ++it) {   // what rounding left: plain halving
+    const double mid = 0.5 * (lo + hi);
+    if (mid <= lo || mid >= hi) break;
+    if (eigenvalue_below(sa, sb2, k, mid)) hi = mid; else lo = mid;
   }
-  __syncthreads();
-  lo = s_lo;
-  hi = s_hi;
-  const long long span = dkey(hi) - dkey(lo);   // hi itself counts
-  if ((long long)threadIdx.x + 1 < span) {
-    const double x = dfromkey(dkey(lo) + threadIdx.x + 1);
-    if (sturm_count(sa, sb2, k, x) >= 1) atomicMin(&s_t, (int)threadIdx.x);
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  const double lam = s_t < RT ? dfromkey(dkey(lo) + s_t + 1) : hi;
-  *L.eval = lam;
-  // LU of T - shift I (no pivoting): sa becomes the pivots, sl the multipliers;
-  // the sweeps multiply by the pivots' reciprocals, formed once
+  const unsigned long long span = doubles_between(lo, hi);   // hi itself counts
+  const int t = first((unsigned long long)threadIdx.x + 1 < span &&
+                      eigenvalue_below(sa, sb2, k, dfromkey(dkey(lo) + threadIdx.x + 1)));
+  if (wid != 0) return;
+  const double lam = t < TT ? dfromkey(dkey(lo) + t + 1) : hi;
+  if (lane == 0) *L.eval = lam;
+  // LU of T - shift I (no pivoting): sl the multipliers, sb2 the pivots' reciprocals
   const double shift = lam - 1e-13 * fmax(1.0, fabs(lam));
-  for (int j = 0; j < k; ++j) sa[j] -= shift;
-  for (int j = 1; j < k; ++j) {
-    const double piv = sa[j - 1] != 0.0 ? sa[j - 1] : 1e-300;
-    sl[j] = sb[j] / piv;
-    sa[j] -= sl[j] * sb[j];
+  double inv = 0.0;
+  for (int j = 0; j < k; ++j) {
+    double piv = sa[j] - shift;
+    if (j > 0) {
+      const double l = sb[j] * inv;
+      sl[j] = l;
+      piv = fma(-l, sb[j], piv);
+    }
+    inv = 1.0 / (piv != 0.0 ? piv : 1e-300);
+    sb2[j] = inv;
   }
-  for (int j = 0; j < k; ++j) sb2[j] = 1.0 / (sa[j] != 0.0 ? sa[j] : 1e-300);   // sb2 is free now
   const double inv0 = 1.0 / sqrt((double)k);
-  for (int j = 0; j < k; ++j) sy[j] = inv0;
+  for (int j = lane; j < k; j += 32) sy[j] = inv0;
+  __syncwarp();
   for (int sweep = 0; sweep < 3; ++sweep) {
-    for (int j = 1; j < k; ++j) sy[j] -= sl[j] * sy[j - 1];
-    sy[k - 1] = sy[k - 1] * sb2[k - 1];
-    for (int j = k - 2; j >= 0; --j) sy[j] = (sy[j] - sb[j + 1] * sy[j + 1]) * sb2[j];
+    double y = sy[0];
+    for (int j = 1; j < k; ++j) {
+      y = fma(-sl[j], y, sy[j]);
+      __syncwarp();
+      sy[j] = y;
+    }
+    y = y * sb2[k - 1];
+    __syncwarp();
+    sy[k - 1] = y;
+    for (int j = k - 2; j >= 0; --j) {
+      y = fma(-sb[j + 1], y, sy[j]) * sb2[j];
+      __syncwarp();
+      sy[j] = y;
+    }
+    __syncwarp();
     double nrm = 0.0;
-    for (int j = 0; j < k; ++j) nrm += sy[j] * sy[j];
-    const double inv = 1.0 / sqrt(nrm);
-    for (int j = 0; j < k; ++j) sy[j] *= inv;
+    for (int j = lane; j < k; j += 32) nrm = fma(sy[j], sy[j], nrm);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+    const double f = 1.0 / sqrt(nrm);
+    for (int j = lane; j < k; j += 32) sy[j] *= f;
+    __syncwarp();
   }
   int jm = 0;
-  for (int j = 1; j < k; ++j)
-    if (fabs(sy[j]) > fabs(sy[jm])) jm = j;
+  unsigned long long best = 0;
+  for (int j = 0; j < k; ++j)
+    if (bits_abs(sy[j]) > best) {
+      best = bits_abs(sy[j]);
+      jm = j;
+    }
   const double sgn = sy[jm] < 0 ? -1.0 : 1.0;
-  for (int j = 0; j < k; ++j) L.y[j] = sgn * sy[j];
+  for (int j = lane; j < k; j += 32) L.y[j] = sgn * sy[j];
 }
 
 __global__ void __launch_bounds__(RT) ritz_kernel(LanczosDev L, double* out) {
@@ -696,7 +786,8 @@ cudaError_t tnx_launch_lanczos_step(const LanczosDev& L, int j, double** next_sl
     if (le != cudaSuccess) return le;
   }
   {
-    const cudaError_t le = tnx_launch(three_term_norm_kernel, dim3(nb), dim3(RT), 0, st, L, j, last, next_slot, tau);
+    const cudaError_t le = tnx_launch(three_term_norm_kernel, dim3(nb), dim3(RT), 0, st, L, j, last, next_slot, tau,
+                                      sqrt((double)L.n) * 0.5 * 2.220446049250313e-16);
     if (le != cudaSuccess) return le;
   }
   {
@@ -720,7 +811,7 @@ cudaError_t tnx_launch_lanczos_step(const LanczosDev& L, int j, double** next_sl
 
 cudaError_t tnx_launch_lanczos_finish(const LanczosDev& L, double* evec, cudaStream_t st) {
   {
-    const cudaError_t le = tnx_launch(tridiag_kernel, dim3(1), dim3(RT), 0, st, L);
+    const cudaError_t le = tnx_launch(tridiag_kernel, dim3(1), dim3(TT), 0, st, L);
     if (le != cudaSuccess) return le;
   }
   tnx_note_launch(1);
