@@ -4,22 +4,28 @@
 // two-site H_eff, Sec. 11) is a small FP64 product between two relayouts: its
 // operand A is gathered from the previous step's output blocks into the packed
 // K-major matrix, and its output C is immediately relaid into the next step's
-// packed operand.  Here one CTA takes a tile of up to 128 rows (p, q) of one row
-// block of A_g:
+// packed operand.  Here one CTA takes a run of tiles of up to 128 rows (p, q) of one
+// row block of A_g.  It lists the nonzeros of every column of the packed B_g (the
+// MPO product is mostly zeros) and stages the columns' descriptors once, then per tile:
 //   1. every A element of the tile is read from its source block through the
 //      descriptor of its column (consecutive threads take consecutive q, the
-//      source blocks' contiguous leg), into the A rows in shared memory;
-//   2. the CTA lists the nonzeros of every column of the packed B_g (the MPO
-//      product is mostly zeros) and two threads form each output row (even and
-//      odd columns), with the same FMA chains as the unfused skinny kernel
-//      (bit-identical; a power-of-two first coefficient is applied on the
-//      integer units, tnx_first_term);
+//      source blocks' contiguous leg) one tile ahead, and put into the A rows in
+//      shared memory;
+//   2. two threads form each output row (even and odd columns), with the same FMA
+//      chains as the unfused skinny kernel (bit-identical; a power-of-two first
+//      coefficient is applied on the integer units, tnx_first_term);
 //   3. every output element is stored through the descriptor of its column
 //      straight into the next step's packed operand (consecutive threads take
 //      consecutive p, that operand's contiguous leg), or the rows are written to
 //      C_g when no next step reads them through descriptors.
 // The packed A and the C rows never reach HBM when both ends are fused.  The
 // descriptors are precomputed by the planner from the two relayouts' bands.
+//
+// Instruction issue bounds it: a charge group has only a few columns, so with one
+// tile per CTA a thread formed 2.4 outputs on average and the warp issued 430
+// instructions for them, mostly the lists, descriptors and index setup, which a
+// run of tiles (tnx_fused_runs, tnx_network.cpp) shares: one apply of the Heisenberg
+// H_eff (ncu, cold) at bond dimension 2048 75 -> 62 us, 4096 244 -> 188 us.
 #include "tnx_internal.h"
 
 namespace {
@@ -41,7 +47,14 @@ struct FusedSmem {
   uint32_t s_p2[FMAXN];           // tnx_pow2_code of each column's first nonzero
 };
 
-__global__ void __launch_bounds__(FT, 6) fused_skinny_kernel(const GemmGroup* __restrict__ groups,
+// t / d for 0 <= t < FR and 1 <= d <= FR through m = ceil(2^16 / d): the estimate
+// exceeds t / d by less than t / 2^16 < 1 / d.
+__device__ __forceinline__ int small_magic(int d) { return (65536 + d - 1) / d; }
+__device__ __forceinline__ int small_div(int t, int m) { return (t * m) >> 16; }
+
+// RUN false: every run of the launch is one tile (nothing is read ahead).
+template <bool RUN>
+__global__ void __launch_bounds__(FT, RUN ? 5 : 6) fused_skinny_kernel(const GemmGroup* __restrict__ groups,
                                                           const FusedTile* __restrict__ tiles,
                                                           const FusedCol* __restrict__ cols, int kp, int np,
                                                           double* const* __restrict__ slots) {
@@ -50,10 +63,12 @@ __global__ void __launch_bounds__(FT, 6) fused_skinny_kernel(const GemmGroup* __
   FusedSmem& S = *(FusedSmem*)dyn;
   double* sA = (double*)(dyn + sizeof(FusedSmem));   // [rows][kp]
   double* sC = sA + FR * kp;                         // [rows][np]
+  FusedCol* s_gc = (FusedCol*)(sC + FR * np);        // RUN: [W] A column descriptors
   const FusedTile T = tiles[blockIdx.x];
   const int tid = threadIdx.x, half = tid / FR, t = tid & (FR - 1);
-  const int rows = T.tP * T.tQ, W = T.W, N = T.N;
-  // output column descriptors (threads [FR + FMAXN, FR + FMAXN + N)), off the gather's path
+  const int W = T.W, N = T.N;
+  // column descriptors: A's by threads [0, W), the output's by [FR + FMAXN, FR + FMAXN + N)
+  if (RUN && tid < W) s_gc[tid] = cols[T.gcol + tid];
   if (tid >= FR + FMAXN && tid - FR - FMAXN < N && T.scol >= 0) S.s_sc[tid - FR - FMAXN] = cols[T.scol + tid - FR - FMAXN];
   // B nonzeros (threads [FR, FR + N))
   const GemmGroup g = groups[T.group];
@@ -75,61 +90,87 @@ __global__ void __launch_bounds__(FT, 6) fused_skinny_kernel(const GemmGroup* __
     S.s_cnt[t] = c;
     S.s_p2[t] = c ? tnx_pow2_code(S.s_v[t][0]) : 0u;
   }
-  // gather: row r = t, q fastest; this thread takes columns half, half + 2, ...
-  if (t < rows) {
-    const int p = t / T.tQ, q = t - p * T.tQ;
-    const int64_t P = T.p0 + p, Q = T.q0 + q;
-    double v[FMAXK / 2];
+  // the current tile: rows p in [p0, p0 + tp), q in [q0, q0 + tq)
+  const int nQ = RUN ? (T.EQ + T.tQ - 1) / T.tQ : 1;
+  const int mQ = RUN ? small_magic(T.tQ) : 0, mP = RUN ? small_magic(T.tP) : 0;
+  int p0 = T.p0, q0 = T.q0, tp = T.eP, tq = T.eQ;
+  auto over_q = [&](int r) { return !RUN ? r / tq : small_div(r, tq == T.tQ ? mQ : small_magic(tq)); };
+  double v[FMAXK / 2];
+  // this thread's entries of the tile's A: row t, q fastest; columns half, half + 2, ...
+  auto fetch = [&](const FusedCol* gc) {
+    if (t < tp * tq) {
+      const int p = over_q(t), q = t - p * tq;
+      const int P = p0 + p, Q = q0 + q;
 #pragma unroll
-    for (int j = 0; j < FMAXK / 2; ++j) {
-      const int c = half + 2 * j;
-      v[j] = 0.0;
-      if (c < W) {
-        const FusedCol d = cols[T.gcol + c];
-        if (d.ptr) v[j] = __ldg(d.ptr + P * d.sP + Q * d.sQ);
+      for (int j = 0; j < FMAXK / 2; ++j) {
+        const int c = half + 2 * j;
+        v[j] = 0.0;
+        if (c < W) {
+          const FusedCol d = gc[c];
+          if (d.ptr) v[j] = __ldg(d.ptr + (int64_t)P * d.sP + (int64_t)Q * d.sQ);
+        }
       }
     }
-#pragma unroll
-    for (int j = 0; j < FMAXK / 2; ++j) {
-      const int c = half + 2 * j;
-      if (c < W) sA[t * kp + c] = v[j];
-    }
-  }
-  __syncthreads();
-  if (t < rows) {
-    const double* arow = sA + t * kp;
-    double* crow = sC + t * np;
-    for (int n = half; n < N; n += 2) {
-      double acc = 0.0;
-      const int c = S.s_cnt[n];
-      if (c > 0) acc = tnx_first_term(arow[S.s_k[n][0]], S.s_v[n][0], S.s_p2[n]);
-      for (int e = 1; e < c; ++e) acc = fma(arow[S.s_k[n][e]], S.s_v[n][e], acc);
-      crow[n] = acc;
-    }
-  }
-  __syncthreads();
-  if (T.scol >= 0) {
-    // scatter: p fastest (row r = p * tQ + q in shared memory)
+  };
+  fetch(cols + T.gcol);   // beside the lists' and descriptors' own loads
+  int pt = RUN ? T.t0 / nQ : 0, qt = RUN ? T.t0 - pt * nQ : 0;
+  for (int i = 0; i < (RUN ? T.nt : 1); ++i) {
+    const int rows = tp * tq;
     if (t < rows) {
-      const int q = t / T.tP, p = t - q * T.tP;
-      const int64_t P = T.p0 + p, Q = T.q0 + q;
-      const double* crow = sC + (p * T.tQ + q) * np;
-      for (int c = half; c < N; c += 2) {
-        const FusedCol d = S.s_sc[c];
-        if (d.ptr) d.ptr[P * d.sP + Q * d.sQ] = crow[c];
+#pragma unroll
+      for (int j = 0; j < FMAXK / 2; ++j) {
+        const int c = half + 2 * j;
+        if (c < W) sA[t * kp + c] = v[j];
       }
     }
-  } else {
-    // rows (p, q) of the block are rows row0 + (p0 + p) * EQ + q0 + q of C_g,
-    // EQ = the band's extent of q (the tiles of a band share T.row0 and EQ)
-    double* C = slots[g.c_slot] + g.c_off;
-    const int EQ = -T.scol - 1;
-    for (int e = tid; e < rows * N; e += FT) {
-      const int r = e / N, n = e - r * N;
-      const int p = r / T.tQ, q = r - p * T.tQ;
-      const int64_t row = (int64_t)T.row0 + (int64_t)(T.p0 + p) * EQ + T.q0 + q;
-      C[row * g.ldc + n] = sC[r * np + n];
+    __syncthreads();
+    const int cp0 = p0, cq0 = q0, ctp = tp, ctq = tq;   // this tile, when p0 .. move on to the next
+    if (RUN && i + 1 < T.nt) {
+      if (++qt == nQ) {
+        qt = 0;
+        ++pt;
+      }
+      p0 = pt * T.tP;
+      q0 = qt * T.tQ;
+      tp = min(T.tP, T.EP - p0);
+      tq = min(T.tQ, T.EQ - q0);
+      fetch(s_gc);
     }
+    if (t < rows) {
+      const double* arow = sA + t * kp;
+      double* crow = sC + t * np;
+      for (int n = half; n < N; n += 2) {
+        double acc = 0.0;
+        const int c = S.s_cnt[n];
+        if (c > 0) acc = tnx_first_term(arow[S.s_k[n][0]], S.s_v[n][0], S.s_p2[n]);
+        for (int e = 1; e < c; ++e) acc = fma(arow[S.s_k[n][e]], S.s_v[n][e], acc);
+        crow[n] = acc;
+      }
+    }
+    __syncthreads();
+    if (T.scol >= 0) {
+      // scatter: p fastest (row r = p * tq + q in shared memory)
+      if (t < rows) {
+        const int q = !RUN ? t / ctp : small_div(t, ctp == T.tP ? mP : small_magic(ctp)), p = t - q * ctp;
+        const int P = cp0 + p, Q = cq0 + q;
+        const double* crow = sC + (p * ctq + q) * np;
+        for (int c = half; c < N; c += 2) {
+          const FusedCol d = S.s_sc[c];
+          if (d.ptr) d.ptr[(int64_t)P * d.sP + (int64_t)Q * d.sQ] = crow[c];
+        }
+      }
+    } else {
+      // row (p, q) of the block is row row0 + p * EQ + q of C_g
+      double* C = slots[g.c_slot] + g.c_off;
+      for (int e = tid; e < rows * N; e += FT) {
+        const int r = e / N, n = e - r * N;
+        const int p = !RUN ? r / ctq : small_div(r, ctq == T.tQ ? mQ : small_magic(ctq)), q = r - p * ctq;
+        const int64_t row = (int64_t)T.row0 + (int64_t)(cp0 + p) * T.EQ + cq0 + q;
+        C[row * g.ldc + n] = sC[r * np + n];
+      }
+    }
+    // the next tile's A rows are written behind this tile's products (the barrier
+    // above), its C rows behind these reads of them (the next iteration's barriers)
   }
 }
 
@@ -137,26 +178,32 @@ __global__ void __launch_bounds__(FT, 6) fused_skinny_kernel(const GemmGroup* __
 
 size_t tnx_fused_smem_bytes(int kp, int np) { return sizeof(FusedSmem) + (size_t)FR * (kp + np) * sizeof(double); }
 
-cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, const FusedCol* cols,
-                                    int kp, int np, double* const* slots, cudaStream_t st) {
-  if (ntiles <= 0) return cudaSuccess;
-  if (kp < 1 || kp > FMAXK + 1 || np < 1 || np > FMAXN + 1) return cudaErrorInvalidValue;
-  const size_t smem = tnx_fused_smem_bytes(kp, np);
+namespace {
+template <bool RUN>
+cudaError_t launch_fused(const GemmGroup* groups, const FusedTile* tiles, int ntiles, const FusedCol* cols, int kp,
+                         int np, double* const* slots, cudaStream_t st) {
   static int attr_dev = -1;   // the opt-in is per device
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (attr_dev != dev) {
-    e = cudaFuncSetAttribute(fused_skinny_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tnx_fused_smem_bytes(FMAXK + 1, FMAXN + 1));
+    e = cudaFuncSetAttribute(fused_skinny_kernel<RUN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(tnx_fused_smem_bytes(FMAXK + 1, FMAXN + 1) + FMAXK * sizeof(FusedCol)));
     if (e != cudaSuccess) return e;
     attr_dev = dev;
   }
-  {
-    const cudaError_t le =
-        tnx_launch(fused_skinny_kernel, dim3(ntiles), dim3(FT), smem, st, groups, tiles, cols, kp, np, slots);
-    if (le != cudaSuccess) return le;
-  }
+  const size_t smem = tnx_fused_smem_bytes(kp, np) + (RUN ? FMAXK * sizeof(FusedCol) : 0);
+  return tnx_launch(fused_skinny_kernel<RUN>, dim3(ntiles), dim3(FT), smem, st, groups, tiles, cols, kp, np, slots);
+}
+}  // namespace
+
+cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, int run,
+                                    const FusedCol* cols, int kp, int np, double* const* slots, cudaStream_t st) {
+  if (ntiles <= 0) return cudaSuccess;
+  if (kp < 1 || kp > FMAXK + 1 || np < 1 || np > FMAXN + 1) return cudaErrorInvalidValue;
+  const cudaError_t le = run > 1 ? launch_fused<true>(groups, tiles, ntiles, cols, kp, np, slots, st)
+                                 : launch_fused<false>(groups, tiles, ntiles, cols, kp, np, slots, st);
+  if (le != cudaSuccess) return le;
   tnx_note_launch(1);
   return cudaGetLastError();
 }

@@ -227,15 +227,15 @@ cudaError_t tnx_launch_copy(const CopyTask* tasks, const int4* chunks, int nchun
 cudaError_t tnx_launch_copy_scaled(const CopyTask* tasks, const int4* chunks, int nchunks, double* const* slots,
                                    const double* src, double* vdst, int64_t vn, int full, const double* inv,
                                    const int32_t* state, cudaStream_t st);
-// Fused skinny step (k_fused.cu): one CTA per tile of up to 128 rows (p, q),
-// p in [p0, p0 + tP), q in [q0, q0 + tQ), of one row block of A_g (the rows a
-// destination band of the step's relayout fills).  Column c < W (= ldK of the
-// group) of those rows is described by FusedCol gcol + c: the A element of row
-// (p, q) lies at ptr + p * sP + q * sQ (ptr null: a structural zero).  The rows
-// are multiplied by the packed B_g (K <= 16, N <= 64) in FP64, and output
-// column c < N of row (p, q) is stored through FusedCol scol + c the same way
-// (ptr null: no step reads it).  scol < 0 writes the output rows to C_g
-// instead: row (p, q) to row row0 + p * EQ + q of the group, EQ = -scol - 1.
+// Fused skinny step (k_fused.cu): one CTA per run of tiles of one row block of A_g
+// (the rows a destination band of the step's relayout fills): EP x EQ rows (p, q),
+// cut into tiles of tP x tQ <= TNX_FUSED_ROWS rows, numbered along q first; a run
+// is the nt tiles from t0 on.  Column c < W (= ldK of the group) of those rows is
+// described by FusedCol gcol + c: the A element of row (p, q) lies at ptr + p * sP + q *
+// sQ (ptr null: a structural zero).  The rows are multiplied by the packed B_g (K <=
+// 16, N <= 64) in FP64, and output column c < N of row (p, q) is stored through
+// FusedCol scol + c the same way (ptr null: no step reads it).  scol < 0 writes the
+// output rows to C_g instead: row (p, q) to row row0 + p * EQ + q of the group.
 // The pointers are plan buffers (fused steps read and write no rebindable
 // slot).  kp, np: shared-memory pitches of the A and output rows (odd, > every
 // W and N).
@@ -245,12 +245,14 @@ struct FusedCol {
 };
 struct FusedTile {
   int32_t group, gcol, scol, row0;
-  int32_t p0, q0, tP, tQ;
-  int32_t W, N, pad0, pad1;
+  int32_t EP, EQ, tP, tQ;
+  int32_t W, N, t0, nt;
+  int32_t p0, q0, eP, eQ;   // the run's first tile: first row and extents
 };
 #define TNX_FUSED_ROWS 128   // rows (p, q) of a fused MPO-step tile at most (two threads per row)
-cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, const FusedCol* cols,
-                                    int kp, int np, double* const* slots, cudaStream_t st);
+// run: the largest nt of the launch
+cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, int run,
+                                    const FusedCol* cols, int kp, int np, double* const* slots, cudaStream_t st);
 size_t tnx_fused_smem_bytes(int kp, int np);
 // edge: rows and columns of a tile (8 or 16; FP32: 64)
 cudaError_t tnx_launch_gemm_f64(const GemmGroup* groups, const GemmTile* tiles, int ntiles, int edge,

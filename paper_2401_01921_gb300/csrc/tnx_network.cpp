@@ -741,6 +741,35 @@ std::vector<GemmTile> tnx_gemm_tiles(const std::vector<GemmGroup>& groups, const
   return tiles;
 }
 
+// Consecutive tiles of a band share a CTA, and its setup, while every SM keeps a few
+// CTAs: runs of at most 8 tiles, of one below six waves of the six CTAs an SM then
+// holds.  Tiles that leave a quarter of their rows empty stay alone (48 Hubbard
+// instances, 40 rows per tile: 178 us alone, 203 in runs, whose kernel holds five CTAs
+// per SM; Heisenberg at bond dimension 2048, 118 rows: 75 alone, 62 in runs of 5).
+std::vector<FusedTile> tnx_fused_runs(const std::vector<FusedTile>& bands, int& run) {
+  int64_t total = 0, rows = 0;
+  for (const FusedTile& b : bands) {
+    total += b.nt;
+    rows += (int64_t)b.EP * b.EQ;
+  }
+  run = rows < 96 * total ? 1 : (int)std::min<int64_t>(8, std::max<int64_t>(1, total / (152 * 6 * 3)));
+  std::vector<FusedTile> out;
+  for (FusedTile t : bands) {
+    const int nt = t.nt;
+    for (int t0 = 0; t0 < nt; t0 += run) {
+      t.t0 = t0;
+      t.nt = std::min(run, nt - t0);
+      const int nQ = (t.EQ + t.tQ - 1) / t.tQ;
+      t.p0 = t0 / nQ * t.tP;
+      t.q0 = t0 % nQ * t.tQ;
+      t.eP = std::min(t.tP, t.EP - t.p0);
+      t.eQ = std::min(t.tQ, t.EQ - t.q0);
+      out.push_back(t);
+    }
+  }
+  return out;
+}
+
 // Columns per skinny tile: 64, or fewer while that leaves SMs without a few tiles
 // (each tile stages its rows of A again).
 std::vector<GemmTile> tnx_skinny_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which) {
@@ -1448,30 +1477,31 @@ bool fuse_skinny_step(Plan& p, size_t si, int ti, bool tA) {
       const int64_t n = (E + Tmax - 1) / Tmax;
       return (E + n - 1) / n;
     };
-    std::vector<FusedTile> tiles;
+    int64_t total = 0, rows = 0;
+    std::vector<FusedTile> tiles;   // one entry per band, all its tiles
     for (size_t b = 0; b < bands.size(); ++b) {
       const Band& B = bands[b];
       const int64_t N = s.mkn[3 * B.g + 2];
       const size_t gcol = add_cols(ta, B.h, s.ldK[B.g], true);
-      int64_t scol = -(int64_t)B.EQ - 1;   // write the rows to C
+      int64_t scol = -1;   // write the rows to C
       if (ti >= 0) scol = (int64_t)add_cols(*tl, sidx[b] < 0 ? (size_t)-1 : (size_t)sidx[b], N, false);
       const int tQ = (int)balance(B.EQ, 16), tP = (int)balance(B.EP, TNX_FUSED_ROWS / tQ);
-      for (int p0 = 0; p0 < B.EP; p0 += tP)
-        for (int q0 = 0; q0 < B.EQ; q0 += tQ)
-          tiles.push_back(FusedTile{B.g, (int32_t)gcol, (int32_t)scol, (int32_t)B.row, p0, q0,
-                                    std::min(tP, B.EP - p0), std::min(tQ, B.EQ - q0), (int32_t)s.ldK[B.g],
-                                    (int32_t)N, 0, 0});
+      const int64_t nt = (int64_t)((B.EP + tP - 1) / tP) * ((B.EQ + tQ - 1) / tQ);
+      if (nt > INT32_MAX) return false;
+      tiles.push_back(FusedTile{B.g, (int32_t)gcol, (int32_t)scol, (int32_t)B.row, B.EP, B.EQ, tP, tQ,
+                                (int32_t)s.ldK[B.g], (int32_t)N, 0, (int32_t)nt, 0, 0, 0, 0});
+      total += nt;
+      rows += (int64_t)B.EP * B.EQ;
     }
     // many nearly empty tiles (small sectors) run faster unfused: plain
     // relayouts pack small blocks, the skinny kernel fills 128-row tiles
-    int64_t rows = 0;
-    for (const Band& B : bands) rows += (int64_t)B.EP * B.EQ;
-    if (!ok || tiles.size() > INT32_MAX || cols.size() > INT32_MAX || rows < 32 * (int64_t)tiles.size()) return false;
+    if (!ok || total > INT32_MAX || cols.size() > INT32_MAX || rows < 32 * total) return false;
     s.hFT = tiles;
+    const std::vector<FusedTile> runs = tnx_fused_runs(tiles, s.frun);
+    s.dFT = p.upload(runs);
+    s.nftiles = (int)runs.size();
     s.hFC = cols;
-    s.dFT = p.upload(tiles);
     s.dFC = p.upload(cols);
-    s.nftiles = (int)tiles.size();
     s.fkp = (int)(maxld | 1);
     s.fnp = (int)(maxN | 1);
     if (ti >= 0) {
@@ -1701,7 +1731,7 @@ void enqueue_plan(Plan& p, cudaStream_t st, uint64_t fixed = 0, int skip_slot = 
     }
     if (s.nftiles) {
       ProfScope ps(c, st, TNX_KC_SKINNY, s.flops_skinny);
-      CUDA_CHECK(tnx_launch_fused_skinny(s.dG, s.dFT, s.nftiles, s.dFC, s.fkp, s.fnp, p.d_slots, st));
+      CUDA_CHECK(tnx_launch_fused_skinny(s.dG, s.dFT, s.nftiles, s.frun, s.dFC, s.fkp, s.fnp, p.d_slots, st));
     } else if (s.nstiles_skinny) {
       ProfScope ps(c, st, TNX_KC_SKINNY, s.flops_skinny);
       CUDA_CHECK(tnx_launch_gemm_skinny(s.dG, s.dTs, s.nstiles_skinny, p.d_slots, st));
