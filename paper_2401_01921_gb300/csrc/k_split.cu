@@ -210,22 +210,71 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 // base-128 digit non-negative (digit i of the sum is digit i of v plus 64)
 constexpr long long DIGIT_BIAS = 64LL * ((1LL << 42) - 1) / 127;
 
+// The six digits of one entry, plus 64 each, as bytes: x[0] holds those of slices 5,
+// 4, 3 (bytes 0, 1, 2), x[1] those of slices 2, 1, 0; byte 3 is the high byte of
+// 128.0 in BF16 (1024.0 in FP16), so that a digit byte below it is the 16-bit float
+// 128 + e (1024 + e), e <= 128.
+struct DigitBytes {
+  uint32_t x[2];
+};
+template <bool F16>
+__device__ __forceinline__ DigitBytes digit_bytes(unsigned long long bits, int shift) {
+  // |x| 2^(F-E-2) rounded half up is (t + 1) / 2 (whole part) with t = m53 >> (shift + 11),
+  // shift = E_row - E >= 0, and with v that value signed, v + DIGIT_BIAS is the whole
+  // part of half of (t or, for x < 0, its complement) + 1 + 2 DIGIT_BIAS.
+  const uint32_t hi = (uint32_t)(bits >> 32);
+  const int s = (hi & 0x7FF00000u) == 0 ? 63 : min(shift + 11, 63);   // zeros and subnormals: t = 0
+  const unsigned long long m53 = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+  const unsigned long long sign = (unsigned long long)((long long)bits >> 63);
+  const unsigned long long u2 = ((m53 >> s) ^ sign) + (unsigned long long)(2 * DIGIT_BIAS + 1);
+  const uint32_t lo = (uint32_t)u2, up = (uint32_t)(u2 >> 22);
+  const uint32_t top = F16 ? 0x64000000u : 0x43000000u;
+  DigitBytes d;
+  d.x[0] = ((lo >> 1) & 0x7Fu) | top;
+  d.x[0] |= lo & 0x7F00u;
+  d.x[0] |= (lo << 1) & 0x7F0000u;
+  d.x[1] = (up & 0x7Fu) | top;
+  d.x[1] |= (up << 1) & 0x7F00u;
+  d.x[1] |= (up << 2) & 0xFF0000u;   // the top digit plus 64 reaches 128
+  return d;
+}
+
+// Digits of slice i (0 = most significant) of two entries, less the 64, as a packed
+// pair of 16-bit floats: 128 + e (1024 + e) less 192 (1088) is exact.
+template <bool F16>
+__device__ __forceinline__ uint32_t digit_pair(const DigitBytes& a, const DigitBytes& b, int i) {
+  const int w = i < 3, byte = w ? 2 - i : 5 - i;
+  const uint32_t p = __byte_perm(a.x[w], b.x[w], 0x7030u + 0x0400u + 0x0101u * (uint32_t)byte);
+  if constexpr (F16) {
+    const __half2 r = __hadd2(*(const __half2*)&p, __floats2half2_rn(-1088.0f, -1088.0f));
+    return *(const uint32_t*)&r;
+  } else {
+    const __nv_bfloat162 r = __hadd2(*(const __nv_bfloat162*)&p, __floats2bfloat162_rn(-192.0f, -192.0f));
+    return *(const uint32_t*)&r;
+  }
+}
+
 // Slices of the packed operands, one CTA (8 warps) per work item.  Rows are
 // taken in groups of 8 (rows past an operand's end give zero slices); in a
 // warp, lane = (row in group) * 4 + (8-column group).  A job gives each group
 // SliceJob::wpg warps (1, 2, 4 or 8: more for longer rows), so an item is
-// 8 / wpg groups.  For a group, first the biased exponent of each row's
-// largest |x| (lanes of a row scan every 4 * wpg-th entry's exponent field,
-// then the lanes and the group's warps combine), stored for the GEMM epilogue;
-// then the group's 32-wide K tiles are sliced, the warps of the group taking
-// every wpg-th tile, 8 entries per lane, 16 bytes per slice per lane written
-// in the tiled core-matrix layout the GEMM copies in.
+// 8 / wpg groups; the warps of a group take every wpg-th 32-wide K tile, 8 entries
+// per lane.  First the biased exponent of each row's largest |x| (over a lane's
+// entries, then the lanes and the group's warps combine), stored for the GEMM
+// epilogue; then the tiles are sliced, 16 bytes per slice per lane written in the
+// tiled core-matrix layout the GEMM copies in.
+// A warp keeps the entries of its first two tiles in registers between the two
+// parts (all of them for K up to 512), and reads ahead by two tiles past that.
 // With KX (K balancing), entry k counts as x * 2^(kx_sign * E_k), E_k the
 // exponent of column k's largest entry in A: A's columns are scaled by 2^-E_k
 // and B's rows by 2^E_k, exactly, so the product is unchanged while a row of
 // A (column of B) whose entries scale differently along K keeps its bits.
 // Only exponents move: the digits of x * 2^s are those of x with the
 // effective exponent E + s.
+// Instruction issue and load latency bound it.  Digits through byte permutes and
+// packed 16-bit adds (33 instead of about 56 integer and FP32 instructions per entry)
+// and one read of every entry instead of two: 47 -> 36 us for the last operand's 7.2M
+// entries at bond dimension 2048 (ncu, cold), the vector mode 21.5 -> 16.4 us.
 __device__ __forceinline__ int kx_shift(int raw, int sign) {
   return raw > 0 ? sign * (raw - 1023) : 0;   // raw: biased exponent, 0 for a zero column
 }
@@ -234,10 +283,11 @@ __device__ __forceinline__ int kx_shift(int raw, int sign) {
 // Lanczos vector through the row table, scaled by *inv, and the scaled values
 // are written out as the next basis vector (VecSrc).
 template <bool F16, bool KX, bool VEC>
-__global__ void __launch_bounds__(256) slice_rows_kernel(const SliceJob* __restrict__ jobs,
-                                                         const int2* __restrict__ items, int64_t total,
-                                                         double* const* __restrict__ slots, VecSrc vs) {
+__global__ void __launch_bounds__(256, 3) slice_rows_kernel(const SliceJob* __restrict__ jobs,
+                                                            const int2* __restrict__ items, int64_t total,
+                                                            double* const* __restrict__ slots, VecSrc vs) {
   static_assert(!(KX && VEC), "vector mode slices without K balancing");
+  static_assert(MAXN * 7 == 42, "digit_bytes: 53 - 42 = 11 bits go with a shift of 0");
   tnx_grid_dependency();
   if constexpr (VEC) {
     if (*(volatile const int32_t*)(vs.state + 1) != 0) return;   // the solve has stopped
@@ -246,15 +296,15 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const SliceJob* __restr
   __shared__ int s_max[8][8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int r8 = lane >> 2, kq = lane & 3;
-  constexpr int F = MAXN * 7;   // six digits of 7 bits (checked by the launcher)
   for (int64_t w = blockIdx.x; w < total; w += gridDim.x) {
     const int2 item = items[w];   // (job, first 8-row group)
     const SliceJob& j = jobs[item.x];
     const int wpg = j.wpg;                        // uniform over the CTA
     const int sub = wid / wpg, wl = wid - sub * wpg;
-    const int64_t ngroups = ((int64_t)j.rows + j.tile_rows - 1) / j.tile_rows * (j.tile_rows / 8);
+    const int tile_rows = j.tile_rows, K = j.K;
+    const int64_t ngroups = ((int64_t)j.rows + tile_rows - 1) / tile_rows * (tile_rows / 8);
     const int64_t rg = (int64_t)item.y + sub;
-    const int KT = (j.K + TK - 1) / TK;
+    const int KT = (K + TK - 1) / TK;
     const int64_t row = rg * 8 + r8;
     const bool live = rg < ngroups && row < j.rows;
     int64_t voff = 0;   // vector mode: offset of the row's K entries in the vector
@@ -265,36 +315,71 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const SliceJob* __restr
     } else {
       src = slots[j.src_slot] + j.src_off + row * j.ld;
     }
-    // row exponent: the largest (effective) exponent field; eight independent
-    // loads of the high words in flight per lane
-    const uint32_t* src_hi = (const uint32_t*)src + 1;
     const int32_t* kxp = KX ? (const int32_t*)slots[j.kx_slot] + j.kx_off : nullptr;
-    const int kstart = wl * 4 + kq, kstep = 4 * wpg;
+    // This lane's 8 entries of K tile kt (zeros past K).  Packed rows are whole
+    // 32-byte units (ld a multiple of 4, bases 32-byte aligned).
+    auto load = [&](int kt, unsigned long long (&x)[8], bool keep) {
+      const int k = kt * TK + kq * 8;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x[e] = 0ull;
+      if (!live || k >= K) return;
+      if constexpr (VEC) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if (k + e < K) {
+            const double v = src[k + e] * vinv;
+            if (keep) vs.vdst[voff + k + e] = v;
+            x[e] = (unsigned long long)__double_as_longlong(v);
+          }
+      } else {
+        const ulonglong2* p = (const ulonglong2*)(src + k);
+#pragma unroll
+        for (int h = 0; h < 4; ++h)
+          if (k + 2 * h < K) {
+            const ulonglong2 v = p[h];
+            x[2 * h] = v.x;
+            x[2 * h + 1] = k + 2 * h + 1 < K ? v.y : 0ull;
+          }
+      }
+    };
+    auto shifts = [&](int kt, int (&sh)[8]) {   // K balancing words: whole K tiles, 16-byte aligned
+      if constexpr (KX) {
+        const int4* p = (const int4*)(kxp + kt * TK + kq * 8);
+        const int4 a = p[0], b = p[1];
+        const int raw[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) sh[e] = kx_shift(raw[e], j.kx_sign);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) sh[e] = 0;
+      }
+    };
     constexpr int ZROW = KX ? -(1 << 20) : 0;   // no nonzero entry
     int mx = ZROW;
-    if (live)
-      for (int k0 = kstart; k0 < j.K; k0 += 8 * kstep) {
-        uint32_t h[8];
-        int sx[8];
+    auto scan = [&](int kt, const unsigned long long (&x)[8]) {   // the largest (effective) exponent field
+      if (!live || kt >= KT) return;
+      int sh[8];
+      shifts(kt, sh);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int k = k0 + u * kstep;
-          if constexpr (VEC)
-            h[u] = k < j.K ? (uint32_t)((unsigned long long)__double_as_longlong(src[k] * vinv) >> 32) : 0u;
-          else
-            h[u] = k < j.K ? src_hi[2 * k] : 0u;
-          if constexpr (KX) sx[u] = k < j.K ? kxp[k] : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int eb = (int)((h[u] >> 20) & 0x7FFu);
-          if constexpr (KX) {
-            if (eb != 0) mx = max(mx, eb + kx_shift(sx[u], j.kx_sign));
-          } else {
-            mx = max(mx, eb);
-          }
+      for (int e = 0; e < 8; ++e) {
+        const int eb = (int)((x[e] >> 52) & 0x7FF);
+        if constexpr (KX) {
+          if (eb != 0) mx = max(mx, eb + sh[e]);
+        } else {
+          mx = max(mx, eb);
         }
       }
+    };
+    unsigned long long x0[8], x1[8];
+    load(wl, x0, true);
+    load(wl + wpg, x1, true);
+    scan(wl, x0);
+    scan(wl + wpg, x1);
+    for (int kt = wl + 2 * wpg; kt < KT; kt += wpg) {
+      unsigned long long x2[8];
+      load(kt, x2, false);
+      scan(kt, x2);
+    }
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (wpg > 1) {
@@ -305,127 +390,28 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const SliceJob* __restr
     }
     if (rg >= ngroups) continue;   // a group past the job's last one
     const int eb_r = mx;
-    const bool nonzero_row = eb_r != ZROW;
-    if (live && kq == 0 && wl == 0) ((int32_t*)slots[j.exp_slot])[j.exp_off + row] = nonzero_row ? eb_r : 0;
-    const int tile_rows = j.tile_rows;
+    if (live && kq == 0 && wl == 0) ((int32_t*)slots[j.exp_slot])[j.exp_off + row] = eb_r != ZROW ? eb_r : 0;
     const int64_t mt = row / tile_rows;
     const int rin = (int)(row % tile_rows);
     const int64_t tile_bytes = (int64_t)tile_rows * TK * 2;
-    char* base = (char*)slots[j.dst_slot] + j.dst_off_bytes;
-    const int64_t inner = (int64_t)(rin >> 3) * 512 + kq * 128 + (rin & 7) * 16;
-    // Digits of one K tile (8 entries per lane); the loads of the lane's next
-    // tile are issued before the current one is converted.
-    // With KX the K-balancing words of the tile come along (each group's region
-    // is padded to whole K tiles and 16-byte aligned).
-    const int kt0 = wl, kts = wpg;
-    unsigned long long cur[8];
-    int4 ckx[2];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int k = kt0 * TK + kq * 8 + e;
-      if constexpr (VEC) {
-        cur[e] = 0ull;
-        if (live && kt0 < KT && k < j.K) {
-          const double x = src[k] * vinv;
-          vs.vdst[voff + k] = x;
-          cur[e] = (unsigned long long)__double_as_longlong(x);
-        }
-      } else {
-        cur[e] = (live && kt0 < KT && k < j.K) ? (unsigned long long)__double_as_longlong(src[k]) : 0ull;
-      }
-    }
-    if constexpr (KX) {
-      const bool ok = live && kt0 < KT;
-      ckx[0] = ok ? *(const int4*)(kxp + kt0 * TK + kq * 8) : make_int4(0, 0, 0, 0);
-      ckx[1] = ok ? *(const int4*)(kxp + kt0 * TK + kq * 8 + 4) : make_int4(0, 0, 0, 0);
-    }
-    for (int kt = kt0; kt < KT; kt += kts) {
-      unsigned long long nxt[8];
-      int4 nkx[2];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int k = (kt + kts) * TK + kq * 8 + e;
-        if constexpr (VEC) {
-          nxt[e] = 0ull;
-          if (live && kt + kts < KT && k < j.K) {
-            const double x = src[k] * vinv;
-            vs.vdst[voff + k] = x;
-            nxt[e] = (unsigned long long)__double_as_longlong(x);
-          }
-        } else {
-          nxt[e] = (live && kt + kts < KT && k < j.K) ? (unsigned long long)__double_as_longlong(src[k]) : 0ull;
-        }
-      }
-      if constexpr (KX) {
-        const bool ok = live && kt + kts < KT;
-        nkx[0] = ok ? *(const int4*)(kxp + (kt + kts) * TK + kq * 8) : make_int4(0, 0, 0, 0);
-        nkx[1] = ok ? *(const int4*)(kxp + (kt + kts) * TK + kq * 8 + 4) : make_int4(0, 0, 0, 0);
-      }
+    char* base = (char*)slots[j.dst_slot] + j.dst_off_bytes + (int64_t)(rin >> 3) * 512 + kq * 128 + (rin & 7) * 16;
+    for (int kt = wl; kt < KT; kt += wpg) {
       int sh[8];
-      if constexpr (KX) {
-        const int raw[8] = {ckx[0].x, ckx[0].y, ckx[0].z, ckx[0].w, ckx[1].x, ckx[1].y, ckx[1].z, ckx[1].w};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) sh[e] = kx_shift(raw[e], j.kx_sign);
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) sh[e] = 0;
-      }
+      shifts(kt, sh);
       uint32_t sl[MAXN][4];
 #pragma unroll
       for (int e = 0; e < 8; e += 2) {
-        float f[2][MAXN];
+        const DigitBytes a = digit_bytes<F16>(x0[e], eb_r - (int)((x0[e] >> 52) & 0x7FF) - sh[e]);
+        const DigitBytes c = digit_bytes<F16>(x0[e + 1], eb_r - (int)((x0[e + 1] >> 52) & 0x7FF) - sh[e + 1]);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const unsigned long long bits = cur[e + h];
-          const int eb = (int)((bits >> 52) & 0x7FF);
-          // |x| 2^(F-E-2) rounded half up: m53 * 2^-rs with rs = 54 - F + E_r - E >= 12
-          unsigned long long fix = 0;
-          if (eb != 0 && nonzero_row) {
-            const unsigned long long m53 = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-            const int rs = 54 - F + (eb_r - (eb + sh[e + h]));
-            fix = rs >= 64 ? 0ull : ((m53 >> (rs - 1)) + 1ull) >> 1;
-          }
-          // Balanced base-128 digits of the signed value v (|v| <= 2^41): with
-          // u = v + 64 * sum_i 128^i >= 0, the plain 7-bit digits e_i of u give
-          // d_i = e_i - 64 in [-64, 63] (the top digit takes the rest, at most 64),
-          // and sum_i d_i 128^i = v.
-          const long long v = (bits >> 63) ? -(long long)fix : (long long)fix;
-          const unsigned long long u = (unsigned long long)(v + DIGIT_BIAS);
-          const uint32_t lo = (uint32_t)(u & 0x1FFFFFull), hi = (uint32_t)(u >> 21);
-          uint32_t dg[MAXN];   // e_i of slice i (slice 0 = most significant)
-          dg[5] = lo & 127u;
-          dg[4] = (lo >> 7) & 127u;
-          dg[3] = lo >> 14;
-          dg[2] = hi & 127u;
-          dg[1] = (hi >> 7) & 127u;
-          dg[0] = hi >> 14;
-          // d = e - 64 exactly as FP32: in the binade of 1.5 * 2^23 one unit of the
-          // bit pattern is one unit of value, so (bits 0x4B400000 + d) - 1.5 * 2^23 = d
-#pragma unroll
-          for (int i = 0; i < MAXN; ++i) f[h][i] = __int_as_float(0x4B3FFFC0 + (int)dg[i]) - 12582912.0f;
-        }
-#pragma unroll
-        for (int i = 0; i < MAXN; ++i) {
-          // |d| <= 64 is exact in BF16 (the top half of the FP32 word) and in FP16
-          if constexpr (F16) {
-            const __half2 hh = __floats2half2_rn(f[0][i], f[1][i]);
-            sl[i][e >> 1] = *(const uint32_t*)&hh;
-          } else {
-            sl[i][e >> 1] = __byte_perm(__float_as_uint(f[0][i]), __float_as_uint(f[1][i]), 0x7632);
-          }
-        }
+        for (int i = 0; i < MAXN; ++i) sl[i][e >> 1] = digit_pair<F16>(a, c, i);
       }
+      char* dst = base + (mt * KT + kt) * MAXN * tile_bytes;
 #pragma unroll
-      for (int i = 0; i < MAXN; ++i) {
-        uint4 v = make_uint4(sl[i][0], sl[i][1], sl[i][2], sl[i][3]);
-        *(uint4*)(base + ((mt * KT + kt) * MAXN + i) * tile_bytes + inner) = v;
-      }
+      for (int i = 0; i < MAXN; ++i) *(uint4*)(dst + i * tile_bytes) = make_uint4(sl[i][0], sl[i][1], sl[i][2], sl[i][3]);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) cur[e] = nxt[e];
-      if constexpr (KX) {
-        ckx[0] = nkx[0];
-        ckx[1] = nkx[1];
-      }
+      for (int e = 0; e < 8; ++e) x0[e] = x1[e];
+      if (kt + 2 * wpg < KT) load(kt + 2 * wpg, x1, true);
     }
   }
 }

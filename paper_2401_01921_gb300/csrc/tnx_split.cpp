@@ -16,14 +16,14 @@ constexpr int64_t KMAX = 8192;   // the 64-bit fixed-point accumulator is exact 
 
 // Work items of one slicing launch (k_split.cu), one CTA (8 warps) each: a
 // job gives each 8-row group 1, 2, 4 or 8 warps by the number of its 32-wide
-// K tiles (a warp then takes about two of them, at most every eighth), and an
-// item holds 8 / wpg consecutive groups of one job.
+// K tiles, so that a warp takes at most two of them, which it keeps in registers
+// (more above K = 512 only), and an item holds 8 / wpg consecutive groups of one job.
 std::vector<int2> tnx_slice_schedule(std::vector<SliceJob>& jobs) {
   std::vector<int2> items;
   for (size_t q = 0; q < jobs.size(); ++q) {
     SliceJob& j = jobs[q];
     const int KT = (j.K + TK - 1) / TK;
-    j.wpg = KT >= 16 ? 8 : KT >= 8 ? 4 : KT >= 3 ? 2 : 1;
+    j.wpg = KT > 8 ? 8 : KT > 4 ? 4 : KT > 2 ? 2 : 1;
     const int64_t g = ((int64_t)j.rows + j.tile_rows - 1) / j.tile_rows * (j.tile_rows / 8);
     if (g > INT32_MAX) fail(TNX_ERR_UNSUPPORTED, "slicing job above 2^31 row groups");
     for (int64_t r = 0; r < g; r += 8 / j.wpg) items.push_back(make_int2((int)q, (int)r));
