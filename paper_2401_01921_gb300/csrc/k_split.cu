@@ -42,6 +42,7 @@
 // two and rounded to TF32 (10 explicit mantissa bits, nearest-even), 16 K
 // values (64 bytes) per stage and row, tcgen05.mma.kind::tf32 with FP32
 // accumulation per 640-long K chunk, chunks summed in FP64 by the epilogue.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -255,7 +256,8 @@ __device__ __forceinline__ uint32_t digit_pair(const DigitBytes& a, const DigitB
 }
 
 // Slices of the packed operands, one CTA (8 warps) per work item.  Rows are
-// taken in groups of 8 (rows past an operand's end give zero slices); in a
+// taken in groups of 8 (rows past the operand's end in its last group give zero
+// slices; the rows that pad it to whole tiles keep the zeros of the allocation); in a
 // warp, lane = (row in group) * 4 + (8-column group).  A job gives each group
 // SliceJob::wpg warps (1, 2, 4 or 8: more for longer rows), so an item is
 // 8 / wpg groups; the warps of a group take every wpg-th 32-wide K tile, 8 entries
@@ -302,7 +304,7 @@ __global__ void __launch_bounds__(256, 3) slice_rows_kernel(const SliceJob* __re
     const int wpg = j.wpg;                        // uniform over the CTA
     const int sub = wid / wpg, wl = wid - sub * wpg;
     const int tile_rows = j.tile_rows, K = j.K;
-    const int64_t ngroups = ((int64_t)j.rows + tile_rows - 1) / tile_rows * (tile_rows / 8);
+    const int64_t ngroups = ((int64_t)j.rows + 7) / 8;
     const int64_t rg = (int64_t)item.y + sub;
     const int KT = (K + TK - 1) / TK;
     const int64_t row = rg * 8 + r8;
@@ -416,50 +418,55 @@ __global__ void __launch_bounds__(256, 3) slice_rows_kernel(const SliceJob* __re
   }
 }
 
-// Zeroes the K-balancing words of every job (whole K tiles), one CTA per job.
-__global__ void kexp_zero_kernel(const KexpJob* __restrict__ jobs, int njobs, double* const* __restrict__ slots) {
+// Column maxima of the exponent fields of A: an item is 32 K indices (one per lane)
+// and all rows (eight per warp and pass, loads in flight together).  Its CL CTAs, a
+// cluster, share the rows; each combines its warps in its shared memory, and the
+// first adds the others' maxima from there and stores one word per K index.  A maximum
+// across unrelated CTAs wanted a launch that zeroes the words first (3 us per product);
+// a single CTA per item is too slow for the 1280 rows of an environment update at
+// bond dimension 2048 (19 us; 12 with the zeroing launch; 11 with clusters of 8).
+constexpr int KEXP_T = 256, KEXP_CL = 8;
+template <int CL>
+__global__ void __launch_bounds__(KEXP_T) kexp_kernel(const KexpJob* __restrict__ jobs,
+                                                      const int2* __restrict__ items, double* const* __restrict__ slots) {
   tnx_grid_dependency();
-  for (int q = blockIdx.x; q < njobs; q += gridDim.x) {
-    const KexpJob& j = jobs[q];
-    int32_t* kx = (int32_t*)slots[j.kx_slot] + j.kx_off;
-    const int n = (j.K + TK - 1) / TK * TK;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) kx[i] = 0;
-  }
-}
-
-// Column maxima of the exponent fields of A: an item is 32 K indices (one per
-// lane) by 64 rows (eight per warp, loads in flight together); the warps
-// combine in shared memory and one atomicMax per K index leaves the CTA.
-__global__ void __launch_bounds__(256) kexp_kernel(const KexpJob* __restrict__ jobs, const int4* __restrict__ items,
-                                                   int64_t nitems, double* const* __restrict__ slots) {
-  tnx_grid_dependency();
-  __shared__ int s_mx[8][32];
+  constexpr int NW = KEXP_T / 32;
+  __shared__ int s_mx[NW][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int64_t w = blockIdx.x; w < nitems; w += gridDim.x) {
-    const int4 it = items[w];   // (job, first K index, first row, -)
-    const KexpJob& j = jobs[it.x];
-    const int k = it.y + lane;
-    int mx = 0;
-    if (k < j.K) {
-      const uint32_t* hi = (const uint32_t*)(slots[j.src_slot] + j.src_off) + 1;
+  const int rank = CL > 1 ? (int)(blockIdx.x % CL) : 0;
+  const int2 it = items[blockIdx.x / CL];   // (job, first K index)
+  const KexpJob& j = jobs[it.x];
+  const int k = it.y + lane;
+  int mx = 0;
+  if (k < j.K) {
+    const uint32_t* hi = (const uint32_t*)(slots[j.src_slot] + j.src_off + k) + 1;
+    for (int r0 = rank * NW + wid; r0 < j.rows; r0 += 8 * NW * CL) {
       uint32_t h[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int r = it.z + wid + 8 * u;
-        h[u] = r < j.rows ? hi[2 * ((int64_t)r * j.ld + k)] : 0u;
+        const int r = r0 + NW * CL * u;
+        h[u] = r < j.rows ? hi[2 * ((int64_t)r * j.ld)] : 0u;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) mx = max(mx, (int)((h[u] >> 20) & 0x7FFu));
     }
-    s_mx[wid][lane] = mx;
-    __syncthreads();
-    if (wid == 0) {
-#pragma unroll
-      for (int q = 1; q < 8; ++q) mx = max(mx, s_mx[q][lane]);
-      if (k < j.K && mx > 0) atomicMax((int32_t*)slots[j.kx_slot] + j.kx_off + k, mx);
-    }
-    __syncthreads();
   }
+  s_mx[wid][lane] = mx;
+  __syncthreads();
+  if (wid == 0) {
+#pragma unroll
+    for (int q = 1; q < NW; ++q) mx = max(mx, s_mx[q][lane]);
+    if (CL > 1) s_mx[0][lane] = mx;
+  }
+  if constexpr (CL > 1) {
+    auto cluster = cooperative_groups::this_cluster();
+    cluster.sync();
+    if (rank == 0 && wid == 0)
+#pragma unroll
+      for (int c = 1; c < CL; ++c) mx = max(mx, cluster.map_shared_rank(&s_mx[0][0], c)[lane]);
+    cluster.sync();   // no CTA leaves while its maxima are read
+  }
+  if (rank == 0 && wid == 0 && k < j.K) ((int32_t*)slots[j.kx_slot])[j.kx_off + k] = mx;
 }
 
 // TF32 operands of the one-pass variant: one CTA (8 warps) per item of eight
@@ -846,16 +853,30 @@ cudaError_t tnx_launch_slices_vec(const SliceJob* jobs, const int2* items, int64
   return cudaGetLastError();
 }
 
-cudaError_t tnx_launch_kexp(const KexpJob* jobs, int njobs, const int4* items, int64_t nitems, double* const* slots,
-                            cudaStream_t st) {
-  if (njobs <= 0 || nitems <= 0) return cudaSuccess;
-  cudaError_t le = tnx_launch(kexp_zero_kernel, dim3(njobs < 1024 ? njobs : 1024), dim3(256), 0, st, jobs, njobs,
-                              slots);
+cudaError_t tnx_launch_kexp(const KexpJob* jobs, const int2* items, int64_t nitems, bool cluster,
+                            double* const* slots, cudaStream_t st) {
+  if (nitems <= 0) return cudaSuccess;
+  if (nitems > INT32_MAX / KEXP_CL) return cudaErrorInvalidValue;
+  cudaError_t le;
+  if (!cluster) {
+    le = tnx_launch(kexp_kernel<1>, dim3((int)nitems), dim3(KEXP_T), 0, st, jobs, items, slots);
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((int)nitems * KEXP_CL);
+    cfg.blockDim = dim3(KEXP_T);
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = KEXP_CL;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    le = cudaLaunchKernelEx(&cfg, kexp_kernel<KEXP_CL>, jobs, items, slots);
+  }
   if (le != cudaSuccess) return le;
-  const int64_t blocks = nitems < 152 * 8 ? nitems : 152 * 8;
-  le = tnx_launch(kexp_kernel, dim3((int)blocks), dim3(256), 0, st, jobs, items, nitems, slots);
-  if (le != cudaSuccess) return le;
-  tnx_note_launch(2);
+  tnx_note_launch(1);
   return cudaGetLastError();
 }
 

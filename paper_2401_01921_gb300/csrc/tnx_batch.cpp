@@ -29,9 +29,9 @@ struct BStep {
   int edge = 64;                // of the FP64 tiles
   StepPlan::Jobs jobs;
   KexpJob* dKJ = nullptr;       // K balancing of the split steps (every launch: all operands are new)
-  int nkj = 0;
-  int4* dKI = nullptr;
+  int2* dKI = nullptr;
   int64_t nki = 0;
+  bool kx_cluster = false;
   SplitGroup* dSG = nullptr;
   GemmTile* dST = nullptr;
   int nst = 0;
@@ -129,7 +129,7 @@ void enqueue_batch(tnx_batch& B, cudaStream_t st) {
     } else {
       if (s.jobs.n) {
         ProfScope ps(c, st, TNX_KC_SLICE, (double)s.jobs.elems * (16.0 + 2.0 * B.nslice));
-        CUDA_CHECK(tnx_launch_kexp(s.dKJ, s.nkj, s.dKI, s.nki, B.d_slots, st));
+        CUDA_CHECK(tnx_launch_kexp(s.dKJ, s.dKI, s.nki, s.kx_cluster, B.d_slots, st));
         CUDA_CHECK(tnx_launch_slices(s.jobs.d, s.jobs.items, s.jobs.nitems, B.nslice, B.beta, f16, B.d_slots, st, 1));
       }
       ProfScope ps(c, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
@@ -294,9 +294,8 @@ extern "C" tnx_status tnx_batch_create(tnx_ctx* ctx, int n, tnx_network* const* 
         bs.jobs.nitems = (int64_t)items.size();
         bs.jobs.d = B->upload(jobs);
         bs.jobs.items = B->upload(items);
-        const std::vector<int4> kitems = tnx_kexp_items(kjobs);
+        const std::vector<int2> kitems = tnx_kexp_items(kjobs, bs.kx_cluster);
         bs.dKJ = B->upload(kjobs);
-        bs.nkj = (int)kjobs.size();
         bs.dKI = B->upload(kitems);
         bs.nki = (int64_t)kitems.size();
         bs.dSG = B->upload(sg);

@@ -78,9 +78,8 @@ struct SliceJob {
 };
 
 // K balancing of a split product: for every K index k of a charge group, the
-// largest exponent field over the rows of the packed A (atomicMax into
-// zeroed int32 words).  Items: (job, first K index, first row), 32 K indices
-// by 64 rows each.
+// largest exponent field over the rows of the packed A.  Items: (job, first K
+// index), 32 K indices each.
 struct KexpJob {
   int32_t src_slot, kx_slot;
   int64_t src_off, kx_off;
@@ -281,9 +280,10 @@ cudaError_t tnx_launch_slices_vec(const SliceJob* jobs, const int2* items, int64
                                   int f16, double* const* slots, const VecSrc& vs, cudaStream_t st);
 cudaError_t tnx_launch_slices(const SliceJob* jobs, const int2* items, int64_t total_items, int nslice, int beta,
                               int f16, double* const* slots, cudaStream_t st, int use_kx = 0);
-// zero the K-balancing words of every job, then their column maxima
-cudaError_t tnx_launch_kexp(const KexpJob* jobs, int njobs, const int4* items, int64_t nitems, double* const* slots,
-                            cudaStream_t st);
+// the K-balancing words of every job (column maxima over its rows); items: (job, first
+// of 32 K indices); cluster: eight CTAs per item instead of one
+cudaError_t tnx_launch_kexp(const KexpJob* jobs, const int2* items, int64_t nitems, bool cluster,
+                            double* const* slots, cudaStream_t st);
 // grid <= 0 or >= ntiles: one CTA per tile; otherwise a persistent grid of `grid` CTAs.
 // tn: tile width (B rows per tile), 64 or 32; the B slices must be tiled with the same width.
 cudaError_t tnx_launch_gemm_split(const SplitGroup* groups, const GemmTile* tiles, int ntiles, int nslice,

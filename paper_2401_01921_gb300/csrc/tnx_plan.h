@@ -70,9 +70,9 @@ struct StepPlan {
   int slotSA = -1, slotSB = -1, slotEA = -1, slotEB = -1;
   int slotKX = -1;              // K balancing words (int32, whole K tiles per group)
   KexpJob* dKJ = nullptr;       // their jobs (one per split group) and work items
-  int nkj = 0;
-  int4* dKI = nullptr;
+  int2* dKI = nullptr;
   int64_t nki = 0;
+  bool kx_cluster = false;
   std::vector<KexpJob> hKJ;     // host copy (batched plans merge them)
   struct Jobs {             // one slicing launch: its jobs and work items
     SliceJob* d = nullptr;
@@ -195,7 +195,8 @@ struct tnx_network {
 // split-precision planning and launch (tnx_split.cpp)
 void tnx_build_split_parts(Plan& p, StepPlan& s);
 // balance: K-balanced slicing (A's column exponents), recomputed when A is
-std::vector<int4> tnx_kexp_items(const std::vector<KexpJob>& jobs);
+// cluster: whether the launch takes a cluster of CTAs per item
+std::vector<int2> tnx_kexp_items(const std::vector<KexpJob>& jobs, bool& cluster);
 void tnx_enqueue_split(Plan& p, StepPlan& s, cudaStream_t st, bool needA, bool needB, bool balance);
 std::vector<int2> tnx_slice_schedule(std::vector<SliceJob>& jobs);
 std::vector<int2> tnx_tf32_schedule(std::vector<SliceJob>& jobs);

@@ -18,13 +18,16 @@ constexpr int64_t KMAX = 8192;   // the 64-bit fixed-point accumulator is exact 
 // job gives each 8-row group 1, 2, 4 or 8 warps by the number of its 32-wide
 // K tiles, so that a warp takes at most two of them, which it keeps in registers
 // (more above K = 512 only), and an item holds 8 / wpg consecutive groups of one job.
+// The groups that only pad an operand to whole GEMM tiles are left out: their slices
+// are zeros since the buffers were allocated, and nothing else writes them (a charge
+// sector of a Hubbard instance has 1 to 30 rows in a tile of 128).
 std::vector<int2> tnx_slice_schedule(std::vector<SliceJob>& jobs) {
   std::vector<int2> items;
   for (size_t q = 0; q < jobs.size(); ++q) {
     SliceJob& j = jobs[q];
     const int KT = (j.K + TK - 1) / TK;
     j.wpg = KT > 8 ? 8 : KT > 4 ? 4 : KT > 2 ? 2 : 1;
-    const int64_t g = ((int64_t)j.rows + j.tile_rows - 1) / j.tile_rows * (j.tile_rows / 8);
+    const int64_t g = ((int64_t)j.rows + 7) / 8;
     if (g > INT32_MAX) fail(TNX_ERR_UNSUPPORTED, "slicing job above 2^31 row groups");
     for (int64_t r = 0; r < g; r += 8 / j.wpg) items.push_back(make_int2((int)q, (int)r));
   }
@@ -140,9 +143,8 @@ void tnx_build_split_parts(Plan& p, StepPlan& s) {
       k.ld = (int32_t)s.ldK[g];
       kj.push_back(k);
     }
-    const std::vector<int4> ki = tnx_kexp_items(kj);
+    const std::vector<int2> ki = tnx_kexp_items(kj, s.kx_cluster);
     s.dKJ = p.upload(kj);
-    s.nkj = (int)kj.size();
     s.dKI = p.upload(ki);
     s.nki = (int64_t)ki.size();
     s.hKJ = kj;
@@ -221,12 +223,20 @@ void tnx_build_split_parts(Plan& p, StepPlan& s) {
   s.hST = tiles;
 }
 
-// Work items of the K-balancing pass: 32 K indices by 64 rows each.
-std::vector<int4> tnx_kexp_items(const std::vector<KexpJob>& jobs) {
-  std::vector<int4> items;
+// Work items of the K-balancing pass: 32 K indices of one job each, all its rows;
+// by a cluster of CTAs when an item has more than 96 rows on average (a CTA reads 64
+// at a time) and the items alone leave the SMs with less than four CTAs (one apply at
+// bond dimension 777: 7 us with clusters, 16 without; at 4096, 1000 items: 28 with, 16
+// without).
+std::vector<int2> tnx_kexp_items(const std::vector<KexpJob>& jobs, bool& cluster) {
+  std::vector<int2> items;
+  int64_t rows = 0;
   for (size_t q = 0; q < jobs.size(); ++q)
-    for (int k0 = 0; k0 < jobs[q].K; k0 += 32)
-      for (int r0 = 0; r0 < jobs[q].rows; r0 += 64) items.push_back(make_int4((int)q, k0, r0, 0));
+    for (int k0 = 0; k0 < jobs[q].K; k0 += 32) {
+      items.push_back(make_int2((int)q, k0));
+      rows += jobs[q].rows;
+    }
+  cluster = rows > 96 * (int64_t)items.size() && items.size() < 4 * 152;
   return items;
 }
 
@@ -247,7 +257,7 @@ void tnx_enqueue_split(Plan& p, StepPlan& s, cudaStream_t st, bool needA, bool n
   }
   if (J && J->n) {
     ProfScope ps(p.ctx, st, TNX_KC_SLICE, (double)J->elems * (8.0 + 8.0 + 2.0 * p.nslice));
-    if (balance && needA) CUDA_CHECK(tnx_launch_kexp(s.dKJ, s.nkj, s.dKI, s.nki, p.d_slots, st));
+    if (balance && needA) CUDA_CHECK(tnx_launch_kexp(s.dKJ, s.dKI, s.nki, s.kx_cluster, p.d_slots, st));
     CUDA_CHECK(tnx_launch_slices(J->d, J->items, J->nitems, p.nslice, p.beta, f16, p.d_slots, st, balance ? 1 : 0));
   }
   ProfScope ps(p.ctx, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
