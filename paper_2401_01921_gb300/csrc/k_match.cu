@@ -16,7 +16,7 @@
 // Tuple spaces are enumerated in mixed radix (first leg most significant), so
 // increasing tuple id is lexicographic order.  One CTA of 1024 threads runs
 // all phases, separated by __syncthreads(); the weighted prefix sums per group
-// use a stable per-thread-chunk counting scan.  Runs once per plan.
+// use a stable per-thread-chunk counting scan, a warp per group.  Runs once per plan.
 #include "tnx_internal.h"
 
 namespace {
@@ -69,32 +69,48 @@ __device__ int64_t kcharge_index(const MatchArgs& a, int64_t id) {
 
 // Stable weighted prefix sum per group over items [0, n) in index order.
 // grp(i) < 0: item skipped.  off[i] = sum of weights of earlier items of the
-// same group; totals[g] = group total.  tmp: T * G int64 scratch.
+// same group; totals[g] = group total.  tmp: T * G int64 scratch, row g holding the
+// chunk sums of group g.  A warp turns a row into prefix sums, 8 x 32 chunks at a time
+// with their loads in flight together (one thread walking its 1024 chunks took most
+// of the kernel: 134 -> 47 us on average for the products of a bond update at bond dimension 256).
 template <class GrpF, class WF>
 __device__ void group_scan(int64_t n, int G, GrpF grp, WF weight, int64_t* off, int64_t* totals, int64_t* tmp) {
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const int64_t c0 = n * t / T, c1 = n * (t + 1) / T;
-  for (int g = 0; g < G; ++g) tmp[(int64_t)t * G + g] = 0;
+  for (int g = 0; g < G; ++g) tmp[(int64_t)g * T + t] = 0;
   for (int64_t i = c0; i < c1; ++i) {
     int g = grp(i);
-    if (g >= 0) tmp[(int64_t)t * G + g] += weight(i);
+    if (g >= 0) tmp[(int64_t)g * T + t] += weight(i);
   }
   __syncthreads();
-  for (int g = t; g < G; g += T) {
+  for (int g = wid; g < G; g += T / 32) {
+    int64_t* row = tmp + (int64_t)g * T;
     int64_t run = 0;
-    for (int c = 0; c < T; ++c) {
-      int64_t v = tmp[(int64_t)c * G + g];
-      tmp[(int64_t)c * G + g] = run;
-      run += v;
+    for (int b = 0; b < T; b += 256) {
+      int64_t v[8], x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = v[u] = row[b + 32 * u + lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int64_t y = __shfl_up_sync(0xffffffffu, x[u], o);
+          if (lane >= o) x[u] += y;
+        }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        row[b + 32 * u + lane] = run + x[u] - v[u];
+        run += __shfl_sync(0xffffffffu, x[u], 31);
+      }
     }
-    totals[g] = run;
+    if (lane == 0) totals[g] = run;
   }
   __syncthreads();
   for (int64_t i = c0; i < c1; ++i) {
     int g = grp(i);
     if (g >= 0) {
-      off[i] = tmp[(int64_t)t * G + g];
-      tmp[(int64_t)t * G + g] += weight(i);
+      off[i] = tmp[(int64_t)g * T + t];
+      tmp[(int64_t)g * T + t] += weight(i);
     }
   }
   __syncthreads();
@@ -104,7 +120,7 @@ __global__ void __launch_bounds__(T) match_kernel(MatchArgs a) {
   const int t = threadIdx.x;
   __shared__ int32_t s_G;
   __shared__ int32_t s_bad;
-  __shared__ int32_t s_scan[T];
+  __shared__ int32_t s_scan[T / 32];
   if (t == 0) s_bad = 0;
 
   // phase 0: clear
@@ -155,15 +171,28 @@ __global__ void __launch_bounds__(T) match_kernel(MatchArgs a) {
     int64_t c0 = chunk * t, c1 = min(a.cspace, c0 + chunk);
     int32_t local = 0;
     for (int64_t i = c0; i < c1; ++i) local += a.cspres[i];
-    s_scan[t] = local;
+    // exclusive sums over the threads: within the warps, then over the 32 warps
+    const int lane = t & 31, wid = t >> 5;
+    int32_t x = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_scan[wid] = x;
     __syncthreads();
-    if (t == 0) {
-      int32_t run = 0;
-      for (int i = 0; i < T; ++i) { int32_t v = s_scan[i]; s_scan[i] = run; run += v; }
-      s_G = run;
+    if (wid == 0) {
+      int32_t w = s_scan[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += y;
+      }
+      s_scan[lane] = w;
+      if (lane == 31) s_G = w;
     }
     __syncthreads();
-    int32_t run = s_scan[t];
+    int32_t run = x - local + (wid > 0 ? s_scan[wid - 1] : 0);
     for (int64_t i = c0; i < c1; ++i) {
       a.csgid[i] = a.cspres[i] ? run : -1;
       run += a.cspres[i];
