@@ -158,16 +158,35 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
     }
     gather.push_back(c);
   }
+  // tables for the kernels: small ones share one device buffer, and go over together
+  // at the next flush (before the launches that read them)
   std::vector<std::unique_ptr<DevBuf>> tmp;
+  constexpr size_t kShared = 256 * 1024, kSmall = 32 * 1024;
+  DevBuf shared(ctx, kShared);
+  std::vector<char> stage(kShared);
+  size_t used = 0, sent = 0;
   auto up = [&](const void* src, size_t bytes) {
-    tmp.emplace_back(new DevBuf(ctx, std::max<size_t>(bytes, 256)));
+    const size_t n = (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
+    if (n <= kSmall && used + n <= kShared) {
+      if (bytes) memcpy(stage.data() + used, src, bytes);
+      void* p = (char*)shared.p + used;
+      used += n;
+      return p;
+    }
+    tmp.emplace_back(new DevBuf(ctx, n));
     if (bytes) CUDA_CHECK(cudaMemcpyAsync(tmp.back()->p, src, bytes, cudaMemcpyHostToDevice, st));
     return tmp.back()->p;
+  };
+  auto flush = [&] {
+    if (used > sent)
+      CUDA_CHECK(cudaMemcpyAsync((char*)shared.p + sent, stage.data() + sent, used - sent, cudaMemcpyHostToDevice, st));
+    sent = used;
   };
   const SvdGroup* dg = (const SvdGroup*)up(hg.data(), hg.size() * sizeof(SvdGroup));
   const int2* dslots = (const int2*)up(slots.data(), slots.size() * sizeof(int2));
   const int2* dvecs = (const int2*)up(vecs.data(), vecs.size() * sizeof(int2));
   const Copy2D* dgather = (const Copy2D*)up(gather.data(), gather.size() * sizeof(Copy2D));
+  flush();
   CUDA_CHECK(cudaMemsetAsync(dX, 0, (size_t)std::max<int64_t>(nX, 1) * 8, st));
   CUDA_CHECK(tnx_launch_copy2d(dgather, (int)gather.size(), st));
   constexpr int MAX_SWEEPS = 60;
@@ -253,6 +272,7 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
     unsigned long long* w = (unsigned long long*)up(zero.data(), zero.size() * 8);
     int* qstat = (int*)(w + 1);
     int* jstat = (int*)(w + MAX_SWEEPS + 3);
+    flush();
     const cudaError_t ce = tnx_launch_qr_coop(dq, dqs, (int)qslots.size(), maxc, w, qstat, st);
     if (ce == cudaSuccess) {
       CUDA_CHECK(tnx_launch_qr_gather_r(dq, ngr, maxc, st));
@@ -288,6 +308,7 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
     unsigned long long* w = (unsigned long long*)up(zero.data(), zero.size() * 8);
     unsigned long long* bar = w + MAX_SWEEPS;
     int* cstat = (int*)(w + MAX_SWEEPS + 1);
+    flush();
     const cudaError_t ce = tnx_launch_jacobi_coop(dg, dslots, (int)slots.size(), maxcp, maxr, MAX_SWEEPS, 1e-13, w,
                                                   bar, cstat, cstat + 1, st);
     if (ce == cudaSuccess) {
@@ -464,6 +485,7 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
   }
   const SvdOut* douts = (const SvdOut*)up(outs.data(), outs.size() * sizeof(SvdOut));
   const Copy2D* dsc = (const Copy2D*)up(scatter.data(), scatter.size() * sizeof(Copy2D));
+  flush();
   CUDA_CHECK(tnx_launch_svd_extract(douts, (int)outs.size(), st));
   CUDA_CHECK(tnx_launch_copy2d(dsc, (int)scatter.size(), st));
   CUDA_CHECK(cudaStreamSynchronize(st));   // the staging buffers are released on return

@@ -180,6 +180,68 @@ Hist hist_conv(const Hist& a, const Hist& b, const SymInfo& sy) {
   return c;
 }
 
+// Histograms of U(1) charges on one integer key: a charge vector q has the key sum_c q_c
+// stride_c, with strides that keep the keys of all sums over a network's legs apart,
+// so that keys add like charges.  Not for Z_n (ok false), nor when the keys would not
+// fit 62 bits.
+typedef std::vector<std::pair<int64_t, double>> FlatHist;   // ascending keys
+
+struct FlatSpace {
+  bool ok = true;
+  std::vector<int64_t> stride;
+
+  FlatSpace(const SymInfo& sy, const std::vector<std::string>& labs,
+            std::map<std::string, std::vector<std::pair<int, const BondD*>>>& occ) {
+    const size_t nsym = sy.kinds.size();
+    stride.resize(nsym);
+    double total = 1.0;
+    for (size_t c = 0; c < nsym; ++c) {
+      if (sy.kinds[c] == TNX_ZN) ok = false;
+      int64_t reach = 0;   // no sum over the legs goes beyond it
+      for (const std::string& l : labs) {
+        int64_t most = 0;
+        for (auto& o : occ[l])
+          for (int s = 0; s < o.second->nsec; ++s)
+            most = std::max<int64_t>(most, std::abs((int64_t)o.second->signed_q(s, (int)c)));
+        reach += most;
+      }
+      stride[c] = (int64_t)total;
+      total *= 2.0 * (double)reach + 1.0;
+      if (total > 4e18) {
+        ok = false;
+        return;
+      }
+    }
+  }
+  FlatHist leg(const BondD& b) const {
+    std::map<int64_t, double> h;
+    for (int s = 0; s < b.nsec; ++s) {
+      int64_t k = 0;
+      for (int c = 0; c < b.nsym; ++c) k += b.signed_q(s, c) * stride[c];
+      h[k] += (double)b.deg[s];
+    }
+    return FlatHist(h.begin(), h.end());
+  }
+  FlatHist conv(const FlatHist& a, const FlatHist& b) const {
+    FlatHist out;
+    if (a.empty() || b.empty()) return out;
+    const int64_t lo = a.front().first + b.front().first, hi = a.back().first + b.back().first;
+    if (hi - lo < (int64_t)1 << 22) {
+      std::vector<double> v((size_t)(hi - lo + 1), 0.0);
+      for (const auto& x : a)
+        for (const auto& y : b) v[(size_t)(x.first + y.first - lo)] += x.second * y.second;
+      for (int64_t k = lo; k <= hi; ++k)
+        if (v[(size_t)(k - lo)] != 0.0) out.push_back({k, v[(size_t)(k - lo)]});
+    } else {
+      std::map<int64_t, double> m;
+      for (const auto& x : a)
+        for (const auto& y : b) m[x.first + y.first] += x.second * y.second;
+      out.assign(m.begin(), m.end());
+    }
+    return out;
+  }
+};
+
 Hist leg_hist(const BondD& b) {
   Hist h;
   for (int s = 0; s < b.nsec; ++s) {
@@ -229,19 +291,59 @@ void sparse_optimal_tree(tnx_network* net) {
     fail(TNX_ERR_NETWORK, "internal: label outside its subset");
     return *occ[labs[l]][0].second;
   };
+  // the histogram of the legs ls as they appear inside subset m, kept by the bonds
+  // they are (a leg belongs to one or two tensors, so few sets differ)
   const Hist unit = {{std::vector<int32_t>(nsym, 0), 1.0}};
-  auto hist_of = [&](const std::vector<int>& ls, uint32_t m) {
+  std::map<std::vector<const BondD*>, Hist> kept;
+  std::map<std::vector<const BondD*>, FlatHist> kept_flat;
+  const FlatSpace space(sy, labs, occ);
+  auto bonds_of = [&](const std::vector<int>& ls, uint32_t m) {
+    std::vector<const BondD*> bs;
+    for (int l : ls) bs.push_back(&bond_in(l, m));
+    return bs;
+  };
+  auto hist_of = [&](const std::vector<int>& ls, uint32_t m) -> const Hist& {
+    const std::vector<const BondD*> bs = bonds_of(ls, m);
+    auto it = kept.find(bs);
+    if (it != kept.end()) return it->second;
     Hist h = unit;
-    for (int l : ls) h = hist_conv(h, leg_hist(bond_in(l, m)), sy);
-    return h;
+    for (const BondD* x : bs) h = hist_conv(h, leg_hist(*x), sy);
+    return kept.emplace(bs, std::move(h)).first->second;
+  };
+  auto flat_of = [&](const std::vector<int>& ls, uint32_t m) -> const FlatHist& {
+    std::vector<const BondD*> bs = bonds_of(ls, m);
+    auto it = kept_flat.find(bs);
+    if (it != kept_flat.end()) return it->second;
+    // one leg more than the histogram of the others
+    FlatHist h{{0, 1.0}};
+    std::vector<const BondD*> head;
+    for (const BondD* x : bs) {
+      head.push_back(x);
+      auto jt = kept_flat.find(head);
+      if (jt == kept_flat.end()) jt = kept_flat.emplace(head, space.conv(h, space.leg(*x))).first;
+      h = jt->second;
+    }
+    return kept_flat.emplace(bs, std::move(h)).first->second;
   };
   auto pair_cost = [&](uint32_t a, uint32_t b) {
     std::vector<int> fa, fb, k;
     for (int l : open[a]) (std::find(open[b].begin(), open[b].end(), l) != open[b].end() ? k : fa).push_back(l);
     for (int l : open[b])
       if (std::find(open[a].begin(), open[a].end(), l) == open[a].end()) fb.push_back(l);
-    const Hist ha = hist_of(fa, a), hk = hist_of(k, a), hb = hist_of(fb, b);
     double c = 0.0;
+    if (space.ok) {
+      const FlatHist &ha = flat_of(fa, a), &hk = flat_of(k, a), &hb = flat_of(fb, b);
+      // keys ascend: -g through ha from its end, g through hb from its start
+      size_t ia = ha.size(), ib = 0;
+      for (const auto& g : hk) {
+        while (ia > 0 && ha[ia - 1].first > -g.first) --ia;
+        while (ib < hb.size() && hb[ib].first < g.first) ++ib;
+        if (ia > 0 && ha[ia - 1].first == -g.first && ib < hb.size() && hb[ib].first == g.first)
+          c += 2.0 * ha[ia - 1].second * g.second * hb[ib].second;
+      }
+      return c;
+    }
+    const Hist &ha = hist_of(fa, a), &hk = hist_of(k, a), &hb = hist_of(fb, b);
     for (auto& g : hk) {
       auto ia = ha.find(sy.neg(g.first));
       auto ib = hb.find(g.first);
@@ -1674,6 +1776,7 @@ std::unique_ptr<Plan> build_plan(tnx_network* net, const std::string& key, const
     }
   }
   p->d_slots = (double**)p->alloc_zero(p->h_slots.size() * sizeof(double*));
+  p->flush();
   p->h_slots_dev.assign(p->h_slots.size(), nullptr);
   CUDA_CHECK(cudaStreamSynchronize(net->ctx->stream));
   return p;

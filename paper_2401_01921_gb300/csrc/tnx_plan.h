@@ -152,20 +152,58 @@ struct Plan {
     dry_next += (n + 255) & ~(size_t)255;
     return p;
   }
+  // Small buffers (tables, tile lists, exponents) share allocations of kArena bytes,
+  // filled through a host copy that goes over in one transfer each (flush, at the end
+  // of build_plan): a plan has about 60 of them, and an allocation through the caller's
+  // allocator and a transfer cost some 10 us each.
+  static constexpr size_t kArena = 256 * 1024, kSmall = 64 * 1024;
+  std::vector<char> stage;
+  char* arena = nullptr;
+  size_t arena_used = 0;
+  size_t small(size_t n) {   // offset of n zeroed bytes in the current arena
+    n = (n + 255) & ~(size_t)255;
+    if (!arena || arena_used + n > kArena) {
+      flush();
+      if (dry) {
+        arena = (char*)dry_take(kArena);
+      } else {
+        bufs.emplace_back(new DevBuf(ctx, kArena));
+        arena = (char*)bufs.back()->p;
+        stage.assign(kArena, 0);
+      }
+      arena_used = 0;
+    }
+    const size_t o = arena_used;
+    arena_used += n;
+    return o;
+  }
+  void flush() {
+    if (arena && !dry && arena_used)
+      CUDA_CHECK(cudaMemcpyAsync(arena, stage.data(), arena_used, cudaMemcpyHostToDevice, ctx->stream));
+    arena = nullptr;
+    arena_used = 0;
+  }
   template <class T>
   T* upload(const std::vector<T>& v) {
     size_t n = std::max<size_t>(v.size(), 1) * sizeof(T);
+    if (n <= kSmall) {
+      const size_t o = small(n);
+      if (!dry && !v.empty()) memcpy(stage.data() + o, v.data(), v.size() * sizeof(T));
+      return (T*)(arena + o);
+    }
     if (dry) return (T*)dry_take(n);
     bufs.emplace_back(new DevBuf(ctx, n));
-    if (!v.empty()) CUDA_CHECK(cudaMemcpyAsync(bufs.back()->p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, ctx->stream));
+    CUDA_CHECK(cudaMemcpyAsync(bufs.back()->p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, ctx->stream));
     return (T*)bufs.back()->p;
   }
   void* alloc_zero(size_t bytes) {
-    if (dry) return dry_take(std::max<size_t>(bytes, 256));
-    bufs.emplace_back(new DevBuf(ctx, std::max<size_t>(bytes, 256)));
-    CUDA_CHECK(cudaMemsetAsync(bufs.back()->p, 0, std::max<size_t>(bytes, 256), ctx->stream));
+    if (bytes <= kSmall) return arena_at(small(std::max<size_t>(bytes, 256)));
+    if (dry) return dry_take(bytes);
+    bufs.emplace_back(new DevBuf(ctx, bytes));
+    CUDA_CHECK(cudaMemsetAsync(bufs.back()->p, 0, bytes, ctx->stream));
     return bufs.back()->p;
   }
+  void* arena_at(size_t o) { return arena + o; }
   std::vector<int64_t> slot_elems;   // size of each slot's buffer, in doubles
   int new_slot(void* p, int64_t elems) {
     h_slots.push_back((double*)p);

@@ -22,7 +22,9 @@ def test_columns_of_different_scale(ctx, m, k, n, prec):  # noqa: F811
     got = _product(ctx, A, B, prec)
     # operands balanced by the exponent of A's column maxima, each entry then rounded 41 bits below
     # its row's (column's) largest, levels below 2^-42 dropped: 2^-38 leaves a factor of four
-    e = np.floor(np.log2(np.max(np.abs(A), axis=0)))
+    # (a column of A without a nonzero entry is not shifted)
+    top = np.max(np.abs(A), axis=0)
+    e = np.floor(np.log2(np.where(top > 0, top, 1.0)))
     row = np.max(np.abs(A * 2.0 ** -e), axis=1)
     col = np.max(np.abs(B * 2.0 ** e[:, None]), axis=0)
     assert np.all(np.abs(got - A @ B) <= 2.0 ** -38 * k * np.outer(row, col))
