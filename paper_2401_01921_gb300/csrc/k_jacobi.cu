@@ -45,9 +45,12 @@
 // CTA runs its slots round by round, so with all CTAs resident (a cooperative
 // launch) each wait ends; all are bounded (about a second of clock) all the
 // same, and on expiry *status is set and every CTA leaves.
+#include "tnx_fp64.cuh"
 #include "tnx_internal.h"
 
 namespace {
+
+using namespace tnx_fp64;
 
 constexpr long long JB_WAIT_LIMIT = 2000000000LL;   // clock cycles
 constexpr int W = 8;                                // warps that rotate: vectors per column block at most
@@ -90,23 +93,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// ---- a double's parts, on the integer units
-__device__ __forceinline__ int expo(int hi) { return (hi >> 20) & 0x7FF; }   // biased exponent
-__device__ __forceinline__ float mant(double x) {                             // |mantissa| in [1, 2), 23 bits
-  return __int_as_float(0x3F800000 | ((__double2hiint(x) & 0xFFFFF) << 3) |
-                        (int)((unsigned)__double2loint(x) >> 29));
-}
-
-// x * 2^k rounded to an integer (0 when x is zero or subnormal or the result is
-// below 1/2 or, for an x that is not finite, above 2^62).
-__device__ __forceinline__ long long scaled_int(double x, int k) {
-  const int hi = __double2hiint(x), e = expo(hi) - 1023 + k;   // |x| 2^k in [2^e, 2^(e+1))
-  if (expo(hi) == 0 || e < -1 || e > 61) return 0;
-  const long long m = ((long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)__double2loint(x);   // 53 bits
-  const long long v = e >= 52 ? m << (e - 52) : ((m >> (51 - e)) + 1) >> 1;
-  return hi < 0 ? -v : v;
-}
-
 // Named barriers: dot products done (rotating warps arrive, angle warps wait),
 // coefficients ready (angle warps 0 and 1 arrive, rotating warps wait), rotating warps
 // among themselves, angle warps among themselves.
@@ -118,14 +104,6 @@ __device__ __forceinline__ void bar_sync(int id, int n) {
 __device__ __forceinline__ void bar_arrive(int id, int n) {
   __syncwarp();
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-
-// Sum over the warp of |v| <= 2^60 in total: limbs of 21, 21 and 20 bits.
-__device__ __forceinline__ long long warp_sum_int(long long v) {
-  const int lo = __reduce_add_sync(0xffffffffu, (int)(v & 0x1FFFFF));
-  const int mid = __reduce_add_sync(0xffffffffu, (int)((v >> 21) & 0x1FFFFF));
-  const int hi = __reduce_add_sync(0xffffffffu, (int)(v >> 42));
-  return ((long long)hi << 42) + ((long long)mid << 21) + lo;
 }
 
 __device__ __forceinline__ bool usable(double n) {   // positive, normal and finite
@@ -201,13 +179,6 @@ __device__ __forceinline__ float norm_left(const Tan& t, const Rough& g, double 
   const float q = mant(a) * r0 * pow2f(expo(__double2hiint(a)) - 1023 - e0);
   const float tg = t.t * g.m * r0 * pow2f(g.e - t.sh - e0);
   return q - ((t.s ^ g.s) < 0 ? -s : s) * tg;
-}
-
-// x * 2^-k for a normal or zero x (0 when the result is not normal)
-__device__ __forceinline__ double shift_down(double x, int k) {
-  const int hi = __double2hiint(x), e = expo(hi) - k;
-  if (expo(hi) == 0 || e <= 0 || e >= 2047) return 0.0;
-  return __hiloint2double((hi & 0x800FFFFF) | (e << 20), __double2loint(x));
 }
 
 // Local vector l < wm lies in the first column block of the slot, l >= wm in the
@@ -386,11 +357,8 @@ __global__ void __launch_bounds__(JB_THREADS) jacobi_block_kernel(const JbGroup*
               g1 = fma(xa[e + 32], xb[e + 32], g1);
             }
             if (e < ldp) g0 = fma(xa[e], xb[e], g0);
-            g0 += g1;
-            // the largest partial sum lies below 2^(top - 1022): 32 of them, in units of 2^-k, below 2^60
-            const int top = __reduce_max_sync(0xffffffffu, expo(__double2hiint(g0)));
-            const int k2 = 55 - (top - 1022);
-            const long long v = warp_sum_int(scaled_int(g0, k2));
+            int k2;
+            const long long v = warp_sum_scaled(g0 + g1, k2);
             if (lane == 0) {
               S.dot[s & 1][wid] = v;
               S.sc[s & 1][wid] = k2;

@@ -24,12 +24,15 @@
 //    x_p / sigma_p on one side and the rows of J on the other.
 // Blocks of 16 or more vectors go through a column-pivoted Householder QR
 // first and the sweeps run on the rows of its triangular factor (see the QR
-// preconditioning section below), the sweeps there by the kernel of k_jacobi.cu
-// (jacobi_coop_kernel when a block is too long for it); the output has the same form.
+// preconditioning section below), done by the kernels of k_qr.cu and k_jacobi.cu
+// (qr_coop_kernel, jacobi_coop_kernel when a block is too long for them); the output has the same form.
 // All arithmetic is FP64.  Block reductions use a fixed order (deterministic).
+#include "tnx_fp64.cuh"
 #include "tnx_internal.h"
 
 namespace {
+
+using tnx_fp64::warp_sum_double;
 
 constexpr int JT = 256;   // threads per pair
 
@@ -370,7 +373,10 @@ __device__ void reflector_store(const SvdQr& q, int k, int u, int lane) {
   reflector(x, len, lane, beta, tau, scale);
   __syncwarp();   // every lane has read x[0] before lane 0 replaces it
   for (int i = lane; i < len; i += 32) x[i] = i == 0 ? beta : x[i] * scale;
-  if (lane == 0) q.tau[k] = tau;
+  if (lane == 0) {
+    q.tau[k] = tau;
+    q.u0[k] = 1.0;
+  }
 }
 
 // The pivoted QR of every block: a slot is (block, position j); step k runs
@@ -506,27 +512,35 @@ __global__ void qr_apply_kernel(const SvdQr* __restrict__ qs, const int2* __rest
     double* xf = q.Xf + (int64_t)p * r;
     if (r <= 32 * VB) {
       double z[VB];
+      const int nm = (r + 31) / 32;   // 32-entry chunks
 #pragma unroll
       for (int m = 0; m < VB; ++m) {
         const int e = lane + 32 * m;
         z[m] = e < c ? jr[e] * dp : 0.0;
       }
-      for (int k = c - 1; k >= 0; --k) {
-        const double tk = q.tau[k];
-        if (tk == 0.0) continue;
-        const double* v = q.X + (int64_t)q.perm[k] * r;   // v_e for e > k; v_k = 1
-        double vv[VB];
-        double w = 0.0;
+      // the reflector of position k has nothing before chunk k / 32: no FP64 work there
 #pragma unroll
-        for (int m = 0; m < VB; ++m) {
-          const int e = lane + 32 * m;
-          vv[m] = e == k ? 1.0 : (e > k && e < r ? v[e] : 0.0);
-          w = fma(vv[m], z[m], w);
+      for (int kb = VB - 1; kb >= 0; --kb) {
+        for (int k = min(c - 1, 32 * kb + 31); k >= 32 * kb; --k) {
+          const double tk = q.tau[k];
+          if (tk == 0.0) continue;
+          const double* v = q.X + (int64_t)q.perm[k] * r;   // u_e for e > k
+          const double u0 = q.u0[k];
+          double vv[VB];
+          double w = 0.0;
+#pragma unroll
+          for (int m = kb; m < VB; ++m) {
+            const int e = lane + 32 * m;
+            if (m < nm) vv[m] = e == k ? u0 : (e > k && e < r ? v[e] : 0.0);
+          }
+#pragma unroll
+          for (int m = kb; m < VB; ++m)
+            if (m < nm) w = fma(vv[m], z[m], w);
+          const double tw = tk * warp_sum_double(w);
+#pragma unroll
+          for (int m = kb; m < VB; ++m)
+            if (m < nm) z[m] = fma(-tw, vv[m], z[m]);
         }
-        w = warp_sum(w);
-        const double tw = tk * w;
-#pragma unroll
-        for (int m = 0; m < VB; ++m) z[m] = fma(-tw, vv[m], z[m]);
       }
 #pragma unroll
       for (int m = 0; m < VB; ++m) {
@@ -539,13 +553,14 @@ __global__ void qr_apply_kernel(const SvdQr* __restrict__ qs, const int2* __rest
         const double tk = q.tau[k];
         if (tk == 0.0) continue;
         const double* v = q.X + (int64_t)q.perm[k] * r;
+        const double u0 = q.u0[k];
         double w = 0.0;
         for (int e = lane; e < r; e += 32)
-          if (e >= k) w = fma(e == k ? 1.0 : v[e], xf[e], w);
+          if (e >= k) w = fma(e == k ? u0 : v[e], xf[e], w);
         w = warp_sum(w);
         const double tw = tk * w;
         for (int e = lane; e < r; e += 32)
-          if (e >= k) xf[e] = fma(-tw, e == k ? 1.0 : v[e], xf[e]);
+          if (e >= k) xf[e] = fma(-tw, e == k ? u0 : v[e], xf[e]);
       }
       for (int e = lane; e < r; e += 32) xf[e] *= sg;
     }

@@ -334,7 +334,8 @@ struct Copy2D {
 // vectors of A) and J the right singular vectors of A as rows.
 struct SvdQr {
   double* X;        // c x r
-  double* tau;      // [c] reflector scalar of pivot position k
+  double* tau;      // [c] reflector scalar of pivot position k: H = I - tau u u^T,
+  double* u0;       // [c] u = (u0, X[perm[k]][k+1], ...)
   int32_t* perm;    // [c] vector at pivot position k
   double* nrm;      // [2][c] squared norms of the trailing parts, by position
   int32_t* pos;     // [2][c] vector at each position
@@ -375,6 +376,22 @@ cudaError_t tnx_launch_jacobi_init(const SvdGroup* groups, int ngroups, cudaStre
 // without cooperative launch
 cudaError_t tnx_launch_qr_coop(const SvdQr* qs, const int2* slots, int nslots, int maxc, unsigned long long* bar,
                                int* status, cudaStream_t st);
+// The same on columns held in shared memory (k_qr.cu): slots (block, slot s) hold
+// columns 8 s .. 8 s + 7 of a block, ns = ceil(c / 8) slots per block, all resident at
+// once (else cudaErrorNotSupported, before anything has run).
+struct QrOffer {
+  double nrm, beta, u0, kappa;
+  int32_t idx, pad0;
+};
+struct QbGroup {
+  QrOffer* offers;    // [2][ns]
+  double* columns;    // [2][ns][r rounded up to 32]
+  unsigned* count;    // zeroed by the caller
+  int32_t ns, pad0;
+};
+int tnx_qr_block_columns(int maxr);   // columns per slot (8), 0: too long for shared memory
+cudaError_t tnx_launch_qr_block(const SvdQr* qs, const QbGroup* groups, const int2* slots, int nslots, int maxr,
+                                int* status, cudaStream_t st);
 // Xr = R (rows, zero below the diagonal) and Jr = identity for every block
 cudaError_t tnx_launch_qr_gather_r(const SvdQr* qs, int nq, int maxc, cudaStream_t st);
 // after the Jacobi on Xr: sigma, J and Xf for every (block, vector)

@@ -209,7 +209,7 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
   }
   std::unique_ptr<DevBuf> QD, QI, QXf;
   if (!done && maxc >= 16) {
-    QD.reset(new DevBuf(ctx, (size_t)(7 * nC + 2 * nC2) * 8));   // tau, nrm[2], D[4], Xr, Jr
+    QD.reset(new DevBuf(ctx, (size_t)(8 * nC + 2 * nC2) * 8));   // tau, nrm[2], D[4], u0, Xr, Jr
     QI.reset(new DevBuf(ctx, (size_t)(3 * nC) * 4));             // perm, pos[2]
     QXf.reset(new DevBuf(ctx, (size_t)std::max<int64_t>(nCR, 1) * 8));
     std::vector<SvdQr> hq(ngr);
@@ -224,8 +224,9 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
       q.tau = (double*)QD->p + oc;
       q.nrm = (double*)QD->p + nC + 2 * oc;
       q.D = (double*)QD->p + 3 * nC + 4 * oc;
-      q.Xr = (double*)QD->p + 7 * nC + oc2;
-      q.Jr = (double*)QD->p + 7 * nC + nC2 + oc2;
+      q.u0 = (double*)QD->p + 7 * nC + oc;
+      q.Xr = (double*)QD->p + 8 * nC + oc2;
+      q.Jr = (double*)QD->p + 8 * nC + nC2 + oc2;
       q.perm = (int32_t*)QI->p + oc;
       q.pos = (int32_t*)QI->p + nC + 2 * oc;
       q.Xf = (double*)QXf->p + ocr;
@@ -272,8 +273,46 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
     unsigned long long* w = (unsigned long long*)up(zero.data(), zero.size() * 8);
     int* qstat = (int*)(w + 1);
     int* jstat = (int*)(w + MAX_SWEEPS + 3);
-    flush();
-    const cudaError_t ce = tnx_launch_qr_coop(dq, dqs, (int)qslots.size(), maxc, w, qstat, st);
+    // the QR on columns in shared memory (k_qr.cu) where its slots fit; else step by
+    // step through L2
+    cudaError_t ce = cudaErrorNotSupported;
+    std::unique_ptr<DevBuf> QB;
+    const int qcols = tnx_qr_block_columns(maxr);
+    if (qcols) {
+      std::vector<QbGroup> hb(ngr);
+      std::vector<int2> bslots;
+      size_t bytes = 0;
+      std::vector<size_t> at(ngr);
+      for (int i = 0; i < ngr; ++i) {
+        const size_t ns = (hq[i].c + qcols - 1) / qcols, rp = ((size_t)hq[i].r + 31) / 32 * 32;
+        hb[i].ns = (int32_t)ns;
+        at[i] = bytes;
+        bytes += 2 * ns * (rp * sizeof(double) + sizeof(QrOffer));
+        bytes = (bytes + 255) & ~(size_t)255;
+        for (size_t s = 0; s < ns; ++s) bslots.push_back(make_int2(i, (int)s));
+      }
+      // the longest factorisations first
+      std::stable_sort(bslots.begin(), bslots.end(), [&](const int2& a, const int2& b) { return hq[a.x].c > hq[b.x].c; });
+      QB.reset(new DevBuf(ctx, std::max<size_t>(bytes, 256)));
+      std::vector<uint32_t> cz(ngr, 0);
+      unsigned* counts = (unsigned*)up(cz.data(), cz.size() * 4);
+      for (int i = 0; i < ngr; ++i) {
+        const size_t rp = ((size_t)hq[i].r + 31) / 32 * 32;
+        hb[i].columns = (double*)((char*)QB->p + at[i]);
+        hb[i].offers = (QrOffer*)(hb[i].columns + 2 * (size_t)hb[i].ns * rp);
+        hb[i].count = counts + i;
+        hb[i].pad0 = 0;
+      }
+      const QbGroup* db = (const QbGroup*)up(hb.data(), hb.size() * sizeof(QbGroup));
+      const int2* dbs = (const int2*)up(bslots.data(), bslots.size() * sizeof(int2));
+      flush();
+      ce = tnx_launch_qr_block(dq, db, dbs, (int)bslots.size(), maxr, qstat, st);
+    }
+    if (ce == cudaErrorNotSupported) {
+      (void)cudaGetLastError();
+      flush();
+      ce = tnx_launch_qr_coop(dq, dqs, (int)qslots.size(), maxc, w, qstat, st);
+    }
     if (ce == cudaSuccess) {
       CUDA_CHECK(tnx_launch_qr_gather_r(dq, ngr, maxc, st));
       // the sweeps run on R: vectors of c entries
