@@ -168,6 +168,20 @@ __device__ __forceinline__ double i64_scaled_fast(long long v, int e) {
   return i64_scaled_to_double(v, e);
 }
 
+// The same value and rounding on the integer units alone, |v| < 2^62: the leading one
+// goes to bit 62, the low 10 bits are rounded off to nearest-even, and a carry out of
+// the mantissa runs into the exponent.
+__device__ __forceinline__ double i64_scaled_alu(long long v, int e) {
+  const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
+  const int lz = __clzll((long long)u);
+  const int ex = 1086 - lz + e;   // biased exponent of the leading one
+  if (v != 0 && (unsigned)(ex - 1) >= 2045u) return i64_scaled_to_double(v, e);
+  const unsigned long long w = u << ((lz - 1) & 63);
+  const unsigned long long m = (w + 0x1FFull + ((w >> 10) & 1ull)) >> 10;   // 2^52 .. 2^53
+  const unsigned long long bits = ((unsigned long long)(unsigned)(ex - 1) << 52) + m;
+  return v != 0 ? __longlong_as_double((long long)(bits | ((unsigned long long)v & (1ull << 63)))) : 0.0;
+}
+
 // kind::tf32: D f32, A/B tf32 (format 2), both K-major, M = 128, N = n
 __device__ __forceinline__ uint32_t instr_desc_tf32(int n) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
@@ -653,7 +667,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) split_gemm_kernel(const Spli
           // A slice i meets the B slices j = 0 .. NS-1-i stacked along N (they are
           // consecutive TNV-row tiles, so the stack is one taller K-major operand);
           // its output columns are the accumulators of levels i .. NS-1, also
-          // consecutive: one MMA (N <= 256, else two) per A slice and K step.
+          // consecutive: one MMA (N <= 256, else two of half the stack) per A slice
+          // and K step.  Halves because an MMA reads 4 KB of A and 32 bytes per
+          // column of B while it computes for N / 2 cycles: below N = 128 it waits for
+          // shared memory (128 bytes per cycle), as a remainder of 64 columns did.
           // A K step is 32 bytes of every row: 16 values of BF16/FP16, 8 of TF32.
 #pragma unroll
           for (int ks = 0; ks < TK / 16; ++ks) {
@@ -661,14 +678,14 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) split_gemm_kernel(const Spli
             for (int i = 0; i < NS; ++i) {
               const uint64_t ad = smem_desc(sa + i * ATILE + ks * 256);
               const uint32_t acc = (first_in_chunk && ks == 0 && i == 0) ? 0u : 1u;
-              const int nj = NS - i;
-              constexpr int PER_MMA = 256 / TNV;   // B slices per MMA (N <= 256)
+              const int cols = (NS - i) * TNV;
+              const int n = cols <= 256 ? cols : cols / 2;
+              static_assert(TNV % 32 == 0 && NS * TNV <= 512, "half a stack is a multiple of 16 columns, at most 256");
 #pragma unroll
-              for (int j0 = 0; j0 < nj; j0 += PER_MMA) {
-                const int cnt = (nj - j0) < PER_MMA ? (nj - j0) : PER_MMA;
-                const uint64_t bd = smem_desc(sb + j0 * BTILE + ks * 256);
-                if constexpr (TF) mma_tf32(tmem + (uint32_t)((i + j0) * TNV), ad, bd, instr_desc_tf32(cnt * TNV), acc);
-                else mma_f16(tmem + (uint32_t)((i + j0) * TNV), ad, bd, instr_desc(f16, cnt * TNV), acc);
+              for (int c0 = 0; c0 < cols; c0 += n) {
+                const uint64_t bd = smem_desc(sb + c0 * (TK * 2) + ks * 256);
+                if constexpr (TF) mma_tf32(tmem + (uint32_t)(i * TNV + c0), ad, bd, instr_desc_tf32(n), acc);
+                else mma_f16(tmem + (uint32_t)(i * TNV + c0), ad, bd, instr_desc(f16, n), acc);
               }
             }
           }
@@ -699,6 +716,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) split_gemm_kernel(const Spli
       const int KT = (gr.K + TKE - 1) / TKE;
       const int nchunks = (KT + KTPC - 1) / KTPC;
       const int row = tl.m0 + sub * 32 + lane;
+      // This warp's part of the tile that exists: no columns when its rows don't.  Short
+      // contractions are bound by this epilogue, not by the tensor cores (about 10 against
+      // 9 thousand cycles a tile at bond dimension 2048), and small blocks leave most of a
+      // tile empty: with the skip, two conversion units and the even MMAs the products of a
+      // batch of 48 small sites went from 344 to 265 us, the two at 4096 from 570 to 545
+      // us (ncu, cold); a solve at 2048 from 6106 to 6034 us.
+      const int ncol = tl.m0 + sub * 32 < gr.M ? min(ECOLS, gr.N - tl.n0 - cb) : 0;
       // Row and column exponents are fetched before the first accumulator
       // wait, so their global-load latency hides behind the MMAs.
       double (*stg)[4] = sh_stage + (warp - 2) * 32;
@@ -725,6 +749,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) split_gemm_kernel(const Spli
         // all levels of 8 columns in flight at once, one wait per column group
 #pragma unroll
         for (int cg = 0; cg < ECOLS / 8; ++cg) {
+          if (cg * 8 >= ncol) break;
           uint32_t v[NS][8];
 #pragma unroll
           for (int t = 0; t < NS; ++t)
@@ -745,10 +770,14 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) split_gemm_kernel(const Spli
               const int lo = d[5] + d[4] * 128, mid = d[3] + d[2] * 128, hi = d[1] + d[0] * 128;   // |.| < 2^30
               acc[cg * 8 + c] += ((long long)hi << 28) + ((long long)mid << 14) + (long long)lo;
             } else {
-              long long x = 0;
+              // level 0 has one digit pair: |sum| <= 640 * 64^2 < 2^22, the exact add (above);
+              // the conversion instruction runs at a quarter of that rate
+              static_assert(KC * 64 * 64 < (1 << 22), "level 0 of a chunk");
+              long long x = (long long)(__float_as_int(__uint_as_float(v[0][c]) + 12582912.0f) - 0x4B400000) *
+                            (1LL << (7 * (NS - 1)));
 #pragma unroll
-              for (int t = 0; t < NS; ++t)
-                x += (long long)__float2int_rn(__uint_as_float(v[t][c])) * (1LL << (beta * (NS - 1 - t)));
+              for (int t = 1; t < NS; ++t)
+                x += (long long)__float2int_rn(__uint_as_float(v[t][c])) * (1LL << (7 * (NS - 1 - t)));
               acc[cg * 8 + c] += x;
             }
           }
@@ -772,6 +801,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) split_gemm_kernel(const Spli
         const int r0 = tl.m0 + sub * 32;
 #pragma unroll
         for (int c4 = 0; c4 < ECOLS / 4; ++c4) {
+          if (c4 * 4 >= ncol) break;
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             if constexpr (TF) {
@@ -779,7 +809,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) split_gemm_kernel(const Spli
               stg[lane][c ^ ((lane >> 2) & 3)] = ldexp(accd[c4 * 4 + c], eb_r + ebc_s[c4 * 4 + c] - 2046);
             } else {
               const int e = eb_r + ebc_s[c4 * 4 + c] - 2044 - 2 * (NS * beta - 1) + beta * (NS - 1);
-              stg[lane][c ^ ((lane >> 2) & 3)] = i64_scaled_fast(acc[c4 * 4 + c], e);
+              // a conversion takes the FP64 unit 64 cycles: half of them run on the
+              // integer units beside it
+              stg[lane][c ^ ((lane >> 2) & 3)] =
+                  c & 1 ? i64_scaled_alu(acc[c4 * 4 + c], e) : i64_scaled_fast(acc[c4 * 4 + c], e);
             }
           }
           __syncwarp();
