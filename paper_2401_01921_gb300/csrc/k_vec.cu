@@ -12,14 +12,16 @@
 // then Sturm bisection on the tridiagonal T and inverse iteration for its
 // eigenvector, and the Ritz vector V y.
 // Reductions are deterministic: per-block partial sums with a fixed grid and
-// a fixed-order tree (warp shuffles), then one block summing the partials in
-// a fixed order.
+// a fixed-order tree (warp shuffles), then the partials in a fixed order.
+#include <cooperative_groups.h>
+
 #include "tnx_internal.h"
 
 namespace {
 
 constexpr int RT = 256;        // threads per reduction block
 constexpr int RBLOCKS = 1216;  // 8 blocks per SM on 152 SMs
+constexpr int LT = 256;        // threads per CTA of a Lanczos step
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -41,11 +43,12 @@ __device__ double block_sum(double v, double* sh) {
 
 __device__ __forceinline__ bool stopped(const int32_t* state) { return *(volatile const int32_t*)(state + 1) != 0; }
 
-// A gated launch of the Gram-Schmidt pass does nothing unless this step's
-// decision asked for the pass.
-__device__ __forceinline__ bool gated_off(const int32_t* state, int gate) {
-  return gate && *(volatile const int32_t*)(state + 2) == 0;
+// The words that the CTAs of a Lanczos step wait on, one per 128 bytes: barrier
+// arrivals, norm arrivals, the decision (2 (j + 1), plus 1 with a pass).
+__device__ __forceinline__ unsigned long long* step_words(const LanczosDev& L) {
+  return (unsigned long long*)(L.state + 32);
 }
+constexpr int SW = 16;   // words apart: polls of one do not meet arrivals at another
 
 // Reductions finish in the launch that produces their partial sums: every
 // block publishes its partials, fences and counts itself in state[4]; the
@@ -114,6 +117,7 @@ __global__ void lanczos_init_kernel(LanczosDev L, const double* v0) {
     L.state[2] = 0;
     L.state[3] = 0;
     L.state[4] = 0;   // the last-block counter
+    for (int q = 0; q < 3; ++q) step_words(L)[q * SW] = 0;
     L.beta[0] = 0.0;
     L.omega[0] = 1.0;   // <v_0, v_0>; the row before it is empty
   }
@@ -122,138 +126,6 @@ __global__ void lanczos_init_kernel(LanczosDev L, const double* v0) {
 __global__ void set_slot_kernel(double** slot, double* p) {
   tnx_grid_dependency();
   *slot = p;
-}
-
-// partial[b*m + i] = <V_i, w> over this block's contiguous chunk, i < m.  A
-// grid of multidot_blocks(n) blocks keeps the number of partial sums (and so the
-// FP64 additions of the reduction tree) bounded; each thread keeps NG <= 16
-// running sums (NG fixed at compile time, so no FP64 instruction is issued for
-// a vector that does not exist), w is read once per group of vectors, and the
-// block reduction goes through shared memory: 16 rows of MD_T values, 8
-// threads per row.  FP64 issue slots are scarce on this part, so the grid is
-// only large enough to keep the loads in flight.
-constexpr int MD_T = 128;
-constexpr int MD_BLOCKS_MAX = 608;
-
-// Blocks of the multidot kernel: about 416 vector entries per block (an
-// L2-resident basis is bound by FP64 issue, where fewer partial sums help),
-// at least 1; above one per SM rounded to a multiple of the SM count, at most 4 per
-// SM (a basis in HBM needs the loads of that many blocks in flight).
-int multidot_blocks(int64_t n) {
-  int64_t b = n / 416;
-  if (b < 1) b = 1;
-  if (b > 152) b = (b + 151) / 152 * 152;
-  if (b > MD_BLOCKS_MAX) b = MD_BLOCKS_MAX;
-  return (int)b;
-}
-
-template <int NG>
-__device__ __forceinline__ void multidot_group(const LanczosDev& L, int g0, int64_t c0, int64_t c1,
-                                               double (*sh)[MD_T + 1]) {
-  // g0 is the basis row of the group's first vector
-  double acc[NG];
-#pragma unroll
-  for (int i = 0; i < NG; ++i) acc[i] = 0.0;
-  // two entries per iteration: both rows' loads are in flight before the FMAs
-  int64_t x = c0 + threadIdx.x;
-  for (; x + MD_T < c1; x += 2 * MD_T) {
-    const double w0 = L.w[x], w1 = L.w[x + MD_T];
-    double v0[NG], v1[NG];
-#pragma unroll
-    for (int i = 0; i < NG; ++i) {
-      v0[i] = L.V[(int64_t)(g0 + i) * L.n + x];
-      v1[i] = L.V[(int64_t)(g0 + i) * L.n + x + MD_T];
-    }
-#pragma unroll
-    for (int i = 0; i < NG; ++i) acc[i] = fma(v1[i], w1, fma(v0[i], w0, acc[i]));
-  }
-  if (x < c1) {
-    const double wx = L.w[x];
-#pragma unroll
-    for (int i = 0; i < NG; ++i) acc[i] = fma(L.V[(int64_t)(g0 + i) * L.n + x], wx, acc[i]);
-  }
-#pragma unroll
-  for (int i = 0; i < NG; ++i) sh[i][threadIdx.x] = acc[i];
-}
-
-// Dots of this block's chunk [c0, c1) against V_vb .. V_{vb+m-1} into partial[b*m + i].
-__device__ void block_multidot(const LanczosDev& L, int m, int64_t c0, int64_t c1, double (*sh)[MD_T + 1],
-                               int vb = 0) {
-  for (int g0 = 0; g0 < m; g0 += 16) {
-    const int ng = m - g0 < 16 ? m - g0 : 16;
-    const int r0 = vb + g0;
-    switch (ng) {
-      case 1: multidot_group<1>(L, r0, c0, c1, sh); break;
-      case 2: multidot_group<2>(L, r0, c0, c1, sh); break;
-      case 3: multidot_group<3>(L, r0, c0, c1, sh); break;
-      case 4: multidot_group<4>(L, r0, c0, c1, sh); break;
-      case 5: multidot_group<5>(L, r0, c0, c1, sh); break;
-      case 6: multidot_group<6>(L, r0, c0, c1, sh); break;
-      case 7: multidot_group<7>(L, r0, c0, c1, sh); break;
-      case 8: multidot_group<8>(L, r0, c0, c1, sh); break;
-      case 9: multidot_group<9>(L, r0, c0, c1, sh); break;
-      case 10: multidot_group<10>(L, r0, c0, c1, sh); break;
-      case 11: multidot_group<11>(L, r0, c0, c1, sh); break;
-      case 12: multidot_group<12>(L, r0, c0, c1, sh); break;
-      case 13: multidot_group<13>(L, r0, c0, c1, sh); break;
-      case 14: multidot_group<14>(L, r0, c0, c1, sh); break;
-      case 15: multidot_group<15>(L, r0, c0, c1, sh); break;
-      default: multidot_group<16>(L, r0, c0, c1, sh); break;
-    }
-    if (ng == 1) {   // a single vector: warp sums (the row sums below would chain 16 additions)
-      const double v = warp_sum(sh[0][threadIdx.x]);
-      __syncthreads();
-      if ((threadIdx.x & 31) == 0) sh[0][threadIdx.x >> 5] = v;
-      __syncthreads();
-      if (threadIdx.x == 0)
-        L.partial[(int64_t)blockIdx.x * m + g0] = (sh[0][0] + sh[0][1]) + (sh[0][2] + sh[0][3]);
-      __syncthreads();
-      continue;
-    }
-    __syncthreads();
-    // thread t sums 16 consecutive entries of row t/8, then 8 partners combine
-    const int row = threadIdx.x >> 3, part = threadIdx.x & 7;
-    if (row < ng) {
-      double v = 0.0;
-#pragma unroll
-      for (int q = 0; q < MD_T / 8; ++q) v += sh[row][part * (MD_T / 8) + q];
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffu << (threadIdx.x & 24), v, o, 8);
-      if (part == 0) L.partial[(int64_t)blockIdx.x * m + g0 + row] = v;
-    }
-    __syncthreads();
-  }
-}
-
-// coef[i] = sum_b partial[b*m + i] over the nb blocks of the launch (fixed
-// order); the sum of row alpha_i (if >= 0) is also alpha_j = <v_j, H v_j>.
-// Run by one block of any width.
-__device__ void finalize_coefs(const LanczosDev& L, int m, int nb, int alpha_i, int alpha_j, double* sh) {
-  for (int i = 0; i < m; ++i) {
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) acc += __ldcg(L.partial + (int64_t)b * m + i);
-    acc = nb > 32 ? block_sum(acc, sh) : warp_sum(acc);   // up to 32 partials lie in one warp
-    if (threadIdx.x == 0) {
-      L.coef[i] = acc;
-      if (i == alpha_i) L.alpha[alpha_j] = acc;
-    }
-  }
-}
-
-// Dots of w against V_vb .. V_{vb+m-1}, the coefficients formed by the last block.
-__global__ void __launch_bounds__(MD_T) multidot_kernel(LanczosDev L, int m, int vb, int gate, int alpha_i,
-                                                        int alpha_j) {
-  tnx_grid_dependency();
-  __shared__ double sh[16][MD_T + 1];
-  __shared__ double shr[32];
-  if (stopped(L.state) || gated_off(L.state, gate)) return;
-  const int64_t chunk = (L.n + gridDim.x - 1) / gridDim.x;
-  const int64_t c0 = chunk * blockIdx.x, c1 = min(L.n, c0 + chunk);
-  block_multidot(L, m, c0, c1, sh, vb);
-  if (last_block(L.state + 4)) {
-    finalize_coefs(L, m, gridDim.x, alpha_i, alpha_j, shr);
-    if (threadIdx.x == 0) L.state[4] = 0;
-  }
 }
 
 // beta_{j+1} = sqrt(sum of the nb norm partials); decide stop; record k; point
@@ -283,53 +155,6 @@ __device__ void beta_decide(const LanczosDev& L, int j, int nb, int last, double
   }
 }
 
-// w -= sum_i coef[i] V_i; with norm != 0 also partial[b] = sum of the new w^2
-// over this block's grid-stride share (fixed order).
-__global__ void __launch_bounds__(RT) gs_update_kernel(LanczosDev L, int m, int norm, int gate, int j, int last,
-                                                        double** next_slot) {
-  tnx_grid_dependency();
-  __shared__ double c[512];
-  __shared__ double sh[32];
-  if (stopped(L.state) || gated_off(L.state, gate)) return;
-  for (int i = threadIdx.x; i < m; i += RT) c[i] = L.coef[i];
-  __syncthreads();
-  double nrm = 0.0;
-  // two entries per iteration (the second one stride later), so that the loads
-  // of both are in flight together; each entry keeps its own subtraction order
-  const int64_t stride = (int64_t)gridDim.x * RT;
-  int64_t x = (int64_t)blockIdx.x * RT + threadIdx.x;
-  for (; x + stride < L.n; x += 2 * stride) {
-    double w0 = L.w[x], w1 = L.w[x + stride];
-#pragma unroll 4
-    for (int i = 0; i < m; ++i) {
-      const double* vi = L.V + (int64_t)i * L.n;
-      const double a0 = vi[x], a1 = vi[x + stride];
-      w0 -= c[i] * a0;
-      w1 -= c[i] * a1;
-    }
-    L.w[x] = w0;
-    L.w[x + stride] = w1;
-    nrm = fma(w0, w0, nrm);
-    nrm = fma(w1, w1, nrm);
-  }
-  if (x < L.n) {
-    double w = L.w[x];
-#pragma unroll 8
-    for (int i = 0; i < m; ++i) w -= c[i] * L.V[(int64_t)i * L.n + x];
-    L.w[x] = w;
-    nrm = fma(w, w, nrm);
-  }
-  if (norm) {
-    nrm = block_sum(nrm, sh);
-    if (threadIdx.x == 0) L.partial[blockIdx.x] = nrm;
-    // the last block: beta_{j+1} and the stopping test of this step
-    if (last_block(L.state + 4)) {
-      beta_decide(L, j, gridDim.x, last, next_slot);
-      if (threadIdx.x == 0) L.state[4] = 0;
-    }
-  }
-}
-
 // Partial reorthogonalisation (Simon, Math. Comp. 42, 1984): omega_{j,k}
 // estimates <v_j, v_k> through the recurrence that the Lanczos relation gives,
 //   beta_{j+1} omega_{j+1,k} = beta_{k+1} omega_{j,k+1} + (alpha_k - alpha_j) omega_{j,k}
@@ -339,18 +164,17 @@ __global__ void __launch_bounds__(RT) gs_update_kernel(LanczosDev L, int m, int 
 // eps1 |T| / beta_{j+1}.  After the three-term step this kernel forms
 // beta_{j+1} = |w| and the estimates of row j+1; the step takes a full
 // Gram-Schmidt pass against v_0..v_j when the largest estimate exceeds
-// tau (1e-10; a negative tau: every step), and so does the step after it (the error that v_j carries reaches
-// v_{j+2} too); after a pass the estimates restart at eps1.  Without a pass
-// it also does what beta_decide does (beta_{j+1}, the stopping
-// test, the next input slot); with one, the gated launches after it do.
+// tau (1e-10; a negative tau: every step), and so does the step after it (the error
+// that v_j carries reaches v_{j+2} too); after a pass the estimates restart at eps1.
+// Without a pass it also does what beta_decide does (beta_{j+1}, the stopping test, the
+// next input slot); with one, the pass does.
 constexpr int PRO_MAX = 514;   // rows of at most 500 steps + 2
 
 // What a step waits for here is FP64 latency: an FP64 instruction takes its SM
 // quarter 64 cycles however few lanes need it (a root ten of them, a division
 // nine), so roots and divisions are taken once, by one warp, maxima of
 // non-negative numbers are formed on their bit patterns, and eps1 comes from the
-// host.  Dense bond dimension 32 (4096 entries): the three-term launch 11.4 -> 9.0 us
-// (ncu, cold caches).
+// host.
 __device__ __forceinline__ unsigned long long bits_abs(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
 }
@@ -360,70 +184,78 @@ __device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
   return v;
 }
 
-// max(|alpha_i|, beta_i) and max(|alpha_i| + beta_i + beta_{i+1}) over i <= j (beta_{j+1}
-// left out), as bit patterns; one warp.
-__device__ __forceinline__ void tridiag_scale(const LanczosDev& L, int j, int lane, unsigned long long& amax,
-                                              unsigned long long& an) {
+// T and the estimates of rows j and j-1 in shared memory, read at the start of a step.
+struct ProRows {
+  double *al, *be, *om, *omp;   // alpha_k (k < j), beta_k (k <= j), omega_{j,k} (k <= j), omega_{j-1,k} (k < j)
+};
+__device__ __forceinline__ void pro_load(const LanczosDev& L, int j, const ProRows& r) {
+  for (int k = threadIdx.x; k <= j; k += LT) {
+    r.be[k] = L.beta[k];
+    r.om[k] = L.omega[k];
+    if (k < j) {
+      r.al[k] = L.alpha[k];
+      r.omp[k] = L.omega[L.nmax + 2 + k];
+    }
+  }
+}
+
+// max(|alpha_i|, beta_i) and max(|alpha_i| + beta_i + beta_{i+1}) over i <= j (alpha_j
+// given, beta_{j+1} left out), as bit patterns; one warp.
+__device__ __forceinline__ void tridiag_scale(const ProRows& r, int j, int lane, double aj,
+                                              unsigned long long& amax, unsigned long long& an) {
   amax = an = 0;
   for (int i = lane; i <= j; i += 32) {
-    const double a = fabs(L.alpha[i]), b = L.beta[i];
+    const double a = fabs(i < j ? r.al[i] : aj), b = r.be[i];
     amax = max(amax, max(bits_abs(a), bits_abs(b)));
-    an = max(an, bits_abs(a + b + (i < j ? L.beta[i + 1] : 0.0)));
+    an = max(an, bits_abs(a + b + (i < j ? r.be[i + 1] : 0.0)));
   }
   amax = warp_max(amax);
   an = warp_max(an);
 }
 
-// Sum of the nb partials, in a fixed order; valid in thread 0.
-__device__ double partial_sum(const double* partial, int nb, double* sh) {
-  double acc = 0.0;
-  for (int b = threadIdx.x; b < nb; b += RT) acc += __ldcg(partial + b);
-  if (nb > 32) return block_sum(acc, sh);   // else the other warps hold zeros
-  return warp_sum(acc);
+// Before the norm is known: the part of each estimate that does not need it, into
+// om_t[0 .. j), and the scales of T.  One block; `a` is alpha_j.
+struct ProScales {
+  unsigned long long amax, an;   // of tridiag_scale
+};
+__device__ void pro_prepare(const ProRows& r, int j, double a, double* om_t, ProScales* sc) {
+  if ((int)threadIdx.x < 32) {
+    unsigned long long amax, an;
+    tridiag_scale(r, j, threadIdx.x, a, amax, an);
+    if (threadIdx.x == 0) *sc = {amax, an};
+  }
+  const double bj = j > 0 ? r.be[j] : 0.0;
+  for (int k = threadIdx.x; k < j; k += LT) {
+    double t = r.be[k + 1] * r.om[k + 1] + (r.al[k] - a) * r.om[k] - bj * r.omp[k];
+    if (k > 0) t += r.be[k] * r.om[k - 1];
+    om_t[k] = t;
+  }
 }
 
-// Run by one block of RT threads over the nb norm partials.
-__device__ void pro_decide(const LanczosDev& L, int j, int nb, int last, double** next_slot, double tau,
-                           double eps1) {
-  __shared__ double sh[32];
-  __shared__ double s_om[PRO_MAX];
+// The decision of a step, by one block, from |w|^2 = acc and what pro_prepare left.
+// Returns whether the step takes the pass; `word` (unless null) receives it for the
+// other CTAs as soon as it is known.
+__device__ bool pro_decide(const LanczosDev& L, int j, double acc, double a, double bj, int last, int forced,
+                           double** next_slot, double tau, double eps1, double* om_t, const ProScales& sc,
+                           unsigned long long* word) {
   __shared__ double s_b, s_inv;
-  __shared__ unsigned long long s_amax, s_an, s_mx[4];
+  __shared__ unsigned long long s_mx[4];
   __shared__ int s_pass;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (wid == 1) {
-    unsigned long long amax, an;
-    tridiag_scale(L, j, lane, amax, an);
-    if (lane == 0) {
-      s_amax = amax;
-      s_an = an;
-    }
-  }
-  const double acc = partial_sum(L.partial, nb, sh);
-  if (threadIdx.x == 0) {
-    s_b = sqrt(acc);
-    s_inv = 1.0 / s_b;
-  }
+  // the root and the reciprocal root side by side, in two SM quarters
+  if (threadIdx.x == 0) s_b = sqrt(acc);
+  if (threadIdx.x == 32) s_inv = rsqrt(acc);
   __syncthreads();
   const double bn = s_b, inv = s_inv;
   // one warp per SM quarter covers the j + 1 estimates
   if (threadIdx.x < 128) {
-    const double* om = L.omega;                  // row j: k = 0..j
-    const double* omp = L.omega + (L.nmax + 2);  // row j-1: k = 0..j-1
-    const double aj = L.alpha[j], bj = j > 0 ? L.beta[j] : 0.0;
-    const double an = __longlong_as_double((long long)max(s_an, bits_abs(fabs(aj) + bj + bn)));
+    const double an = __longlong_as_double((long long)max(sc.an, bits_abs(fabs(a) + bj + bn)));
     const double round = eps1 * an;
     unsigned long long mx = 0;
     for (int k = threadIdx.x; k <= j; k += 128) {
-      double e;
-      if (k < j) {
-        double t = L.beta[k + 1] * om[k + 1] + (L.alpha[k] - aj) * om[k] - bj * omp[k];
-        if (k > 0) t += L.beta[k] * om[k - 1];
-        e = (t + copysign(round, t)) * inv;
-      } else {
-        e = round * inv;
-      }
-      s_om[k] = e;
+      const double t = k < j ? om_t[k] : 0.0;
+      const double e = k < j ? (t + copysign(round, t)) * inv : round * inv;
+      om_t[k] = e;
       // beta_{j+1} = 0 or an overflowing estimate (its bit pattern lies above every
       // finite one's) counts as lost orthogonality
       mx = max(mx, bits_abs(e));
@@ -434,7 +266,6 @@ __device__ void pro_decide(const LanczosDev& L, int j, int nb, int last, double*
   __syncthreads();
   if (threadIdx.x == 0) {
     const unsigned long long m = max(max(s_mx[0], s_mx[1]), max(s_mx[2], s_mx[3]));
-    const int forced = L.state[3];
     const int pass = forced || !(tau >= 0.0 && m <= bits_abs(tau));
     s_pass = pass;
     L.state[2] = pass;
@@ -443,54 +274,360 @@ __device__ void pro_decide(const LanczosDev& L, int j, int nb, int last, double*
       L.beta[j + 1] = bn;
       L.scratch[3 * L.nmax + 3] = inv;   // for the normalising kernel
       L.state[0] = j + 1;
-      if (last || bn < 1e-14 * __longlong_as_double((long long)s_amax)) L.state[1] = 1;
+      if (last || bn < 1e-14 * __longlong_as_double((long long)sc.amax)) L.state[1] = 1;
       else *next_slot = L.V + (int64_t)(j + 1) * L.n;
     }
+    if (word)
+      asm volatile("st.release.gpu.u64 [%0], %1;" ::"l"(word), "l"(2ull * (j + 1) + (pass ? 1 : 0)) : "memory");
   }
   __syncthreads();
-  // shift the rows: row j becomes row j-1, the new estimates row j+1
-  double* cur = L.omega;
-  double* prev = L.omega + (L.nmax + 2);
-  for (int k = threadIdx.x; k <= j; k += RT) {
-    prev[k] = cur[k];
-    cur[k] = s_pass ? eps1 : s_om[k];
-  }
-  if (threadIdx.x == 0) cur[j + 1] = 1.0;
+  return s_pass != 0;
 }
 
-// The three-term step w <- (w - alpha_j v_j) - beta_j v_{j-1} (beta_0 = 0), with
-// partial[b] = this block's share of the new |w|^2 (fixed order).
-__global__ void __launch_bounds__(RT) three_term_norm_kernel(LanczosDev L, int j, int last, double** next_slot,
-                                                              double tau, double eps1) {
+// Row j of the estimates becomes row j-1, the new ones row j+1.
+__device__ __forceinline__ void pro_shift(const LanczosDev& L, int j, bool pass, double eps1, const double* om_t,
+                                          const double* om) {
+  for (int k = threadIdx.x; k <= j; k += LT) {
+    L.omega[L.nmax + 2 + k] = om[k];
+    L.omega[k] = pass ? eps1 : om_t[k];
+  }
+  if (threadIdx.x == 0) L.omega[j + 1] = 1.0;
+}
+
+// ---------------------------------------------------------------- one step in one launch
+// Waits among the CTAs of a step.  A cluster uses the hardware's cluster barrier.  A
+// grid (cooperative: all CTAs resident, which the launch checks) counts arrivals in
+// 64-bit words that only grow during a solve (lanczos_init_kernel zeroes them);
+// every poll is bounded by the clock (about a second).
+constexpr long long STEP_WAIT = 2000000000LL;
+constexpr int STEP_CL = 8;   // CTAs of the cluster
+
+__device__ bool poll_at_least(const unsigned long long* word, unsigned long long target) {
+  const long long t0 = clock64();
+  for (;;) {
+    unsigned long long cur;
+    asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(cur) : "l"(word) : "memory");
+    if (cur >= target) return true;
+    if (clock64() - t0 > STEP_WAIT) return false;
+  }
+}
+
+__device__ __forceinline__ unsigned long long arrive(unsigned long long* word) {
+  unsigned long long old;
+  asm volatile("atom.add.release.gpu.u64 %0, [%1], 1;" : "=l"(old) : "l"(word) : "memory");
+  return old;
+}
+
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// All CTAs; what thread 0 of each wrote before is visible to every thread after.
+template <bool CLUSTER>
+__device__ bool step_barrier(const LanczosDev& L) {
+  if (CLUSTER) {
+    cluster_arrive();
+    cluster_wait();
+    return true;
+  }
+  bool ok = true;
+  if (threadIdx.x == 0) {
+    // the count before this arrival lies in [k G, (k + 1) G) at barrier k of G CTAs
+    const unsigned long long old = arrive(step_words(L));
+    ok = poll_at_least(step_words(L), (old / gridDim.x + 1) * (unsigned long long)gridDim.x);
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+// Sum over the block, valid in warp 0's first eight lanes.
+__device__ __forceinline__ double step_block_sum(double v, double* sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  v = warp_sum(v);
+  if (lane == 0) sh[wid] = v;
+  __syncthreads();
+  if (wid == 0) {
+    v = lane < LT / 32 ? sh[lane] : 0.0;
+#pragma unroll
+    for (int o = LT / 64; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  }
+  return v;
+}
+
+// Leaves this CTA's partial (of step_block_sum) where every CTA's step_total finds it: in
+// a cluster in the others' shared memory, else in part[].
+template <bool CLUSTER>
+__device__ __forceinline__ void step_publish(double v, double* part, double* s_part) {
+  static_assert(LT / 32 >= STEP_CL, "lanes that hold the sum");
+  if (CLUSTER) {
+    if (threadIdx.x < STEP_CL)
+      *cooperative_groups::this_cluster().map_shared_rank(s_part + blockIdx.x, threadIdx.x) = v;
+  } else if (threadIdx.x == 0) {
+    part[blockIdx.x] = v;
+  }
+}
+
+// Sum of every CTA's partial, in the same order in every CTA; valid in all threads.
+template <bool CLUSTER>
+__device__ double step_total(const double* part, const double* s_part, double* sh) {
+  if (CLUSTER) {   // every warp for itself
+    double v = s_part[threadIdx.x & (STEP_CL - 1)];
+#pragma unroll
+    for (int o = STEP_CL / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  }
+  double v = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += LT) v += __ldcg(part + b);
+  v = step_block_sum(v, sh);
+  if (threadIdx.x == 0) sh[LT / 32] = v;
+  __syncthreads();
+  return sh[LT / 32];
+}
+
+// Dots of w against NG basis vectors from row g0 over this CTA's entries [c0, c1), left
+// per thread in sh (NG fixed at compile time, so no FP64 instruction is issued for
+// a vector that does not exist).
+template <int NG>
+__device__ __forceinline__ void multidot_group(const LanczosDev& L, int g0, int64_t c0, int64_t c1,
+                                               double (*sh)[LT + 1]) {
+  double acc[NG];
+#pragma unroll
+  for (int i = 0; i < NG; ++i) acc[i] = 0.0;
+  for (int64_t x = c0 + threadIdx.x; x < c1; x += LT) {
+    const double wx = L.w[x];
+    double v[NG];
+#pragma unroll
+    for (int i = 0; i < NG; ++i) v[i] = L.V[(int64_t)(g0 + i) * L.n + x];
+#pragma unroll
+    for (int i = 0; i < NG; ++i) acc[i] = fma(v[i], wx, acc[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < NG; ++i) sh[i][threadIdx.x] = acc[i];
+}
+
+// Dots of this CTA's entries against V_0 .. V_{m-1} into out[i].
+__device__ void block_multidot(const LanczosDev& L, int m, int64_t c0, int64_t c1, double (*sh)[LT + 1],
+                               double* out) {
+  for (int g0 = 0; g0 < m; g0 += 16) {
+    const int ng = m - g0 < 16 ? m - g0 : 16;
+    switch ((ng + 1) / 2) {
+      case 1: ng == 1 ? multidot_group<1>(L, g0, c0, c1, sh) : multidot_group<2>(L, g0, c0, c1, sh); break;
+      case 2: ng == 3 ? multidot_group<3>(L, g0, c0, c1, sh) : multidot_group<4>(L, g0, c0, c1, sh); break;
+      case 3: ng == 5 ? multidot_group<5>(L, g0, c0, c1, sh) : multidot_group<6>(L, g0, c0, c1, sh); break;
+      case 4: ng == 7 ? multidot_group<7>(L, g0, c0, c1, sh) : multidot_group<8>(L, g0, c0, c1, sh); break;
+      case 5: ng == 9 ? multidot_group<9>(L, g0, c0, c1, sh) : multidot_group<10>(L, g0, c0, c1, sh); break;
+      case 6: ng == 11 ? multidot_group<11>(L, g0, c0, c1, sh) : multidot_group<12>(L, g0, c0, c1, sh); break;
+      case 7: ng == 13 ? multidot_group<13>(L, g0, c0, c1, sh) : multidot_group<14>(L, g0, c0, c1, sh); break;
+      default: ng == 15 ? multidot_group<15>(L, g0, c0, c1, sh) : multidot_group<16>(L, g0, c0, c1, sh); break;
+    }
+    __syncthreads();
+    // thread t sums every 16th entry of row t / 16, then its 16 partners combine
+    const int row = threadIdx.x >> 4, part = threadIdx.x & 15;
+    if (row < ng) {
+      double v = 0.0;
+#pragma unroll
+      for (int q = 0; q < LT / 16; ++q) v += sh[row][part + 16 * q];
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffu << (threadIdx.x & 16), v, o, 16);
+      if (part == 0) out[g0 + row] = v;
+    }
+    __syncthreads();
+  }
+}
+
+// A whole Lanczos step after w = H v_j, in one launch: alpha_j = <v_j, w>; the
+// three-term step w <- (w - alpha_j v_j) - beta_j v_{j-1} (beta_0 = 0) with |w|^2; the
+// decision above, by CTA 0 while the others wait for it; and, in a step that takes it,
+// the Gram-Schmidt pass c = V^T w, w <- w - V c against v_0 .. v_j with the new
+// norm, beta_{j+1} and the stopping test (by the CTA that finishes last).  Each CTA
+// keeps to its own contiguous run of entries, so that only the partial sums cross
+// CTAs, in regions of L.partial that no CTA can still be reading when they are
+// rewritten.  The sums' order is fixed by the grid.
+//
+// Bound by latency up to some 10^5 entries and by FP64 issue above (4 fused
+// multiply-adds per entry at 2 per clock and SM; a pass 2 (j + 1) + 1 more).  As four
+// launches (the dots, the three-term step, and two that returned at once in a step
+// without the pass) a step took 22, 27 and 50 us at 4096, 126780 and 1.46M entries;
+// in one launch it takes 9.6, 12.5 and 25.5 (ncu, cold caches).
+template <bool CLUSTER>
+__global__ void __launch_bounds__(LT, 2) lanczos_step_kernel(LanczosDev L, int j, int last, double** next_slot,
+                                                             double tau, double eps1, int32_t* status) {
   tnx_grid_dependency();
+  __shared__ double sh_rows[16][LT + 1];
+  __shared__ double s_v[PRO_MAX];   // estimates, then the pass's coefficients
   __shared__ double sh[32];
+  __shared__ ProScales s_sc;
+  __shared__ int s_ok, s_pass;
+  __shared__ double s_part[2][STEP_CL];
   if (stopped(L.state)) return;
-  const double a = L.alpha[j], b = j > 0 ? L.beta[j] : 0.0;
+  const int nb = gridDim.x, tid = threadIdx.x;
+  const int64_t chunk = ((L.n + nb - 1) / nb + 31) / 32 * 32;
+  const int64_t c0 = min(L.n, chunk * blockIdx.x), c1 = min(L.n, c0 + chunk);
   const double* vj = L.V + (int64_t)j * L.n;
   const double* vp = L.V + (int64_t)(j > 0 ? j - 1 : 0) * L.n;
+  double* part = L.partial;   // [nb] alpha (later the pass's norms), [nb] norms, [nb][j + 1] dots
+  // a wait that ran out: the solve stops, with an eigenvalue that is not a number
+  auto give_up = [&](int code) {
+    if (tid == 0) {
+      atomicExch(status, code);
+      L.alpha[j] = __longlong_as_double(0x7FF8000000000000ll);
+      L.state[0] = j + 1;
+      L.state[1] = 1;
+    }
+  };
+
+  // Everything that does not depend on the sums is read at once: the first U entries
+  // per thread of all three vectors (kept in registers), beta_j and, in CTA 0, T and the
+  // estimates; a load that waits for a sum or a decision costs the step its latency.
+  constexpr int U = 4;
+  const ProRows rows = {&sh_rows[0][0], &sh_rows[0][0] + PRO_MAX, &sh_rows[0][0] + 2 * PRO_MAX,
+                        &sh_rows[0][0] + 3 * PRO_MAX};
+  static_assert(4 * PRO_MAX <= 16 * (LT + 1), "the rows lie where a pass keeps its products");
+  const int64_t x0 = c0 + tid;
+  double w0[U], v0[U], p0[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    w0[u] = v0[u] = p0[u] = 0.0;
+    if (x0 + u * LT < c1) {
+      w0[u] = L.w[x0 + u * LT];
+      v0[u] = vj[x0 + u * LT];
+      p0[u] = vp[x0 + u * LT];
+    }
+  }
+  const double b = j > 0 ? L.beta[j] : 0.0;
+  int forced = 0;
+  if (blockIdx.x == 0) {
+    pro_load(L, j, rows);
+    if (tid == 0) forced = L.state[3];
+  }
+  double acc = 0.0;
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (x0 + u * LT < c1) acc = fma(w0[u], v0[u], acc);
+  for (int64_t x = x0 + U * LT; x < c1; x += U * LT) {
+    double w[U], v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (x + u * LT < c1) {
+        w[u] = L.w[x + u * LT];
+        v[u] = vj[x + u * LT];
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (x + u * LT < c1) acc = fma(w[u], v[u], acc);
+  }
+  acc = step_block_sum(acc, sh);
+  step_publish<CLUSTER>(acc, part, s_part[0]);
+  if (!step_barrier<CLUSTER>(L)) return give_up(41);
+  const double a = step_total<CLUSTER>(part, s_part[0], sh);
+  __syncthreads();   // sh is reused
+
   double nrm = 0.0;
-  const int64_t stride = (int64_t)gridDim.x * RT;
-  int64_t x = (int64_t)blockIdx.x * RT + threadIdx.x;
-  for (; x + stride < L.n; x += 2 * stride) {
-    const double w0 = L.w[x], w1 = L.w[x + stride];
-    const double a0 = vj[x], a1 = vj[x + stride];
-    const double p0 = vp[x], p1 = vp[x + stride];
-    const double u0 = (w0 - a * a0) - b * p0, u1 = (w1 - a * a1) - b * p1;
-    L.w[x] = u0;
-    L.w[x + stride] = u1;
-    nrm = fma(u0, u0, nrm);
-    nrm = fma(u1, u1, nrm);
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (x0 + u * LT < c1) {
+      const double r = (w0[u] - a * v0[u]) - b * p0[u];
+      L.w[x0 + u * LT] = r;
+      nrm = fma(r, r, nrm);
+    }
+  for (int64_t x = x0 + U * LT; x < c1; x += U * LT) {
+    double w[U], v[U], p[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (x + u * LT < c1) {
+        w[u] = L.w[x + u * LT];
+        v[u] = vj[x + u * LT];
+        p[u] = vp[x + u * LT];
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (x + u * LT < c1) {
+        const double r = (w[u] - a * v[u]) - b * p[u];
+        L.w[x + u * LT] = r;
+        nrm = fma(r, r, nrm);
+      }
   }
-  if (x < L.n) {
-    const double u = (L.w[x] - a * vj[x]) - b * vp[x];
-    L.w[x] = u;
-    nrm = fma(u, u, nrm);
+  nrm = step_block_sum(nrm, sh);
+  step_publish<CLUSTER>(nrm, part + nb, s_part[1]);
+
+  bool pass;
+  if (CLUSTER) {
+    cluster_arrive();
+    if (blockIdx.x == 0) {
+      pro_prepare(rows, j, a, s_v, &s_sc);
+      if (tid == 0) L.alpha[j] = a;
+    }
+    cluster_wait();
+    if (blockIdx.x == 0) {
+      __syncthreads();
+      pass = pro_decide(L, j, step_total<CLUSTER>(part + nb, s_part[1], sh), a, b, last, forced, next_slot, tau, eps1, s_v, s_sc,
+                        nullptr);
+      if (tid < STEP_CL) *cooperative_groups::this_cluster().map_shared_rank(&s_pass, tid) = pass;
+      cluster_arrive();
+      pro_shift(L, j, pass, eps1, s_v, rows.om);
+    } else {
+      cluster_arrive();
+    }
+    cluster_wait();
+    pass = s_pass != 0;
+  } else {
+    unsigned long long* words = step_words(L);
+    if (tid == 0) arrive(words + SW);
+    if (blockIdx.x == 0) {
+      pro_prepare(rows, j, a, s_v, &s_sc);
+      if (tid == 0) {
+        L.alpha[j] = a;
+        s_ok = poll_at_least(words + SW, (unsigned long long)(j + 1) * nb);
+      }
+      __syncthreads();
+      if (!s_ok) return give_up(42);
+      pass = pro_decide(L, j, step_total<CLUSTER>(part + nb, s_part[1], sh), a, b, last, forced, next_slot, tau, eps1, s_v, s_sc,
+                        words + 2 * SW);
+      pro_shift(L, j, pass, eps1, s_v, rows.om);
+    } else {
+      // nothing is left for these CTAs but to learn whether there is a pass
+      if (tid == 0) {
+        s_ok = poll_at_least(words + 2 * SW, 2ull * (j + 1));
+        s_pass = (int)(*(volatile unsigned long long*)(words + 2 * SW) & 1);
+      }
+      __syncthreads();
+      if (!s_ok) return give_up(43);
+      pass = s_pass != 0;
+    }
   }
-  nrm = block_sum(nrm, sh);
-  if (threadIdx.x == 0) L.partial[blockIdx.x] = nrm;
+  if (!pass) return;
+
+  __syncthreads();   // the rows and estimates have been read
+  const int m = j + 1;
+  double* dots = part + 2 * nb;
+  block_multidot(L, m, c0, c1, sh_rows, dots + (int64_t)blockIdx.x * m);
+  __threadfence();   // the dots come from 16 threads, the barrier's arrival from one
+  __syncthreads();
+  if (!step_barrier<CLUSTER>(L)) return give_up(44);
+  for (int i = tid >> 5; i < m; i += LT / 32) {
+    double v = 0.0;
+    for (int q = tid & 31; q < nb; q += 32) v += __ldcg(dots + (int64_t)q * m + i);
+    v = warp_sum(v);
+    if ((tid & 31) == 0) s_v[i] = v;
+  }
+  __syncthreads();
+  nrm = 0.0;
+  for (int64_t x = c0 + tid; x < c1; x += LT) {
+    double w = L.w[x];
+#pragma unroll 8
+    for (int i = 0; i < m; ++i) w -= s_v[i] * L.V[(int64_t)i * L.n + x];
+    L.w[x] = w;
+    nrm = fma(w, w, nrm);
+  }
+  nrm = step_block_sum(nrm, sh);
+  if (tid == 0) part[blockIdx.x] = nrm;
   if (last_block(L.state + 4)) {
-    pro_decide(L, j, gridDim.x, last, next_slot, tau, eps1);
-    if (threadIdx.x == 0) L.state[4] = 0;
+    beta_decide(L, j, nb, last, next_slot);
+    if (tid == 0) L.state[4] = 0;
   }
 }
 
@@ -766,44 +903,60 @@ cudaError_t tnx_launch_lanczos_set_input(double** slot_ptr, const LanczosDev& L,
 
 // The operator has been applied: L.w = H v_j.  One Lanczos step (without the
 // final v_{j+1} = w / beta_{j+1} when `normalize` is false: the caller then
-// fuses it with the next apply's relayout of the vector): alpha_j = <v_j, w>;
-// the three-term step w <- w - alpha_j v_j - beta_j v_{j-1} with |w|; the
-// orthogonality estimates, which decide whether this step takes a classical
-// Gram-Schmidt pass c = V^T w, w <- w - V c against v_0..v_j (the gated
-// launches: a step without the pass returns from them at once); then
-// beta_{j+1}, the stopping test and v_{j+1} = w / beta_{j+1}.  FP64 work per
-// entry: 3 fused multiply-adds, plus 2 (j + 1) + 1 in a step with the pass.
+// fuses it with the next apply's relayout of the vector).
+//
+// Up to 20480 entries the step is one cluster of eight CTAs (barriers and partial sums
+// stay among eight SMs, and its launch overlaps the end of the apply); above, where eight
+// SMs' FP64 units would bound it, a resident grid of CTAs of 1024 entries, at most one
+// per SM up to 4096 entries each, then two (more loads in flight).  Whole solves of 20
+// steps, cluster | grid: 4096 entries 1033 | 1100 us, 16384 1179 | 1208, 25676 1538 |
+// 1515, 37344 1117 | 1049, 126780 1661 | 1330; one | two CTAs per SM: 1.46M entries
+// 5757 | 5676 us.
+constexpr int64_t STEP_CLUSTER_MAX = 20480;
+
 cudaError_t tnx_launch_lanczos_step(const LanczosDev& L, int j, double** next_slot, cudaStream_t st, bool normalize,
-                                    bool always_pass) {
+                                    bool always_pass, int32_t* status) {
   if (j + 2 > PRO_MAX) return cudaErrorInvalidValue;
   const double tau = always_pass ? -1.0 : 1e-10;
-  const int nb = grid_for(L.n);
-  const int m = j + 1;
-  const int mb = multidot_blocks(L.n);
+  const double eps1 = sqrt((double)L.n) * 0.5 * 2.220446049250313e-16;
   const int last = j == L.nmax - 1;
-  {
-    const cudaError_t le = tnx_launch(multidot_kernel, dim3(mb), dim3(MD_T), 0, st, L, 1, j, 0, 0, j);
-    if (le != cudaSuccess) return le;
+  const bool cluster = L.n <= STEP_CLUSTER_MAX;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  cfg.blockDim = dim3(LT);
+  cfg.stream = st;
+  cfg.attrs = at;
+  if (cluster) {
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = STEP_CL;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+    cfg.gridDim = dim3(STEP_CL);
+  } else {
+    int dev = 0, nsm = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lanczos_step_kernel<false>, LT, 0);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorNotSupported;
+    const int64_t want = (L.n + 4 * LT - 1) / (4 * LT);
+    int64_t nb = want <= nsm ? want : want <= 4 * (int64_t)nsm || per_sm < 2 ? nsm : 2 * (int64_t)nsm;
+    if (nb > TNX_LANCZOS_BLOCKS) nb = TNX_LANCZOS_BLOCKS;
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3((unsigned)nb);
   }
-  {
-    const cudaError_t le = tnx_launch(three_term_norm_kernel, dim3(nb), dim3(RT), 0, st, L, j, last, next_slot, tau,
-                                      sqrt((double)L.n) * 0.5 * 2.220446049250313e-16);
-    if (le != cudaSuccess) return le;
-  }
-  {
-    const cudaError_t le = tnx_launch(multidot_kernel, dim3(mb), dim3(MD_T), 0, st, L, m, 0, 1, -1, 0);
-    if (le != cudaSuccess) return le;
-  }
-  {
-    const cudaError_t le = tnx_launch(gs_update_kernel, dim3(nb), dim3(RT), 0, st, L, m, 1, 1, j, last, next_slot);
-    if (le != cudaSuccess) return le;
-  }
-  tnx_note_launch(4);
+  const cudaError_t le = cluster
+      ? cudaLaunchKernelEx(&cfg, lanczos_step_kernel<true>, L, j, last, next_slot, tau, eps1, status)
+      : cudaLaunchKernelEx(&cfg, lanczos_step_kernel<false>, L, j, last, next_slot, tau, eps1, status);
+  if (le != cudaSuccess) return le;
+  tnx_note_launch(1);
   if (normalize) {
-    {
-      const cudaError_t le = tnx_launch(lanczos_normalize_kernel, dim3(nb), dim3(RT), 0, st, L, j);
-      if (le != cudaSuccess) return le;
-    }
+    const cudaError_t e = tnx_launch(lanczos_normalize_kernel, dim3(grid_for(L.n)), dim3(RT), 0, st, L, j);
+    if (e != cudaSuccess) return e;
     tnx_note_launch(1);
   }
   return cudaGetLastError();

@@ -418,17 +418,18 @@ cudaError_t tnx_launch_norm2(const double* x, int64_t n, double* partial, double
 int tnx_reduce_blocks(int64_t n);
 
 // Lanczos device state
+#define TNX_LANCZOS_BLOCKS 304   // CTAs of a step at most
 struct LanczosDev {
   double* V;          // [nmax+1][n] basis
   double* w;          // [n]
   double* alpha;      // [nmax]
   double* beta;       // [nmax+1]
-  double* coef;       // [nmax+1]  Gram-Schmidt coefficients
-  double* partial;    // [nblocks * (nmax+1)]
+  double* partial;    // max(1216, TNX_LANCZOS_BLOCKS * (nmax+2)) partial sums
   double* y;          // [nmax]    Ritz coefficients
   double* scratch;    // [4*nmax]
   int32_t* state;     // [0] = active steps done (k), [1] = stopped flag, [2] = this step reorthogonalises,
-                      // [3] = the next step must reorthogonalise too, [4] = blocks done (last-block reductions)
+                      // [3] = the next step must reorthogonalise too, [4] = blocks done (last-block reductions),
+                      // from [32], 128 bytes apart, three 64-bit words that the CTAs of a step wait on
   double* omega;      // [2][nmax+2] estimates of <v_j, v_k> (row j, then row j-1)
   double* eval;       // [1]
   int64_t n;
@@ -439,7 +440,8 @@ cudaError_t tnx_launch_lanczos_init(const LanczosDev& L, const double* v0, cudaS
 cudaError_t tnx_launch_lanczos_set_input(double** slot_ptr, const LanczosDev& L, int j, cudaStream_t st);
 // normalize = false leaves out v_{j+1} = w / beta_{j+1} (1 / beta_{j+1} is in
 // scratch[3 * nmax + 3]) for the caller to fuse with its next relayout;
-// always_pass: a Gram-Schmidt pass in every step (an operator far from symmetric)
+// always_pass: a Gram-Schmidt pass in every step (an operator far from symmetric);
+// *status receives 41..44 when a wait among the step's CTAs ran out (the solve stops)
 cudaError_t tnx_launch_lanczos_step(const LanczosDev& L, int j, double** next_slot, cudaStream_t st, bool normalize,
-                                    bool always_pass);
+                                    bool always_pass, int32_t* status);
 cudaError_t tnx_launch_lanczos_finish(const LanczosDev& L, double* evec, cudaStream_t st);

@@ -2173,11 +2173,11 @@ tnx_network::~tnx_network() = default;
 
 namespace {
 // Bytes of the Lanczos workspace buffers, in allocation order: V, w, alpha,
-// beta, coef, partial sums, y, scratch, state, eval, omega.
+// beta, partial sums, y, scratch, state, eval, omega.
 std::vector<size_t> lanczos_buffer_sizes(int64_t n, int nsteps) {
   return {(size_t)(nsteps + 1) * n * 8, (size_t)n * 8, (size_t)(nsteps + 1) * 8, (size_t)(nsteps + 2) * 8,
-          (size_t)(nsteps + 2) * 8, (size_t)std::max<int64_t>(1216, (int64_t)608 * (nsteps + 2)) * 8,
-          (size_t)(nsteps + 1) * 8, (size_t)(4 * (nsteps + 1)) * 8, 64, 64, (size_t)(2 * (nsteps + 2)) * 8};
+          (size_t)std::max<int64_t>(1216, (int64_t)TNX_LANCZOS_BLOCKS * (nsteps + 2)) * 8,
+          (size_t)(nsteps + 1) * 8, (size_t)(4 * (nsteps + 1)) * 8, 512, 64, (size_t)(2 * (nsteps + 2)) * 8};
 }
 }  // namespace
 
@@ -2308,13 +2308,12 @@ void tnx_lanczos_enqueue(tnx_network* net, int slot, tnx_tensor* v0, int nsteps,
     L.w = (double*)dev(sz[1]);
     L.alpha = (double*)dev(sz[2]);
     L.beta = (double*)dev(sz[3]);
-    L.coef = (double*)dev(sz[4]);
-    L.partial = (double*)dev(sz[5]);
-    L.y = (double*)dev(sz[6]);
-    L.scratch = (double*)dev(sz[7]);
-    L.state = (int32_t*)dev(sz[8]);
-    L.eval = (double*)dev(sz[9]);
-    L.omega = (double*)dev(sz[10]);
+    L.partial = (double*)dev(sz[4]);
+    L.y = (double*)dev(sz[5]);
+    L.scratch = (double*)dev(sz[6]);
+    L.state = (int32_t*)dev(sz[7]);
+    L.eval = (double*)dev(sz[8]);
+    L.omega = (double*)dev(sz[9]);
   }
   LanczosDev& L = lc->L;
   bind_inputs(net, *p);
@@ -2417,7 +2416,7 @@ void tnx_lanczos_enqueue(tnx_network* net, int slot, tnx_tensor* v0, int nsteps,
       // (j+1)n + 2n for the update
       ProfScope ps(ctx, st, TNX_KC_VECTOR, 8.0 * (double)n * 8);
       CUDA_CHECK(tnx_launch_lanczos_step(L, j, p->d_slots + slot, st, vcopy == nullptr,
-                                         p->prec == TNX_PREC_F32 || p->prec == TNX_PREC_TF32));
+                                         p->prec == TNX_PREC_F32 || p->prec == TNX_PREC_TF32, ctx->d_status));
       if (vslice) {
         // v_{j+1} and the next apply's slices of the vector operand in one pass over w
         const VecSrc vs{(const int64_t*)lc->vs_rowtab->p, L.w, L.V + (int64_t)(j + 1) * n,
