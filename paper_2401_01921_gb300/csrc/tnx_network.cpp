@@ -285,11 +285,13 @@ void sparse_optimal_tree(tnx_network* net) {
       if (cnt[l] == 1) open[m].push_back(l);
   }
   // the bond of label l as it appears inside subset m
+  std::vector<std::vector<std::pair<int, const BondD*>>> at;   // occ by label index
+  for (auto& kv : occ) at.push_back(kv.second);
   auto bond_in = [&](int l, uint32_t m) -> const BondD& {
-    for (auto& o : occ[labs[l]])
+    for (auto& o : at[l])
       if (m >> o.first & 1) return *o.second;
     fail(TNX_ERR_NETWORK, "internal: label outside its subset");
-    return *occ[labs[l]][0].second;
+    return *at[l][0].second;
   };
   // the histogram of the legs ls as they appear inside subset m, kept by the bonds
   // they are (a leg belongs to one or two tensors, so few sets differ)
