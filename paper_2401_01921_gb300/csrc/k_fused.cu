@@ -174,6 +174,104 @@ __global__ void __launch_bounds__(FT, RUN ? 5 : 6) fused_skinny_kernel(const Gem
   }
 }
 
+// The same step for small bands (charge blocks of a few rows), one warp per tile of at
+// most FR rows.  A row belongs to one lane: it gathers the row's A elements into a column
+// of the warp's shared memory that only it reads (the list of nonzeros picks elements by
+// number), forms the outputs and stores them at once.  Lanes walk q, then p, of tiles at
+// most 8 wide along q when the band allows it, so that 32-byte sectors are read whole
+// along q and written whole along p without a transposing stage.
+//
+// A tile of 128 rows by 8 warps spends its time on the chain of loads before the
+// product (tile, group and descriptors, B and A), whatever the number of rows, and an SM
+// holds six; here it holds 28 chains.  Still bound by instruction issue and latency (about
+// 1000 warp instructions a tile, 40% of the issue slots, FP64 pipe 30%).  48 Hubbard
+// sites (75 thousand bands of 1 to 256 rows): 166 us for what took 178 (the instances
+// with 32 rows per tile and more) and 135 (relayouts and skinny products of the others)
+// before; the two MPO steps of one at bond dimension 601: 25 us for 41 (ncu, cold).
+constexpr int FW = 4;   // warps per CTA, each on its own tile
+
+__host__ __device__ constexpr size_t warp_smem(int kp, int np) {
+  return ((size_t)kp * 32 * 8 + (size_t)np * kp * 9 + (size_t)(kp + np) * sizeof(FusedCol) + (size_t)np * 8 + 15) / 16 *
+         16;
+}
+
+__global__ void __launch_bounds__(32 * FW, 8) fused_warp_kernel(const GemmGroup* __restrict__ groups,
+                                                                const FusedTile* __restrict__ tiles, int ntiles,
+                                                                const FusedCol* __restrict__ cols, int kp, int np,
+                                                                double* const* __restrict__ slots) {
+  tnx_grid_dependency();
+  extern __shared__ __align__(16) unsigned char dyn[];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int ti = blockIdx.x * FW + wid;
+  if (ti >= ntiles) return;
+  unsigned char* base = dyn + (size_t)wid * warp_smem(kp, np);
+  FusedCol* s_d = (FusedCol*)base;                        // [kp] of A, [np] of the output
+  double* s_a = (double*)(s_d + kp + np) + lane;          // [kp][32]: this lane's column
+  double* s_v = (double*)(s_d + kp + np) + kp * 32;       // [np][kp] nonzeros
+  int* s_cnt = (int*)(s_v + np * kp);                     // [np]
+  uint32_t* s_p2 = (uint32_t*)(s_cnt + np);               // [np]
+  unsigned char* s_k = (unsigned char*)(s_p2 + np);       // [np][kp]
+  const FusedTile T = tiles[ti];
+  const int W = T.W, N = T.N;
+  const GemmGroup g = groups[T.group];
+  const int nd = T.scol >= 0 ? W + N : W;
+  for (int i = lane; i < nd; i += 32) s_d[i < W ? i : kp + i - W] = cols[i < W ? T.gcol + i : T.scol + i - W];
+  for (int n = lane; n < N; n += 32) {
+    const double* brow = slots[g.b_slot] + g.b_off + (int64_t)n * g.ldb;
+    int c = 0;
+    for (int k0 = 0; k0 < g.K; k0 += 4) {
+      double b[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) b[k] = k0 + k < g.K ? brow[k0 + k] : 0.0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (b[k] != 0.0) {
+          s_v[n * kp + c] = b[k];
+          s_k[n * kp + c] = (unsigned char)(k0 + k);
+          ++c;
+        }
+      }
+    }
+    s_cnt[n] = c;
+    s_p2[n] = c ? tnx_pow2_code(s_v[n * kp]) : 0u;
+  }
+  __syncwarp();
+  double* C = T.scol >= 0 ? nullptr : slots[g.c_slot] + g.c_off;
+  const int rows = T.eP * T.eQ, mq = small_magic(T.eQ);
+  for (int r = lane; r < rows; r += 32) {
+    const int p = small_div(r, mq), q = r - p * T.eQ;
+    const int64_t P = T.p0 + p, Q = T.q0 + q;
+    for (int c0 = 0; c0 < W; c0 += 4) {
+      double v[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        v[c] = 0.0;
+        if (c0 + c < W) {
+          const FusedCol d = s_d[c0 + c];
+          if (d.ptr) v[c] = __ldg(d.ptr + P * d.sP + Q * d.sQ);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c0 + c < W) s_a[(c0 + c) * 32] = v[c];
+    }
+    for (int n = 0; n < N; ++n) {
+      double acc = 0.0;
+      const int c = s_cnt[n];
+      const double* bv = s_v + n * kp;
+      const unsigned char* bk = s_k + n * kp;
+      if (c > 0) acc = tnx_first_term(s_a[bk[0] * 32], bv[0], s_p2[n]);
+      for (int e = 1; e < c; ++e) acc = fma(s_a[bk[e] * 32], bv[e], acc);
+      if (C) {
+        C[((int64_t)T.row0 + P * T.EQ + Q) * g.ldc + n] = acc;
+      } else {
+        const FusedCol d = s_d[kp + n];
+        if (d.ptr) d.ptr[P * d.sP + Q * d.sQ] = acc;
+      }
+    }
+  }
+}
+
 }  // namespace
 
 size_t tnx_fused_smem_bytes(int kp, int np) { return sizeof(FusedSmem) + (size_t)FR * (kp + np) * sizeof(double); }
@@ -195,14 +293,30 @@ cudaError_t launch_fused(const GemmGroup* groups, const FusedTile* tiles, int nt
   const size_t smem = tnx_fused_smem_bytes(kp, np) + (RUN ? FMAXK * sizeof(FusedCol) : 0);
   return tnx_launch(fused_skinny_kernel<RUN>, dim3(ntiles), dim3(FT), smem, st, groups, tiles, cols, kp, np, slots);
 }
+cudaError_t launch_fused_warp(const GemmGroup* groups, const FusedTile* tiles, int ntiles, const FusedCol* cols, int kp,
+                              int np, double* const* slots, cudaStream_t st) {
+  static int attr_dev = -1;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (attr_dev != dev) {
+    e = cudaFuncSetAttribute(fused_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(FW * warp_smem(FMAXK + 1, FMAXN + 1)));
+    if (e != cudaSuccess) return e;
+    attr_dev = dev;
+  }
+  return tnx_launch(fused_warp_kernel, dim3((ntiles + FW - 1) / FW), dim3(32 * FW), FW * warp_smem(kp, np), st, groups,
+                    tiles, ntiles, cols, kp, np, slots);
+}
 }  // namespace
 
 cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, int run,
                                     const FusedCol* cols, int kp, int np, double* const* slots, cudaStream_t st) {
   if (ntiles <= 0) return cudaSuccess;
   if (kp < 1 || kp > FMAXK + 1 || np < 1 || np > FMAXN + 1) return cudaErrorInvalidValue;
-  const cudaError_t le = run > 1 ? launch_fused<true>(groups, tiles, ntiles, cols, kp, np, slots, st)
-                                 : launch_fused<false>(groups, tiles, ntiles, cols, kp, np, slots, st);
+  const cudaError_t le = run == 0  ? launch_fused_warp(groups, tiles, ntiles, cols, kp, np, slots, st)
+                         : run > 1 ? launch_fused<true>(groups, tiles, ntiles, cols, kp, np, slots, st)
+                                   : launch_fused<false>(groups, tiles, ntiles, cols, kp, np, slots, st);
   if (le != cudaSuccess) return le;
   tnx_note_launch(1);
   return cudaGetLastError();

@@ -172,6 +172,7 @@ extern "C" tnx_status tnx_batch_create(tnx_ctx* ctx, int n, tnx_network* const* 
       for (int j = 0; j < i; ++j)
         if (nets[j] == nets[i]) fail(TNX_ERR_ARG, "a network appears twice in the batch");
       // one merged launch needs one tile width: networks in a batch keep 64-wide split tiles
+      // (and fuse their MPO steps however small)
       nets[i]->narrow_tiles = false;
       Plan* p = tnx_ensure_plan(nets[i]);
       if (i > 0 && (p->steps.size() != B->plans[0]->steps.size() || p->prec != B->prec))

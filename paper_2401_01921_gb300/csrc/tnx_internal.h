@@ -249,7 +249,7 @@ struct FusedTile {
   int32_t p0, q0, eP, eQ;   // the run's first tile: first row and extents
 };
 #define TNX_FUSED_ROWS 128   // rows (p, q) of a fused MPO-step tile at most (two threads per row)
-// run: the largest nt of the launch
+// run: the largest nt of the launch, or 0 for the kernel with a warp per tile (nt 1)
 cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, int run,
                                     const FusedCol* cols, int kp, int np, double* const* slots, cudaStream_t st);
 size_t tnx_fused_smem_bytes(int kp, int np);

@@ -845,18 +845,36 @@ std::vector<GemmTile> tnx_gemm_tiles(const std::vector<GemmGroup>& groups, const
   return tiles;
 }
 
+// The largest part of E cut into equal parts of at most `most`.
+static int even_part(int64_t E, int64_t most) {
+  const int64_t n = (E + most - 1) / most;
+  return (int)((E + n - 1) / n);
+}
+
 // Consecutive tiles of a band share a CTA, and its setup, while every SM keeps a few
 // CTAs: runs of at most 8 tiles, of one below six waves of the six CTAs an SM then
-// holds.  Tiles that leave a quarter of their rows empty stay alone (48 Hubbard
-// instances, 40 rows per tile: 178 us alone, 203 in runs, whose kernel holds five CTAs
-// per SM; Heisenberg at bond dimension 2048, 118 rows: 75 alone, 62 in runs of 5).
-std::vector<FusedTile> tnx_fused_runs(const std::vector<FusedTile>& bands, int& run) {
+// holds (Heisenberg at bond dimension 2048, 118 rows per tile: 75 us alone, 62 in runs of
+// 5).  Tiles that leave a quarter of their rows empty are not worth a run.  When there
+// are many they go to the kernel with a warp per tile (run 0): 48 Hubbard instances 1043
+// -> 898 us, one at bond dimension 601 191 -> 179.  Few of them stay one to a CTA, two
+// threads to a row, because a warp takes a tile's rows one after the other (Heisenberg at
+// 150, 186 tiles: an apply 70 against 79 us).
+std::vector<FusedTile> tnx_fused_runs(const std::vector<FusedTile>& all, int& run) {
+  std::vector<FusedTile> bands = all;
   int64_t total = 0, rows = 0;
   for (const FusedTile& b : bands) {
     total += b.nt;
     rows += (int64_t)b.EP * b.EQ;
   }
-  run = rows < 96 * total ? 1 : (int)std::min<int64_t>(8, std::max<int64_t>(1, total / (152 * 6 * 3)));
+  const bool warps = rows < 96 * total && total >= 16 * 152;
+  if (warps) {
+    for (FusedTile& b : bands) {
+      b.tQ = even_part(b.EQ, std::max(8, TNX_FUSED_ROWS / b.EP));
+      b.tP = even_part(b.EP, TNX_FUSED_ROWS / b.tQ);
+      b.nt = ((b.EP + b.tP - 1) / b.tP) * ((b.EQ + b.tQ - 1) / b.tQ);
+    }
+  }
+  run = warps ? 1 : (int)std::min<int64_t>(8, std::max<int64_t>(1, total / (152 * 6 * 3)));
   std::vector<FusedTile> out;
   for (FusedTile t : bands) {
     const int nt = t.nt;
@@ -871,6 +889,7 @@ std::vector<FusedTile> tnx_fused_runs(const std::vector<FusedTile>& bands, int& 
       out.push_back(t);
     }
   }
+  if (warps) run = 0;
   return out;
 }
 
@@ -1577,10 +1596,6 @@ bool fuse_skinny_step(Plan& p, size_t si, int ti, bool tA) {
       }
       return first;
     };
-    auto balance = [](int64_t E, int64_t Tmax) {
-      const int64_t n = (E + Tmax - 1) / Tmax;
-      return (E + n - 1) / n;
-    };
     int64_t total = 0, rows = 0;
     std::vector<FusedTile> tiles;   // one entry per band, all its tiles
     for (size_t b = 0; b < bands.size(); ++b) {
@@ -1589,7 +1604,7 @@ bool fuse_skinny_step(Plan& p, size_t si, int ti, bool tA) {
       const size_t gcol = add_cols(ta, B.h, s.ldK[B.g], true);
       int64_t scol = -1;   // write the rows to C
       if (ti >= 0) scol = (int64_t)add_cols(*tl, sidx[b] < 0 ? (size_t)-1 : (size_t)sidx[b], N, false);
-      const int tQ = (int)balance(B.EQ, 16), tP = (int)balance(B.EP, TNX_FUSED_ROWS / tQ);
+      const int tQ = even_part(B.EQ, std::max(16, TNX_FUSED_ROWS / B.EP)), tP = even_part(B.EP, TNX_FUSED_ROWS / tQ);
       const int64_t nt = (int64_t)((B.EP + tP - 1) / tP) * ((B.EQ + tQ - 1) / tQ);
       if (nt > INT32_MAX) return false;
       tiles.push_back(FusedTile{B.g, (int32_t)gcol, (int32_t)scol, (int32_t)B.row, B.EP, B.EQ, tP, tQ,
@@ -1597,9 +1612,11 @@ bool fuse_skinny_step(Plan& p, size_t si, int ti, bool tA) {
       total += nt;
       rows += (int64_t)B.EP * B.EQ;
     }
-    // many nearly empty tiles (small sectors) run faster unfused: plain
-    // relayouts pack small blocks, the skinny kernel fills 128-row tiles
-    if (!ok || total > INT32_MAX || cols.size() > INT32_MAX || rows < 32 * total) return false;
+    // a network of its own runs many nearly empty tiles (small sectors) faster unfused:
+    // plain relayouts pack small blocks, the skinny kernel fills 128-row tiles (Hubbard
+    // at 300: an apply 138 against 146 us).  In a batch the merged launch has the tiles
+    // to fill the chip (48 Hubbard instances: 898 against 976 us)
+    if (!ok || total > INT32_MAX || cols.size() > INT32_MAX || rows < (p.narrow_tiles ? 32 : 1) * total) return false;
     s.hFT = tiles;
     const std::vector<FusedTile> runs = tnx_fused_runs(tiles, s.frun);
     s.dFT = p.upload(runs);

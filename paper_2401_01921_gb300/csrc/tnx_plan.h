@@ -96,7 +96,7 @@ struct StepPlan {
   // skinny product and (when fscatter is set) the next step's relayout of C
   FusedTile* dFT = nullptr;
   FusedCol* dFC = nullptr;
-  int nftiles = 0, frun = 1;    // runs of tiles, and the most tiles in one
+  int nftiles = 0, frun = 1;    // runs of tiles, and the most tiles in one (0: a warp per tile)
   int fkp = 0, fnp = 0;
   bool fscatter = false;               // output stored into the next step's operand
   bool skipA = false, skipB = false;   // this step's operand relayout is done by a fused step
@@ -135,7 +135,7 @@ struct Plan {
   bool fin_folded = false;       // the last split product writes the output itself (fin unused)
   int prec = TNX_PREC_F64;
   int nslice = 6, beta = 7;
-  bool narrow_tiles = true;       // from the network (a batch needs the same tile width in every plan)
+  bool narrow_tiles = true;       // from the network (false in a batch: one split tile width, MPO steps always fused)
   int32_t* d_status = nullptr;
   std::string key;
   std::string order;
