@@ -4,28 +4,18 @@
 // two-site H_eff, Sec. 11) is a small FP64 product between two relayouts: its
 // operand A is gathered from the previous step's output blocks into the packed
 // K-major matrix, and its output C is immediately relaid into the next step's
-// packed operand.  Here one CTA takes a run of tiles of up to 128 rows (p, q) of one
-// row block of A_g.  It lists the nonzeros of every column of the packed B_g (the
-// MPO product is mostly zeros) and stages the columns' descriptors once, then per tile:
-//   1. every A element of the tile is read from its source block through the
-//      descriptor of its column (consecutive threads take consecutive q, the
-//      source blocks' contiguous leg) one tile ahead, and put into the A rows in
-//      shared memory;
-//   2. two threads form each output row (even and odd columns), with the same FMA
-//      chains as the unfused skinny kernel (bit-identical; a power-of-two first
-//      coefficient is applied on the integer units, tnx_first_term);
-//   3. every output element is stored through the descriptor of its column
-//      straight into the next step's packed operand (consecutive threads take
-//      consecutive p, that operand's contiguous leg), or the rows are written to
-//      C_g when no next step reads them through descriptors.
-// The packed A and the C rows never reach HBM when both ends are fused.  The
-// descriptors are precomputed by the planner from the two relayouts' bands.
+// packed operand.  Here a CTA or a warp takes a tile of up to 128 rows (p, q) of one row
+// block of A_g, lists the nonzeros of every column of the packed B_g (the MPO product is
+// mostly zeros), reads every A element of the tile from its source block through
+// the descriptor of its column, forms the output rows with the same FMA chains as the
+// unfused skinny kernel (bit-identical; a power-of-two first coefficient is applied on
+// the integer units, tnx_first_term), and stores every output element through the
+// descriptor of its column straight into the next step's packed operand, or writes the
+// rows to C_g when no next step reads them through descriptors.  The packed A and
+// the C rows never reach HBM when both ends are fused.  The descriptors are precomputed by
+// the planner from the two relayouts' bands.
 //
-// Instruction issue bounds it: a charge group has only a few columns, so with one
-// tile per CTA a thread formed 2.4 outputs on average and the warp issued 430
-// instructions for them, mostly the lists, descriptors and index setup, which a
-// run of tiles (tnx_fused_runs, tnx_network.cpp) shares: one apply of the Heisenberg
-// H_eff (ncu, cold) at bond dimension 2048 75 -> 62 us, 4096 244 -> 188 us.
+// Which of the kernels takes a launch is decided by tnx_fused_tiles (tnx_network.cpp).
 #include "tnx_internal.h"
 
 namespace {
@@ -52,23 +42,24 @@ struct FusedSmem {
 __device__ __forceinline__ int small_magic(int d) { return (65536 + d - 1) / d; }
 __device__ __forceinline__ int small_div(int t, int m) { return (t * m) >> 16; }
 
-// RUN false: every run of the launch is one tile (nothing is read ahead).
-template <bool RUN>
-__global__ void __launch_bounds__(FT, RUN ? 5 : 6) fused_skinny_kernel(const GemmGroup* __restrict__ groups,
-                                                          const FusedTile* __restrict__ tiles,
-                                                          const FusedCol* __restrict__ cols, int kp, int np,
-                                                          double* const* __restrict__ slots) {
+// One CTA per tile, two threads per row (even and odd columns): A goes to shared memory
+// along q, the source blocks' contiguous leg, and the output leaves it along p, the next
+// operand's.  For launches of few tiles, whose time is one tile's chain of loads and
+// products: 186 tiles (Heisenberg at bond dimension 150) 7.3 us against 9.7 with the
+// kernel below, 1372 tiles (512) 11.0 against 10.8 (ncu, cold).
+__global__ void __launch_bounds__(FT, 6) fused_skinny_kernel(const GemmGroup* __restrict__ groups,
+                                                             const FusedTile* __restrict__ tiles,
+                                                             const FusedCol* __restrict__ cols, int kp, int np,
+                                                             double* const* __restrict__ slots) {
   tnx_grid_dependency();
   extern __shared__ __align__(16) unsigned char dyn[];
   FusedSmem& S = *(FusedSmem*)dyn;
   double* sA = (double*)(dyn + sizeof(FusedSmem));   // [rows][kp]
   double* sC = sA + FR * kp;                         // [rows][np]
-  FusedCol* s_gc = (FusedCol*)(sC + FR * np);        // RUN: [W] A column descriptors
   const FusedTile T = tiles[blockIdx.x];
   const int tid = threadIdx.x, half = tid / FR, t = tid & (FR - 1);
-  const int W = T.W, N = T.N;
-  // column descriptors: A's by threads [0, W), the output's by [FR + FMAXN, FR + FMAXN + N)
-  if (RUN && tid < W) s_gc[tid] = cols[T.gcol + tid];
+  const int W = T.W, N = T.N, tq = T.eQ, tp = T.eP, rows = tp * tq;
+  // output column descriptors (threads [FR + FMAXN, FR + FMAXN + N))
   if (tid >= FR + FMAXN && tid - FR - FMAXN < N && T.scol >= 0) S.s_sc[tid - FR - FMAXN] = cols[T.scol + tid - FR - FMAXN];
   // B nonzeros (threads [FR, FR + N))
   const GemmGroup g = groups[T.group];
@@ -90,111 +81,80 @@ __global__ void __launch_bounds__(FT, RUN ? 5 : 6) fused_skinny_kernel(const Gem
     S.s_cnt[t] = c;
     S.s_p2[t] = c ? tnx_pow2_code(S.s_v[t][0]) : 0u;
   }
-  // the current tile: rows p in [p0, p0 + tp), q in [q0, q0 + tq)
-  const int nQ = RUN ? (T.EQ + T.tQ - 1) / T.tQ : 1;
-  const int mQ = RUN ? small_magic(T.tQ) : 0, mP = RUN ? small_magic(T.tP) : 0;
-  int p0 = T.p0, q0 = T.q0, tp = T.eP, tq = T.eQ;
-  auto over_q = [&](int r) { return !RUN ? r / tq : small_div(r, tq == T.tQ ? mQ : small_magic(tq)); };
-  double v[FMAXK / 2];
-  // this thread's entries of the tile's A: row t, q fastest; columns half, half + 2, ...
-  auto fetch = [&](const FusedCol* gc) {
-    if (t < tp * tq) {
-      const int p = over_q(t), q = t - p * tq;
-      const int P = p0 + p, Q = q0 + q;
+  // this thread's entries of A: row t, q fastest; columns half, half + 2, ...
+  if (t < rows) {
+    const int p = t / tq, q = t - p * tq;
+    const int P = T.p0 + p, Q = T.q0 + q;
 #pragma unroll
-      for (int j = 0; j < FMAXK / 2; ++j) {
-        const int c = half + 2 * j;
-        v[j] = 0.0;
-        if (c < W) {
-          const FusedCol d = gc[c];
-          if (d.ptr) v[j] = __ldg(d.ptr + (int64_t)P * d.sP + (int64_t)Q * d.sQ);
-        }
+    for (int j = 0; j < FMAXK / 2; ++j) {
+      const int c = half + 2 * j;
+      if (c < W) {
+        const FusedCol d = cols[T.gcol + c];
+        sA[t * kp + c] = d.ptr ? __ldg(d.ptr + (int64_t)P * d.sP + (int64_t)Q * d.sQ) : 0.0;
       }
     }
-  };
-  fetch(cols + T.gcol);   // beside the lists' and descriptors' own loads
-  int pt = RUN ? T.t0 / nQ : 0, qt = RUN ? T.t0 - pt * nQ : 0;
-  for (int i = 0; i < (RUN ? T.nt : 1); ++i) {
-    const int rows = tp * tq;
+  }
+  __syncthreads();
+  if (t < rows) {
+    const double* arow = sA + t * kp;
+    double* crow = sC + t * np;
+    for (int n = half; n < N; n += 2) {
+      double acc = 0.0;
+      const int c = S.s_cnt[n];
+      if (c > 0) acc = tnx_first_term(arow[S.s_k[n][0]], S.s_v[n][0], S.s_p2[n]);
+      for (int e = 1; e < c; ++e) acc = fma(arow[S.s_k[n][e]], S.s_v[n][e], acc);
+      crow[n] = acc;
+    }
+  }
+  __syncthreads();
+  if (T.scol >= 0) {
+    // scatter: p fastest (row r = p * tq + q in shared memory)
     if (t < rows) {
-#pragma unroll
-      for (int j = 0; j < FMAXK / 2; ++j) {
-        const int c = half + 2 * j;
-        if (c < W) sA[t * kp + c] = v[j];
+      const int q = t / tp, p = t - q * tp;
+      const int P = T.p0 + p, Q = T.q0 + q;
+      const double* crow = sC + (p * tq + q) * np;
+      for (int c = half; c < N; c += 2) {
+        const FusedCol d = S.s_sc[c];
+        if (d.ptr) d.ptr[(int64_t)P * d.sP + (int64_t)Q * d.sQ] = crow[c];
       }
     }
-    __syncthreads();
-    const int cp0 = p0, cq0 = q0, ctp = tp, ctq = tq;   // this tile, when p0 .. move on to the next
-    if (RUN && i + 1 < T.nt) {
-      if (++qt == nQ) {
-        qt = 0;
-        ++pt;
-      }
-      p0 = pt * T.tP;
-      q0 = qt * T.tQ;
-      tp = min(T.tP, T.EP - p0);
-      tq = min(T.tQ, T.EQ - q0);
-      fetch(s_gc);
+  } else {
+    // row (p, q) of the block is row row0 + p * EQ + q of C_g
+    double* C = slots[g.c_slot] + g.c_off;
+    for (int e = tid; e < rows * N; e += FT) {
+      const int r = e / N, n = e - r * N;
+      const int p = r / tq, q = r - p * tq;
+      const int64_t row = (int64_t)T.row0 + (int64_t)(T.p0 + p) * T.EQ + T.q0 + q;
+      C[row * g.ldc + n] = sC[r * np + n];
     }
-    if (t < rows) {
-      const double* arow = sA + t * kp;
-      double* crow = sC + t * np;
-      for (int n = half; n < N; n += 2) {
-        double acc = 0.0;
-        const int c = S.s_cnt[n];
-        if (c > 0) acc = tnx_first_term(arow[S.s_k[n][0]], S.s_v[n][0], S.s_p2[n]);
-        for (int e = 1; e < c; ++e) acc = fma(arow[S.s_k[n][e]], S.s_v[n][e], acc);
-        crow[n] = acc;
-      }
-    }
-    __syncthreads();
-    if (T.scol >= 0) {
-      // scatter: p fastest (row r = p * tq + q in shared memory)
-      if (t < rows) {
-        const int q = !RUN ? t / ctp : small_div(t, ctp == T.tP ? mP : small_magic(ctp)), p = t - q * ctp;
-        const int P = cp0 + p, Q = cq0 + q;
-        const double* crow = sC + (p * ctq + q) * np;
-        for (int c = half; c < N; c += 2) {
-          const FusedCol d = S.s_sc[c];
-          if (d.ptr) d.ptr[(int64_t)P * d.sP + (int64_t)Q * d.sQ] = crow[c];
-        }
-      }
-    } else {
-      // row (p, q) of the block is row row0 + p * EQ + q of C_g
-      double* C = slots[g.c_slot] + g.c_off;
-      for (int e = tid; e < rows * N; e += FT) {
-        const int r = e / N, n = e - r * N;
-        const int p = !RUN ? r / ctq : small_div(r, ctq == T.tQ ? mQ : small_magic(ctq)), q = r - p * ctq;
-        const int64_t row = (int64_t)T.row0 + (int64_t)(cp0 + p) * T.EQ + cq0 + q;
-        C[row * g.ldc + n] = sC[r * np + n];
-      }
-    }
-    // the next tile's A rows are written behind this tile's products (the barrier
-    // above), its C rows behind these reads of them (the next iteration's barriers)
   }
 }
 
-// The same step for small bands (charge blocks of a few rows), one warp per tile of at
-// most FR rows.  A row belongs to one lane: it gathers the row's A elements into a column
-// of the warp's shared memory that only it reads (the list of nonzeros picks elements by
-// number), forms the outputs and stores them at once.  Lanes walk q, then p, of tiles at
-// most 8 wide along q when the band allows it, so that 32-byte sectors are read whole
-// along q and written whole along p without a transposing stage.
+// The same step for many tiles, one warp per tile.  A row belongs to one lane (R rows to a
+// lane at once): it gathers the row's A elements into columns of the warp's shared memory
+// that only it reads (the list of nonzeros picks elements by number), forms the outputs and
+// stores them at once.  Lanes walk q, then p, of tiles at most 8 wide along q when
+// the band allows it, so that 32-byte sectors are read whole along q and written whole
+// along p without a transposing stage, and no barrier.
 //
-// A tile of 128 rows by 8 warps spends its time on the chain of loads before the
-// product (tile, group and descriptors, B and A), whatever the number of rows, and an SM
-// holds six; here it holds 28 chains.  Still bound by instruction issue and latency (about
-// 1000 warp instructions a tile, 40% of the issue slots, FP64 pipe 30%).  48 Hubbard
-// sites (75 thousand bands of 1 to 256 rows): 166 us for what took 178 (the instances
-// with 32 rows per tile and more) and 135 (relayouts and skinny products of the others)
-// before; the two MPO steps of one at bond dimension 601: 25 us for 41 (ncu, cold).
+// Bound by instruction issue and the latency of its loads (48 Hubbard sites: about 1000
+// warp instructions a tile, 40% of the issue slots, FP64 pipe 30%).  A CTA per tile spent
+// its time on the chain of loads before the product (tile, group and descriptors, B and
+// A), six tiles to an SM; here an SM holds 28 or more.  Two rows per lane share the
+// lists' and descriptors' reads where tiles are full (four took 156 us at 4096, one
+// 168); bands of a few rows take one.  One apply (ncu, cold), before -> now: Heisenberg
+// at bond dimension 2048 60 -> 42 us, 4096 182 -> 136, environment step at 2048
+// 46 -> 21.5; 48 Hubbard sites 178 us for the instances with 32 rows per tile and more and
+// 135 for the relayouts and skinny products of the others -> 165 for all; the two MPO
+// steps of one at 601 41 -> 25.
 constexpr int FW = 4;   // warps per CTA, each on its own tile
 
-__host__ __device__ constexpr size_t warp_smem(int kp, int np) {
-  return ((size_t)kp * 32 * 8 + (size_t)np * kp * 9 + (size_t)(kp + np) * sizeof(FusedCol) + (size_t)np * 8 + 15) / 16 *
+__host__ __device__ constexpr size_t warp_smem(int kp, int np, int R) {
+  return ((size_t)kp * 32 * R * 8 + (size_t)np * kp * 9 + (size_t)(kp + np) * sizeof(FusedCol) + (size_t)np * 8 + 15) / 16 *
          16;
 }
 
+template <int R>
 __global__ void __launch_bounds__(32 * FW, 8) fused_warp_kernel(const GemmGroup* __restrict__ groups,
                                                                 const FusedTile* __restrict__ tiles, int ntiles,
                                                                 const FusedCol* __restrict__ cols, int kp, int np,
@@ -204,10 +164,10 @@ __global__ void __launch_bounds__(32 * FW, 8) fused_warp_kernel(const GemmGroup*
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int ti = blockIdx.x * FW + wid;
   if (ti >= ntiles) return;
-  unsigned char* base = dyn + (size_t)wid * warp_smem(kp, np);
+  unsigned char* base = dyn + (size_t)wid * warp_smem(kp, np, R);
   FusedCol* s_d = (FusedCol*)base;                        // [kp] of A, [np] of the output
-  double* s_a = (double*)(s_d + kp + np) + lane;          // [kp][32]: this lane's column
-  double* s_v = (double*)(s_d + kp + np) + kp * 32;       // [np][kp] nonzeros
+  double* s_a = (double*)(s_d + kp + np) + lane;          // [kp][R][32]: this lane's columns
+  double* s_v = (double*)(s_d + kp + np) + kp * 32 * R;     // [np][kp] nonzeros
   int* s_cnt = (int*)(s_v + np * kp);                     // [np]
   uint32_t* s_p2 = (uint32_t*)(s_cnt + np);               // [np]
   unsigned char* s_k = (unsigned char*)(s_p2 + np);       // [np][kp]
@@ -238,35 +198,66 @@ __global__ void __launch_bounds__(32 * FW, 8) fused_warp_kernel(const GemmGroup*
   __syncwarp();
   double* C = T.scol >= 0 ? nullptr : slots[g.c_slot] + g.c_off;
   const int rows = T.eP * T.eQ, mq = small_magic(T.eQ);
-  for (int r = lane; r < rows; r += 32) {
-    const int p = small_div(r, mq), q = r - p * T.eQ;
-    const int64_t P = T.p0 + p, Q = T.q0 + q;
+  for (int r = lane; r < rows; r += 32 * R) {
+    int64_t P[R], Q[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int x = min(r + 32 * i, rows - 1), p = small_div(x, mq);
+      P[i] = T.p0 + p;
+      Q[i] = T.q0 + x - p * T.eQ;
+    }
     for (int c0 = 0; c0 < W; c0 += 4) {
-      double v[4];
+      double v[4][R];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        v[c] = 0.0;
+#pragma unroll
+        for (int i = 0; i < R; ++i) v[c][i] = 0.0;
         if (c0 + c < W) {
           const FusedCol d = s_d[c0 + c];
-          if (d.ptr) v[c] = __ldg(d.ptr + P * d.sP + Q * d.sQ);
+          if (d.ptr) {
+#pragma unroll
+            for (int i = 0; i < R; ++i) v[c][i] = __ldg(d.ptr + P[i] * d.sP + Q[i] * d.sQ);
+          }
         }
       }
 #pragma unroll
       for (int c = 0; c < 4; ++c)
-        if (c0 + c < W) s_a[(c0 + c) * 32] = v[c];
+        if (c0 + c < W) {
+#pragma unroll
+          for (int i = 0; i < R; ++i) s_a[((c0 + c) * R + i) * 32] = v[c][i];
+        }
     }
     for (int n = 0; n < N; ++n) {
-      double acc = 0.0;
+      double acc[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) acc[i] = 0.0;
       const int c = s_cnt[n];
       const double* bv = s_v + n * kp;
       const unsigned char* bk = s_k + n * kp;
-      if (c > 0) acc = tnx_first_term(s_a[bk[0] * 32], bv[0], s_p2[n]);
-      for (int e = 1; e < c; ++e) acc = fma(s_a[bk[e] * 32], bv[e], acc);
+      if (c > 0) {
+        const double* a = s_a + bk[0] * (32 * R);
+        const double x = bv[0];
+        const uint32_t code = s_p2[n];
+#pragma unroll
+        for (int i = 0; i < R; ++i) acc[i] = tnx_first_term(a[i * 32], x, code);
+      }
+      for (int e = 1; e < c; ++e) {
+        const double* a = s_a + bk[e] * (32 * R);
+        const double x = bv[e];
+#pragma unroll
+        for (int i = 0; i < R; ++i) acc[i] = fma(a[i * 32], x, acc[i]);
+      }
       if (C) {
-        C[((int64_t)T.row0 + P * T.EQ + Q) * g.ldc + n] = acc;
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+          if (r + 32 * i < rows) C[((int64_t)T.row0 + P[i] * T.EQ + Q[i]) * g.ldc + n] = acc[i];
       } else {
         const FusedCol d = s_d[kp + n];
-        if (d.ptr) d.ptr[P * d.sP + Q * d.sQ] = acc;
+        if (d.ptr) {
+#pragma unroll
+          for (int i = 0; i < R; ++i)
+            if (r + 32 * i < rows) d.ptr[P[i] * d.sP + Q[i] * d.sQ] = acc[i];
+        }
       }
     }
   }
@@ -277,7 +268,6 @@ __global__ void __launch_bounds__(32 * FW, 8) fused_warp_kernel(const GemmGroup*
 size_t tnx_fused_smem_bytes(int kp, int np) { return sizeof(FusedSmem) + (size_t)FR * (kp + np) * sizeof(double); }
 
 namespace {
-template <bool RUN>
 cudaError_t launch_fused(const GemmGroup* groups, const FusedTile* tiles, int ntiles, const FusedCol* cols, int kp,
                          int np, double* const* slots, cudaStream_t st) {
   static int attr_dev = -1;   // the opt-in is per device
@@ -285,14 +275,16 @@ cudaError_t launch_fused(const GemmGroup* groups, const FusedTile* tiles, int nt
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (attr_dev != dev) {
-    e = cudaFuncSetAttribute(fused_skinny_kernel<RUN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(tnx_fused_smem_bytes(FMAXK + 1, FMAXN + 1) + FMAXK * sizeof(FusedCol)));
+    e = cudaFuncSetAttribute(fused_skinny_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)tnx_fused_smem_bytes(FMAXK + 1, FMAXN + 1));
     if (e != cudaSuccess) return e;
     attr_dev = dev;
   }
-  const size_t smem = tnx_fused_smem_bytes(kp, np) + (RUN ? FMAXK * sizeof(FusedCol) : 0);
-  return tnx_launch(fused_skinny_kernel<RUN>, dim3(ntiles), dim3(FT), smem, st, groups, tiles, cols, kp, np, slots);
+  return tnx_launch(fused_skinny_kernel, dim3(ntiles), dim3(FT), tnx_fused_smem_bytes(kp, np), st, groups, tiles, cols,
+                    kp, np, slots);
 }
+
+template <int R>
 cudaError_t launch_fused_warp(const GemmGroup* groups, const FusedTile* tiles, int ntiles, const FusedCol* cols, int kp,
                               int np, double* const* slots, cudaStream_t st) {
   static int attr_dev = -1;
@@ -300,23 +292,23 @@ cudaError_t launch_fused_warp(const GemmGroup* groups, const FusedTile* tiles, i
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (attr_dev != dev) {
-    e = cudaFuncSetAttribute(fused_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(FW * warp_smem(FMAXK + 1, FMAXN + 1)));
+    e = cudaFuncSetAttribute(fused_warp_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(FW * warp_smem(FMAXK + 1, FMAXN + 1, R)));
     if (e != cudaSuccess) return e;
     attr_dev = dev;
   }
-  return tnx_launch(fused_warp_kernel, dim3((ntiles + FW - 1) / FW), dim3(32 * FW), FW * warp_smem(kp, np), st, groups,
-                    tiles, ntiles, cols, kp, np, slots);
+  return tnx_launch(fused_warp_kernel<R>, dim3((ntiles + FW - 1) / FW), dim3(32 * FW), FW * warp_smem(kp, np, R), st,
+                    groups, tiles, ntiles, cols, kp, np, slots);
 }
 }  // namespace
 
-cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, int run,
+cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, int lane_rows,
                                     const FusedCol* cols, int kp, int np, double* const* slots, cudaStream_t st) {
   if (ntiles <= 0) return cudaSuccess;
   if (kp < 1 || kp > FMAXK + 1 || np < 1 || np > FMAXN + 1) return cudaErrorInvalidValue;
-  const cudaError_t le = run == 0  ? launch_fused_warp(groups, tiles, ntiles, cols, kp, np, slots, st)
-                         : run > 1 ? launch_fused<true>(groups, tiles, ntiles, cols, kp, np, slots, st)
-                                   : launch_fused<false>(groups, tiles, ntiles, cols, kp, np, slots, st);
+  const cudaError_t le = lane_rows == 0   ? launch_fused(groups, tiles, ntiles, cols, kp, np, slots, st)
+                         : lane_rows == 1 ? launch_fused_warp<1>(groups, tiles, ntiles, cols, kp, np, slots, st)
+                                          : launch_fused_warp<2>(groups, tiles, ntiles, cols, kp, np, slots, st);
   if (le != cudaSuccess) return le;
   tnx_note_launch(1);
   return cudaGetLastError();

@@ -41,7 +41,7 @@ struct BStep {
   // column descriptors (the other instances run copies and skinny tiles)
   FusedTile* dFT = nullptr;
   FusedCol* dFC = nullptr;
-  int nft = 0, frun = 1, fkp = 0, fnp = 0;
+  int nft = 0, frows = 0, fkp = 0, fnp = 0;
 };
 
 struct tnx_batch {
@@ -109,7 +109,7 @@ void enqueue_batch(tnx_batch& B, cudaStream_t st) {
     }
     if (s.nft) {
       ProfScope ps(c, st, TNX_KC_SKINNY, s.flops_skinny);
-      CUDA_CHECK(tnx_launch_fused_skinny(s.dG, s.dFT, s.nft, s.frun, s.dFC, s.fkp, s.fnp, B.d_slots, st));
+      CUDA_CHECK(tnx_launch_fused_skinny(s.dG, s.dFT, s.nft, s.frows, s.dFC, s.fkp, s.fnp, B.d_slots, st));
     }
     if (s.nts) {
       ProfScope ps(c, st, TNX_KC_SKINNY, s.flops_skinny);
@@ -277,11 +277,11 @@ extern "C" tnx_status tnx_batch_create(tnx_ctx* ctx, int n, tnx_network* const* 
       bs.dTs = B->upload(ts);
       bs.nts = (int)ts.size();
       if (!ft.empty()) {
-        const std::vector<FusedTile> runs = tnx_fused_runs(ft, bs.frun);
-        if (runs.size() > (size_t)INT32_MAX) fail(TNX_ERR_UNSUPPORTED, "too many fused tiles in one batch");
-        bs.dFT = B->upload(runs);
+        const std::vector<FusedTile> cut = tnx_fused_tiles(ft, bs.frows);
+        if (cut.size() > (size_t)INT32_MAX) fail(TNX_ERR_UNSUPPORTED, "too many fused tiles in one batch");
+        bs.dFT = B->upload(cut);
         bs.dFC = B->upload(fc);
-        bs.nft = (int)runs.size();
+        bs.nft = (int)cut.size();
       }
       if (split) {
         // longest K first, so a persistent grid ends with short tiles

@@ -226,10 +226,9 @@ cudaError_t tnx_launch_copy(const CopyTask* tasks, const int4* chunks, int nchun
 cudaError_t tnx_launch_copy_scaled(const CopyTask* tasks, const int4* chunks, int nchunks, double* const* slots,
                                    const double* src, double* vdst, int64_t vn, int full, const double* inv,
                                    const int32_t* state, cudaStream_t st);
-// Fused skinny step (k_fused.cu): one CTA per run of tiles of one row block of A_g
-// (the rows a destination band of the step's relayout fills): EP x EQ rows (p, q),
-// cut into tiles of tP x tQ <= TNX_FUSED_ROWS rows, numbered along q first; a run
-// is the nt tiles from t0 on.  Column c < W (= ldK of the group) of those rows is
+// Fused skinny step (k_fused.cu), one CTA or warp per tile: rows p0 .. p0 + eP, q0 .. q0 +
+// eQ, TNX_FUSED_ROWS at most, of one row block of A_g (the EP x EQ rows (p, q) that a
+// destination band of the step's relayout fills).  Column c < W (= ldK of the group) is
 // described by FusedCol gcol + c: the A element of row (p, q) lies at ptr + p * sP + q *
 // sQ (ptr null: a structural zero).  The rows are multiplied by the packed B_g (K <=
 // 16, N <= 64) in FP64, and output column c < N of row (p, q) is stored through
@@ -245,12 +244,12 @@ struct FusedCol {
 struct FusedTile {
   int32_t group, gcol, scol, row0;
   int32_t EP, EQ, tP, tQ;
-  int32_t W, N, t0, nt;
-  int32_t p0, q0, eP, eQ;   // the run's first tile: first row and extents
+  int32_t W, N, nt, pad0;   // nt: of a band's entry, its tiles of tP x tQ rows
+  int32_t p0, q0, eP, eQ;   // first row and extents of a tile
 };
 #define TNX_FUSED_ROWS 128   // rows (p, q) of a fused MPO-step tile at most (two threads per row)
-// run: the largest nt of the launch, or 0 for the kernel with a warp per tile (nt 1)
-cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, int run,
+// lane_rows: 0 a CTA per tile, 1 or 2 a warp per tile with that many rows to a lane
+cudaError_t tnx_launch_fused_skinny(const GemmGroup* groups, const FusedTile* tiles, int ntiles, int lane_rows,
                                     const FusedCol* cols, int kp, int np, double* const* slots, cudaStream_t st);
 size_t tnx_fused_smem_bytes(int kp, int np);
 // edge: rows and columns of a tile (8 or 16; FP32: 64)

@@ -851,45 +851,33 @@ static int even_part(int64_t E, int64_t most) {
   return (int)((E + n - 1) / n);
 }
 
-// Consecutive tiles of a band share a CTA, and its setup, while every SM keeps a few
-// CTAs: runs of at most 8 tiles, of one below six waves of the six CTAs an SM then
-// holds (Heisenberg at bond dimension 2048, 118 rows per tile: 75 us alone, 62 in runs of
-// 5).  Tiles that leave a quarter of their rows empty are not worth a run.  When there
-// are many they go to the kernel with a warp per tile (run 0): 48 Hubbard instances 1043
-// -> 898 us, one at bond dimension 601 191 -> 179.  Few of them stay one to a CTA, two
-// threads to a row, because a warp takes a tile's rows one after the other (Heisenberg at
-// 150, 186 tiles: an apply 70 against 79 us).
-std::vector<FusedTile> tnx_fused_runs(const std::vector<FusedTile>& all, int& run) {
-  std::vector<FusedTile> bands = all;
+// The tiles of a fused launch and the kernel that takes it: lane_rows 0 a CTA per tile,
+// else a warp per tile with that many rows to a lane.  From 16 tiles per SM on there are
+// warps enough (ncu, cold, CTA | warp: Heisenberg at bond dimension 512, 1372 tiles, 11.0 |
+// 10.8 us, 777, 2714 tiles, 18.0 | 16.1, 150, 186 tiles, 7.3 | 9.7).  Two rows to a lane
+// when three quarters of a 128-row tile exist (Heisenberg: 118 rows on average at 2048;
+// Hubbard batches: 19).
+std::vector<FusedTile> tnx_fused_tiles(const std::vector<FusedTile>& bands, int& lane_rows) {
   int64_t total = 0, rows = 0;
   for (const FusedTile& b : bands) {
     total += b.nt;
     rows += (int64_t)b.EP * b.EQ;
   }
-  const bool warps = rows < 96 * total && total >= 16 * 152;
-  if (warps) {
-    for (FusedTile& b : bands) {
-      b.tQ = even_part(b.EQ, std::max(8, TNX_FUSED_ROWS / b.EP));
-      b.tP = even_part(b.EP, TNX_FUSED_ROWS / b.tQ);
-      b.nt = ((b.EP + b.tP - 1) / b.tP) * ((b.EQ + b.tQ - 1) / b.tQ);
-    }
-  }
-  run = warps ? 1 : (int)std::min<int64_t>(8, std::max<int64_t>(1, total / (152 * 6 * 3)));
+  lane_rows = total < 16 * 152 ? 0 : rows < 96 * total ? 1 : 2;
   std::vector<FusedTile> out;
   for (FusedTile t : bands) {
-    const int nt = t.nt;
-    for (int t0 = 0; t0 < nt; t0 += run) {
-      t.t0 = t0;
-      t.nt = std::min(run, nt - t0);
-      const int nQ = (t.EQ + t.tQ - 1) / t.tQ;
-      t.p0 = t0 / nQ * t.tP;
-      t.q0 = t0 % nQ * t.tQ;
-      t.eP = std::min(t.tP, t.EP - t.p0);
-      t.eQ = std::min(t.tQ, t.EQ - t.q0);
-      out.push_back(t);
+    if (lane_rows != 0) {
+      t.tQ = even_part(t.EQ, std::max(8, TNX_FUSED_ROWS / t.EP));
+      t.tP = even_part(t.EP, TNX_FUSED_ROWS / t.tQ);
     }
+    t.nt = 1;
+    for (t.p0 = 0; t.p0 < t.EP; t.p0 += t.tP)
+      for (t.q0 = 0; t.q0 < t.EQ; t.q0 += t.tQ) {
+        t.eP = std::min(t.tP, t.EP - t.p0);
+        t.eQ = std::min(t.tQ, t.EQ - t.q0);
+        out.push_back(t);
+      }
   }
-  if (warps) run = 0;
   return out;
 }
 
@@ -1608,7 +1596,7 @@ bool fuse_skinny_step(Plan& p, size_t si, int ti, bool tA) {
       const int64_t nt = (int64_t)((B.EP + tP - 1) / tP) * ((B.EQ + tQ - 1) / tQ);
       if (nt > INT32_MAX) return false;
       tiles.push_back(FusedTile{B.g, (int32_t)gcol, (int32_t)scol, (int32_t)B.row, B.EP, B.EQ, tP, tQ,
-                                (int32_t)s.ldK[B.g], (int32_t)N, 0, (int32_t)nt, 0, 0, 0, 0});
+                                (int32_t)s.ldK[B.g], (int32_t)N, (int32_t)nt, 0, 0, 0, 0, 0});
       total += nt;
       rows += (int64_t)B.EP * B.EQ;
     }
@@ -1618,9 +1606,10 @@ bool fuse_skinny_step(Plan& p, size_t si, int ti, bool tA) {
     // to fill the chip (48 Hubbard instances: 898 against 976 us)
     if (!ok || total > INT32_MAX || cols.size() > INT32_MAX || rows < (p.narrow_tiles ? 32 : 1) * total) return false;
     s.hFT = tiles;
-    const std::vector<FusedTile> runs = tnx_fused_runs(tiles, s.frun);
-    s.dFT = p.upload(runs);
-    s.nftiles = (int)runs.size();
+    const std::vector<FusedTile> cut = tnx_fused_tiles(tiles, s.frows);
+    if (cut.size() > (size_t)INT32_MAX) fail(TNX_ERR_UNSUPPORTED, "too many fused tiles");
+    s.dFT = p.upload(cut);
+    s.nftiles = (int)cut.size();
     s.hFC = cols;
     s.dFC = p.upload(cols);
     s.fkp = (int)(maxld | 1);
@@ -1853,7 +1842,7 @@ void enqueue_plan(Plan& p, cudaStream_t st, uint64_t fixed = 0, int skip_slot = 
     }
     if (s.nftiles) {
       ProfScope ps(c, st, TNX_KC_SKINNY, s.flops_skinny);
-      CUDA_CHECK(tnx_launch_fused_skinny(s.dG, s.dFT, s.nftiles, s.frun, s.dFC, s.fkp, s.fnp, p.d_slots, st));
+      CUDA_CHECK(tnx_launch_fused_skinny(s.dG, s.dFT, s.nftiles, s.frows, s.dFC, s.fkp, s.fnp, p.d_slots, st));
     } else if (s.nstiles_skinny) {
       ProfScope ps(c, st, TNX_KC_SKINNY, s.flops_skinny);
       CUDA_CHECK(tnx_launch_gemm_skinny(s.dG, s.dTs, s.nstiles_skinny, p.d_slots, st));

@@ -96,11 +96,11 @@ struct StepPlan {
   // skinny product and (when fscatter is set) the next step's relayout of C
   FusedTile* dFT = nullptr;
   FusedCol* dFC = nullptr;
-  int nftiles = 0, frun = 1;    // runs of tiles, and the most tiles in one (0: a warp per tile)
+  int nftiles = 0, frows = 0;   // tiles, and lane_rows of tnx_fused_tiles
   int fkp = 0, fnp = 0;
   bool fscatter = false;               // output stored into the next step's operand
   bool skipA = false, skipB = false;   // this step's operand relayout is done by a fused step
-  std::vector<FusedTile> hFT;   // one entry per band, all its tiles (t0 = 0)
+  std::vector<FusedTile> hFT;   // one entry per band, nt its tiles for a CTA each
   std::vector<FusedCol> hFC;
 };
 
@@ -244,7 +244,7 @@ std::vector<int2> tnx_tf32_schedule(std::vector<SliceJob>& jobs);
 int tnx_f64_edge(const std::vector<GemmGroup>& groups, const std::vector<int>& which);
 std::vector<GemmTile> tnx_gemm_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which, int edge);
 // runs of fused-step tiles from entries that hold whole bands; run gets the most tiles in one
-std::vector<FusedTile> tnx_fused_runs(const std::vector<FusedTile>& bands, int& run);
+std::vector<FusedTile> tnx_fused_tiles(const std::vector<FusedTile>& bands, int& lane_rows);
 std::vector<GemmTile> tnx_skinny_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which);
 
 // relayout chunks (tnx_network.cpp)

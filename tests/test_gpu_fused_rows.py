@@ -1,6 +1,6 @@
-"""GPU: the fused MPO step with runs of tiles (several tiles of a band per CTA, the last run shorter, ragged
-last tiles): FP64 applies of the Heisenberg H_eff large enough for runs of 2 and 3 tiles, against the
-oracle, in the tree that scatters into the last operand and the one that writes the rows out."""
+"""GPU: the fused MPO step on full tiles, two rows to a lane (ragged last tiles, an odd number of rows):
+FP64 applies of the Heisenberg H_eff, against the oracle, in the tree that scatters into the last
+operand and the one that writes the rows out."""
 import pytest
 
 import tnx_inputs as I
@@ -19,7 +19,7 @@ def ctx():
 
 
 @pytest.mark.parametrize("chi,n,order", [(1301, 33, "(L,((psi,R),(W1,W2)))"), (1597, 35, "(((psi,R),(W1,W2)),L)")])
-def test_apply_with_runs_of_tiles(ctx, chi, n, order):
+def test_apply_with_full_tiles(ctx, chi, n, order):
     wl = I.heisenberg_workload(chi, n)
     net, T, B = lib_heff(ctx, wl, order=order)
     onet, _ = oracle_heff(wl, order=order)

@@ -8,7 +8,7 @@ import paper_2401_01921_gb300 as tnx
 import tnx_inputs as I
 
 from gpu_harness import lib_heff, oracle_heff, rel_fro
-from test_gpu_fused_runs import ctx  # noqa: F401 (a fixture)
+from test_gpu_fused_rows import ctx  # noqa: F401 (a fixture)
 
 pytestmark = pytest.mark.gpu
 
