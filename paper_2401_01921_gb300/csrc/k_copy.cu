@@ -24,6 +24,14 @@
 // an index is split over the legs with multiply-high divisions by the leg
 // extents (constants the planner precomputes) instead of hardware integer
 // divisions.
+//
+// Bound by instruction issue and latency, not by HBM: 400 instructions per warp of a
+// transposing tile went mostly into splitting indices.  A tile's row indices are now split
+// once per warp (the loads take their rows' offsets by shuffles, the stores' row is the
+// lane's own), no division is spent on the slowest leg, and a packed chunk's starts are
+// prefix sums by a warp: the six relayouts of one apply at bond dimension 4096 145 -> 95
+// us, the five of an environment step at 2048 63 -> 46, the seven of a batch of 48 Hubbard
+// sites 112 -> 90 (ncu, cold).
 #include <algorithm>
 
 #include "tnx_band.cuh"
@@ -50,14 +58,16 @@ __device__ void copy_transpose(const CopyTask& t, int tile, double* const* __res
   const int nrows = (int)(t.nelem / ncols);
   const int nct = (ncols + 31) >> 5;
   const int r0 = (tile / nct) << 5, c0 = (tile % nct) << 5;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const double* src = SCALED ? src_base + t.src_off : (t.src_slot >= 0 ? slots[t.src_slot] + t.src_off : nullptr);
   double* dst = slots[t.dst_slot] + t.dst_off;
-  // row index -> (source offset, destination offset) over the legs other than S
-  auto bases = [&](int row, int& so, int& dof) {
-    so = 0;
-    dof = 0;
-    for (int l = r - 1; l >= 0; --l) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // source and destination offsets of row r0 + lane over the legs other than S: once per
+  // warp and tile, the loads take those of their rows by shuffles
+  int so = 0, dof = 0;
+  {
+    int row = min(r0 + lane, nrows - 1);
+    const int first = S == 0 ? 1 : 0;   // the slowest of the other legs: what is left is its index
+    for (int l = r - 1; l > first; --l) {
       if (l == S) continue;
       const int q = fdiv(row, t.magic[l], t.shift[l]);
       const int rem = row - q * t.shape[l];
@@ -65,33 +75,34 @@ __device__ void copy_transpose(const CopyTask& t, int tile, double* const* __res
       so += rem * t.sstride[l];
       dof += rem * t.dstride[l];
     }
-  };
-  const int c = c0 + lane;
+    if (first < r && first != S) {
+      so += row * t.sstride[first];
+      dof += row * t.dstride[first];
+    }
+  }
+  const int c = c0 + lane, sc = c * t.sstride[S];
+  double x[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int rr = wid + 8 * i, row = r0 + rr;
-    if (row < nrows && c < ncols) {
-      int so, dof;
-      bases(row, so, dof);
-      const double x = src ? __ldg(src + so + c * t.sstride[S]) : 0.0;
+    const int rr = wid + 8 * i, o = __shfl_sync(0xffffffffu, so, rr) + sc;
+    x[i] = 0.0;
+    if (r0 + rr < nrows && c < ncols) {
+      if (src) x[i] = __ldg(src + o);
       if (SCALED) {
-        const double y = x * scale;
-        sm[rr][lane] = y;
-        if (vdst_base) vdst_base[t.src_off + so + c * t.sstride[S]] = y;
-      } else {
-        sm[rr][lane] = x;
+        x[i] *= scale;
+        if (vdst_base) vdst_base[t.src_off + o] = x[i];
       }
     }
   }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) sm[wid + 8 * i][lane] = x[i];
   __syncthreads();
-  const int row = r0 + lane;
-  if (row < nrows) {
-    int so, dof;
-    bases(row, so, dof);
+  if (r0 + lane < nrows) {
+    const int ds = t.dstride[S];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int cc = wid + 8 * i, col = c0 + cc;
-      if (col < ncols) dst[dof + col * t.dstride[S]] = sm[lane][cc];
+      if (col < ncols) dst[dof + col * ds] = sm[lane][cc];
     }
   }
 }
@@ -177,15 +188,16 @@ __device__ void copy_band(const CopyTask* __restrict__ tasks, int h, int tile, d
 __device__ __forceinline__ void offsets(const CopyTask& t, int i, int& so, int& dof) {
   so = 0;
   dof = 0;
-#pragma unroll
-  for (int l = TNX_MAXR - 1; l >= 0; --l) {
-    if (l < t.rank) {
-      const int q = fdiv(i, t.magic[l], t.shift[l]);
-      const int rem = i - q * t.shape[l];
-      i = q;
-      so += rem * t.sstride[l];
-      dof += rem * t.dstride[l];
-    }
+  for (int l = t.rank - 1; l > 0; --l) {
+    const int q = fdiv(i, t.magic[l], t.shift[l]);
+    const int rem = i - q * t.shape[l];
+    i = q;
+    so += rem * t.sstride[l];
+    dof += rem * t.dstride[l];
+  }
+  if (t.rank > 0) {   // the slowest leg's index is what is left
+    so += i * t.sstride[0];
+    dof += i * t.dstride[0];
   }
 }
 
@@ -313,13 +325,19 @@ __global__ void __launch_bounds__(CT) copy_kernel(const CopyTask* __restrict__ t
     for (int i = threadIdx.x; i < words; i += CT) sm[i] = g[i];
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int k = 0; k < nt; ++k) {
-      sstart[k] = acc;
-      acc += (int)st[k].nelem;
+  if (threadIdx.x < 32) {   // starts: prefix sums by a warp, two tasks per lane
+    static_assert(TNX_COPY_PACK <= 64, "two tasks per lane");
+    const int k = 2 * threadIdx.x;
+    const int n0 = k < nt ? (int)st[k].nelem : 0, n1 = k + 1 < nt ? (int)st[k + 1].nelem : 0;
+    int end = n0 + n1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(0xffffffffu, end, o);
+      if ((int)threadIdx.x >= o) end += up;
     }
-    sstart[nt] = acc;
+    if (k < nt) sstart[k] = end - n0 - n1;
+    if (k + 1 < nt) sstart[k + 1] = end - n1;
+    if (threadIdx.x == 31) sstart[nt] = end;
   }
   __syncthreads();
   for (int e = threadIdx.x; e < ch.w; e += CT) {
