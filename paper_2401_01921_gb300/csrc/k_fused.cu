@@ -85,13 +85,20 @@ __global__ void __launch_bounds__(FT, 6) fused_skinny_kernel(const GemmGroup* __
   if (t < rows) {
     const int p = t / tq, q = t - p * tq;
     const int P = T.p0 + p, Q = T.q0 + q;
+    double v[FMAXK / 2];   // all loads in flight before the first store
 #pragma unroll
     for (int j = 0; j < FMAXK / 2; ++j) {
       const int c = half + 2 * j;
+      v[j] = 0.0;
       if (c < W) {
         const FusedCol d = cols[T.gcol + c];
-        sA[t * kp + c] = d.ptr ? __ldg(d.ptr + (int64_t)P * d.sP + (int64_t)Q * d.sQ) : 0.0;
+        if (d.ptr) v[j] = __ldg(d.ptr + (int64_t)P * d.sP + (int64_t)Q * d.sQ);
       }
+    }
+#pragma unroll
+    for (int j = 0; j < FMAXK / 2; ++j) {
+      const int c = half + 2 * j;
+      if (c < W) sA[t * kp + c] = v[j];
     }
   }
   __syncthreads();
