@@ -882,7 +882,11 @@ std::vector<FusedTile> tnx_fused_tiles(const std::vector<FusedTile>& bands, int&
 }
 
 // Columns per skinny tile: 64, or fewer while that leaves SMs without a few tiles
-// (each tile stages its rows of A again).
+// (each tile stages its rows of A again), and in the groups whose tiles would be longer
+// than a sixth of an SM's share of the launch; the longest tiles first.  A batch of 48
+// Hubbard sites (3685 tiles of 64 columns, the longest 34 us, in group order): FP64 pipe
+// busy 84% of the time an SM had a tile, 51% of the launch; 162 -> 102 us (ncu,
+// cold).
 std::vector<GemmTile> tnx_skinny_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which) {
   int width = 64;
   auto count = [&](int w) {
@@ -891,11 +895,24 @@ std::vector<GemmTile> tnx_skinny_tiles(const std::vector<GemmGroup>& groups, con
     return n;
   };
   while (width > 8 && count(width) < 4 * 152) width /= 2;
-  std::vector<GemmTile> tiles;
-  for (int g : which)
-    for (int m0 = 0; m0 < groups[g].M; m0 += 128)
-      for (int n0 = 0; n0 < groups[g].N; n0 += width) tiles.push_back(GemmTile{g, m0, n0, width});
-  return tiles;
+  // FP64 instructions of a tile's warps, its rows by w columns
+  auto cost = [&](const GemmGroup& g, int rows, int w) { return (int64_t)((rows + 31) / 32) * w * g.K; };
+  int64_t all = 0;
+  for (int g : which) all += cost(groups[g], groups[g].M, groups[g].N);
+  const int64_t most = all / (152 * 6);
+  std::vector<std::pair<int64_t, GemmTile>> tiles;
+  for (int g : which) {
+    const GemmGroup& G = groups[g];
+    int w = width;
+    while (w > 8 && cost(G, std::min(G.M, 128), std::min(G.N, w)) > most) w /= 2;
+    for (int m0 = 0; m0 < G.M; m0 += 128)
+      for (int n0 = 0; n0 < G.N; n0 += w)
+        tiles.push_back({cost(G, std::min(128, G.M - m0), std::min(w, G.N - n0)), GemmTile{g, m0, n0, w}});
+  }
+  std::stable_sort(tiles.begin(), tiles.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  std::vector<GemmTile> out;
+  for (const auto& t : tiles) out.push_back(t.second);
+  return out;
 }
 
 // Chunks of the relayout kernel (see k_copy.cu): large tasks cut into pieces of
