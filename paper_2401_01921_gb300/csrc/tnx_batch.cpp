@@ -36,6 +36,7 @@ struct BStep {
   GemmTile* dST = nullptr;
   int nst = 0;
   int kmax = 0;                 // largest K of the merged split groups
+  int grid = 0;                 // CTAs that dST is scheduled for
   double flops = 0, flops_skinny = 0;
   // the fused MPO steps of the instances that fuse this step: merged tiles and
   // column descriptors (the other instances run copies and skinny tiles)
@@ -56,7 +57,7 @@ struct tnx_batch {
   double** d_slots = nullptr;
   std::vector<BStep> steps;
   TaskList fin;
-  int split_grid = 0;
+  int split_grid = 0;         // CTAs of the split GEMMs (autotune); 0: each step's schedule
   std::unique_ptr<GraphRec> graph;
 
   template <class T>
@@ -125,7 +126,8 @@ void enqueue_batch(tnx_batch& B, cudaStream_t st) {
         CUDA_CHECK(tnx_launch_tf32_rows(s.jobs.d, s.jobs.items, s.jobs.nitems, B.d_slots, st));
       }
       ProfScope ps(c, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
-      CUDA_CHECK(tnx_launch_gemm_tf32(s.dSG, s.dST, s.nst, B.d_slots, c->d_status, st, B.split_grid, 64));
+      CUDA_CHECK(tnx_launch_gemm_tf32(s.dSG, s.dST, s.nst, B.d_slots, c->d_status, st,
+                                      B.split_grid ? B.split_grid : s.grid, 64));
     } else {
       if (s.jobs.n) {
         ProfScope ps(c, st, TNX_KC_SLICE, (double)s.jobs.elems * (16.0 + 2.0 * B.nslice));
@@ -134,7 +136,7 @@ void enqueue_batch(tnx_batch& B, cudaStream_t st) {
       }
       ProfScope ps(c, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
       CUDA_CHECK(tnx_launch_gemm_split(s.dSG, s.dST, s.nst, B.nslice, B.beta, f16, B.d_slots, c->d_status, st,
-                                       B.split_grid, 64, s.kmax <= 160 ? 2 : 0));
+                                       B.split_grid ? B.split_grid : s.grid, 64, s.kmax <= 160 ? 2 : 0));
     }
   }
   ProfScope ps(c, st, TNX_KC_FINAL, 16.0 * (double)B.fin.total);
@@ -300,8 +302,9 @@ extern "C" tnx_status tnx_batch_create(tnx_ctx* ctx, int n, tnx_network* const* 
         bs.dKI = B->upload(kitems);
         bs.nki = (int64_t)kitems.size();
         bs.dSG = B->upload(sg);
-        bs.dST = B->upload(st);
-        bs.nst = (int)st.size();
+        const std::vector<GemmTile> sched = tnx_split_schedule(st, sg, B->prec == TNX_PREC_TF32 ? 16 : 32, bs.grid);
+        bs.dST = B->upload(sched);
+        bs.nst = (int)sched.size();
         for (const GemmTile& t : st) bs.kmax = std::max(bs.kmax, (int)sg[t.group].K);
       }
     }

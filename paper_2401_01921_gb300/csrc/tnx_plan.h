@@ -245,6 +245,9 @@ int tnx_f64_edge(const std::vector<GemmGroup>& groups, const std::vector<int>& w
 std::vector<GemmTile> tnx_gemm_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which, int edge);
 // runs of fused-step tiles from entries that hold whole bands; run gets the most tiles in one
 std::vector<FusedTile> tnx_fused_tiles(const std::vector<FusedTile>& bands, int& lane_rows);
+// tke: K values of a tile; grid: the CTAs that walk the returned list (tnx_split.cpp)
+std::vector<GemmTile> tnx_split_schedule(const std::vector<GemmTile>& tiles, const std::vector<SplitGroup>& sg, int tke,
+                                         int& grid);
 std::vector<GemmTile> tnx_skinny_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which);
 
 // relayout chunks (tnx_network.cpp)
