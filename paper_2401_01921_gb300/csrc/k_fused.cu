@@ -149,11 +149,12 @@ __global__ void __launch_bounds__(FT, 6) fused_skinny_kernel(const GemmGroup* __
 // its time on the chain of loads before the product (tile, group and descriptors, B and
 // A), six tiles to an SM; here an SM holds 28 or more.  Two rows per lane share the
 // lists' and descriptors' reads where tiles are full (four took 156 us at 4096, one
-// 168); bands of a few rows take one.  One apply (ncu, cold), before -> now: Heisenberg
-// at bond dimension 2048 60 -> 42 us, 4096 182 -> 136, environment step at 2048
-// 46 -> 21.5; 48 Hubbard sites 178 us for the instances with 32 rows per tile and more and
-// 135 for the relayouts and skinny products of the others -> 165 for all; the two MPO
-// steps of one at 601 41 -> 25.
+// 168); bands of a few rows take one.  One apply (ncu, cold), with a CTA per tile ->
+// now: Heisenberg at bond dimension 2048 75 -> 42 us, 4096 244 -> 136 (60 and 182 with
+// runs of tiles to a CTA), environment step at 2048 50 -> 21; the two MPO steps of one
+// Hubbard site at 601 41 -> 25; 48 Hubbard sites 178 us for the instances with 32 rows per
+// tile and more and 135 for the relayouts and skinny products of the others -> 165 for
+// all.
 constexpr int FW = 4;   // warps per CTA, each on its own tile
 
 __host__ __device__ constexpr size_t warp_smem(int kp, int np, int R) {

@@ -33,7 +33,7 @@
 //    warps' rotations and next dot products.
 // Measured (the sweeps alone, wavefunctions of the U(1) Heisenberg chain with
 // spectra over 12 decades): bond dimension 200 (blocks of up to 83 vectors) 4.6 ->
-// 1.7 ms, 1024 (up to 294) 49 -> 15 ms.  At 294 the rotations' FP64 issue on the SMs
+// 1.6 ms, 1024 (up to 294) 49 -> 13.5 ms.  At 294 the rotations' FP64 issue on the SMs
 // that hold the largest blocks bounds a step, at 83 the chain dot, angle, rotation.
 //
 // The rotations, thresholds and stopping rule are those of k_svd.cu: a pair with
