@@ -488,8 +488,10 @@ __global__ void qr_gather_r_kernel(const SvdQr* __restrict__ qs, int nq) {
   }
 }
 
-// One warp per (block, vector p), after the Jacobi on the rows of R (both rows
-// count times the vector's factor D[4 p]): sigma_p = |Xr[p,:]|; J[p][perm[i]] = Xr[p][i] / sigma_p (the right singular
+// One warp per (block, vector p), after the Jacobi on the rows of R.  Both rows count
+// times one factor, the one that makes Jr[p,:] a unit vector (rounding lets the factor that
+// the sweeps carry, and the rows' own norms, drift by some units in the last place):
+// sigma_p = |Xr[p,:]|; J[p][perm[i]] = Xr[p][i] / sigma_p (the right singular
 // vector of A, 0 when sigma_p = 0); Xf[p,:] = sigma_p Q Jr[p,:]^T, with Q
 // applied as H_0 H_1 ... H_{c-1} to (Jr[p,:], 0, ..., 0).  Lane l keeps the
 // entries e = l (mod 32) of z throughout, in registers when r <= 32 VB.
@@ -502,13 +504,17 @@ __global__ void qr_apply_kernel(const SvdQr* __restrict__ qs, const int2* __rest
     const SvdQr q = qs[gv.x];
     const int p = gv.y, c = q.c, r = q.r;
     const double* xr = q.Xr + (int64_t)p * q.ldr;
-    double s = 0.0;
-    for (int i = lane; i < c; i += 32) s = fma(xr[i], xr[i], s);
+    const double* jr = q.Jr + (int64_t)p * q.ldr;
+    double s = 0.0, sj = 0.0;
+    for (int i = lane; i < c; i += 32) {
+      s = fma(xr[i], xr[i], s);
+      sj = fma(jr[i], jr[i], sj);
+    }
     s = warp_sum(s);
-    const double dp = q.D[4 * p], nx = sqrt(s), sg = nx * dp, inv = nx > 0.0 ? 1.0 / nx : 0.0;
+    sj = warp_sum(sj);
+    const double dp = 1.0 / sqrt(sj), nx = sqrt(s), sg = nx * dp, inv = nx > 0.0 ? 1.0 / nx : 0.0;
     for (int i = lane; i < c; i += 32) q.J[(int64_t)p * c + q.perm[i]] = xr[i] * inv;
     if (lane == 0) q.sigma[p] = sg;
-    const double* jr = q.Jr + (int64_t)p * q.ldr;
     double* xf = q.Xf + (int64_t)p * r;
     if (r <= 32 * VB) {
       double z[VB];
