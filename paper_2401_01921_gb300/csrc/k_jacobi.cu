@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(JB_THREADS) jacobi_block_kernel(const JbGroup*
   double* buf = (double*)(jb_dyn + (sizeof(JbShared) + 15) / 16 * 16);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < TNX_JB_MAXSLOTS / 32; i += JB_THREADS) S.done[i] = 0;
+  if (threadIdx.x == 0) S.big = 0;
   __syncthreads();
   bool ok = true, more = true;
   for (int it = 0; ok && more; ++it) {
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(JB_THREADS) jacobi_block_kernel(const JbGroup*
           S.nrm[lane] = __ldcg(D + 2);
           S.n0[lane] = __ldcg(D + 3);
         }
-        if (lane == 0) S.any = S.big = 0;
+        if (lane == 0) S.any = 0;
       }
       asm volatile("cp.async.wait_all;" ::: "memory");
       __syncthreads();
@@ -486,7 +487,11 @@ __global__ void __launch_bounds__(JB_THREADS) jacobi_block_kernel(const JbGroup*
       }
       __syncthreads();
       if (threadIdx.x == 0) {
+        // The flag is cleared by its reader: nothing orders this read before the other
+        // warps' start on the CTA's next slot, whose first barrier orders the clear
+        // before the angle warps set the flag again.
         if (S.big) __stcg(met + (int64_t)sl.x * max_sweeps + sw, 1);
+        S.big = 0;
         __threadfence();   // one fence for the stores of the whole CTA, then plain flags
         asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(g.ver + p), "r"(it + 1) : "memory");
         asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(g.ver + q), "r"(it + 1) : "memory");
