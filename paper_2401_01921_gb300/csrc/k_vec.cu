@@ -318,6 +318,11 @@ __device__ __forceinline__ unsigned long long arrive(unsigned long long* word) {
   return old;
 }
 
+// Without ordering memory: that every CTA of the cluster has started is all it says.
+__device__ __forceinline__ void cluster_arrive_started() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_arrive() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -463,7 +468,10 @@ __global__ void __launch_bounds__(LT, 2) lanczos_step_kernel(LanczosDev L, int j
   __shared__ ProScales s_sc;
   __shared__ int s_ok, s_pass;
   __shared__ double s_part[2][STEP_CL];
-  if (stopped(L.state)) return;
+  if (stopped(L.state)) return;   // all CTAs alike: what sets the flag waits for every CTA first
+  // A CTA of the cluster may be written to (step_publish) once it is known to run; the wait
+  // stands before the first such write, behind the loads.
+  if (CLUSTER) cluster_arrive_started();
   const int nb = gridDim.x, tid = threadIdx.x;
   const int64_t chunk = ((L.n + nb - 1) / nb + 31) / 32 * 32;
   const int64_t c0 = min(L.n, chunk * blockIdx.x), c1 = min(L.n, c0 + chunk);
@@ -521,6 +529,7 @@ __global__ void __launch_bounds__(LT, 2) lanczos_step_kernel(LanczosDev L, int j
       if (x + u * LT < c1) acc = fma(w[u], v[u], acc);
   }
   acc = step_block_sum(acc, sh);
+  if (CLUSTER) cluster_wait();   // every CTA has started
   step_publish<CLUSTER>(acc, part, s_part[0]);
   if (!step_barrier<CLUSTER>(L)) return give_up(41);
   const double a = step_total<CLUSTER>(part, s_part[0], sh);
