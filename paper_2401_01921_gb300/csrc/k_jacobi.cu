@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(JB_THREADS) jacobi_block_kernel(const JbGroup*
   for (int i = threadIdx.x; i < TNX_JB_MAXSLOTS / 32; i += JB_THREADS) S.done[i] = 0;
   if (threadIdx.x == 0) S.big = 0;
   __syncthreads();
-  bool ok = true, more = true;
+  bool ok = *(volatile int*)status == 0, more = true;   // an expired QR leaves nothing to sweep
   for (int it = 0; ok && more; ++it) {
     more = false;
     int mine = 0;

@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(CJT) jacobi_coop_kernel(const SvdGroup* __rest
   const int lane = threadIdx.x & 31;
   const int gw = blockIdx.x * (CJT / 32) + (threadIdx.x >> 5), nwarps = gridDim.x * (CJT / 32);
   int sw = 0;
-  bool ok = true;
+  bool ok = *(volatile int*)status == 0;   // an expired QR leaves nothing to sweep
   while (ok && sw < max_sweeps) {
     double off_w = 0.0;   // this warp's largest squared relative off-diagonal of the sweep
     for (int round = 0; round < maxcp - 1 && ok; ++round) {
@@ -471,8 +471,10 @@ __global__ void __launch_bounds__(CJT) qr_coop_kernel(const SvdQr* __restrict__ 
 }
 
 // Xr[p][j] = R[p][j] = X[perm[j]][p] for p <= j < c (0 elsewhere in the row), Jr = I
-__global__ void qr_gather_r_kernel(const SvdQr* __restrict__ qs, int nq) {
+// (nothing when the QR's wait ran out: perm is then only partly written)
+__global__ void qr_gather_r_kernel(const SvdQr* __restrict__ qs, int nq, const int* status) {
   tnx_grid_dependency();
+  if (*(const volatile int*)status != 0) return;
   for (int gi = blockIdx.y; gi < nq; gi += gridDim.y) {
     const SvdQr q = qs[gi];
     const int64_t n = (int64_t)q.c * q.ldr;
@@ -494,10 +496,13 @@ __global__ void qr_gather_r_kernel(const SvdQr* __restrict__ qs, int nq) {
 // sigma_p = |Xr[p,:]|; J[p][perm[i]] = Xr[p][i] / sigma_p (the right singular
 // vector of A, 0 when sigma_p = 0); Xf[p,:] = sigma_p Q Jr[p,:]^T, with Q
 // applied as H_0 H_1 ... H_{c-1} to (Jr[p,:], 0, ..., 0).  Lane l keeps the
-// entries e = l (mod 32) of z throughout, in registers when r <= 32 VB.
+// entries e = l (mod 32) of z throughout, in registers when r <= 32 VB.  Nothing when a wait
+// of the QR or the sweeps ran out.
 template <int VB>
-__global__ void qr_apply_kernel(const SvdQr* __restrict__ qs, const int2* __restrict__ vecs, int nvec) {
+__global__ void qr_apply_kernel(const SvdQr* __restrict__ qs, const int2* __restrict__ vecs, int nvec,
+                                const int* status) {
   tnx_grid_dependency();
+  if (*(const volatile int*)status != 0) return;
   const int lane = threadIdx.x & 31;
   for (int vi = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); vi < nvec; vi += gridDim.x * (blockDim.x >> 5)) {
     const int2 gv = vecs[vi];
@@ -719,23 +724,26 @@ cudaError_t tnx_launch_qr_coop(const SvdQr* qs, const int2* slots, int nslots, i
   return cudaSuccess;
 }
 
-cudaError_t tnx_launch_qr_gather_r(const SvdQr* qs, int nq, int maxc, cudaStream_t st) {
+cudaError_t tnx_launch_qr_gather_r(const SvdQr* qs, int nq, int maxc, const int* status, cudaStream_t st) {
   if (nq <= 0) return cudaSuccess;
   int bx = (int)(((int64_t)maxc * maxc + 255) / 256);
   if (bx > 64) bx = 64;
   if (bx < 1) bx = 1;
-  const cudaError_t le = tnx_launch(qr_gather_r_kernel, dim3(bx, nq < 65535 ? nq : 65535), dim3(256), 0, st, qs, nq);
+  const cudaError_t le = tnx_launch(qr_gather_r_kernel, dim3(bx, nq < 65535 ? nq : 65535), dim3(256), 0, st, qs, nq,
+                                    status);
   if (le != cudaSuccess) return le;
   tnx_note_launch(1);
   return cudaGetLastError();
 }
 
-cudaError_t tnx_launch_qr_apply(const SvdQr* qs, const int2* vecs, int nvec, int maxr, cudaStream_t st) {
+cudaError_t tnx_launch_qr_apply(const SvdQr* qs, const int2* vecs, int nvec, int maxr, const int* status,
+                                cudaStream_t st) {
   if (nvec <= 0) return cudaSuccess;
   // one warp per vector, two warps per CTA: the vectors spread over the SMs' FP64 pipes
   const int grid = (nvec + 1) / 2;
-  const cudaError_t le = maxr <= 32 * 8 ? tnx_launch(qr_apply_kernel<8>, dim3(grid), dim3(64), 0, st, qs, vecs, nvec)
-                                        : tnx_launch(qr_apply_kernel<16>, dim3(grid), dim3(64), 0, st, qs, vecs, nvec);
+  const cudaError_t le =
+      maxr <= 32 * 8 ? tnx_launch(qr_apply_kernel<8>, dim3(grid), dim3(64), 0, st, qs, vecs, nvec, status)
+                     : tnx_launch(qr_apply_kernel<16>, dim3(grid), dim3(64), 0, st, qs, vecs, nvec, status);
   if (le != cudaSuccess) return le;
   tnx_note_launch(1);
   return cudaGetLastError();

@@ -391,11 +391,14 @@ struct QbGroup {
 int tnx_qr_block_columns(int maxr);   // columns per slot (8), 0: too long for shared memory
 cudaError_t tnx_launch_qr_block(const SvdQr* qs, const QbGroup* groups, const int2* slots, int nslots, int maxr,
                                 int* status, cudaStream_t st);
-// Xr = R (rows, zero below the diagonal) and Jr = identity for every block
-cudaError_t tnx_launch_qr_gather_r(const SvdQr* qs, int nq, int maxc, cudaStream_t st);
+// Xr = R (rows, zero below the diagonal) and Jr = identity for every block.  It, the sweeps
+// and tnx_launch_qr_apply do nothing when *status is set: the QR's permutation and
+// reflectors are then only partly written.
+cudaError_t tnx_launch_qr_gather_r(const SvdQr* qs, int nq, int maxc, const int* status, cudaStream_t st);
 // after the Jacobi on Xr: sigma, J and Xf for every (block, vector)
 // (maxr: the longest vector of the launch, which picks the register width)
-cudaError_t tnx_launch_qr_apply(const SvdQr* qs, const int2* vecs, int nvec, int maxr, cudaStream_t st);
+cudaError_t tnx_launch_qr_apply(const SvdQr* qs, const int2* vecs, int nvec, int maxr, const int* status,
+                                cudaStream_t st);
 // round r of a sweep over slots (group, pair index); maxoff gets the largest
 // |x_p . x_q| / (|x_p| |x_q|) met, as the bits of a non-negative double
 // every round and sweep in one cooperative launch; offmax[max_sweeps], *bar

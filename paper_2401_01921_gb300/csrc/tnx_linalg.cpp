@@ -268,11 +268,11 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
     }
     const JbGroup* dj = (const JbGroup*)up(hj.data(), hj.size() * sizeof(JbGroup));
     const int2* djs = (const int2*)up(jslots.data(), jslots.size() * sizeof(int2));
-    // [QR barrier count | QR status, pad | offmax per sweep | Jacobi barrier count | Jacobi status, sweeps]
-    std::vector<uint64_t> zero(MAX_SWEEPS + 4, 0);
+    // [QR barrier count | status, sweeps | offmax per sweep | Jacobi barrier count]; one status
+    // word for all: after a wait that ran out, the kernels behind it touch nothing
+    std::vector<uint64_t> zero(MAX_SWEEPS + 3, 0);
     unsigned long long* w = (unsigned long long*)up(zero.data(), zero.size() * 8);
-    int* qstat = (int*)(w + 1);
-    int* jstat = (int*)(w + MAX_SWEEPS + 3);
+    int* stat = (int*)(w + 1);
     // the QR on columns in shared memory (k_qr.cu) where its slots fit; else step by
     // step through L2
     cudaError_t ce = cudaErrorNotSupported;
@@ -306,29 +306,28 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
       const QbGroup* db = (const QbGroup*)up(hb.data(), hb.size() * sizeof(QbGroup));
       const int2* dbs = (const int2*)up(bslots.data(), bslots.size() * sizeof(int2));
       flush();
-      ce = tnx_launch_qr_block(dq, db, dbs, (int)bslots.size(), maxr, qstat, st);
+      ce = tnx_launch_qr_block(dq, db, dbs, (int)bslots.size(), maxr, stat, st);
     }
     if (ce == cudaErrorNotSupported) {
       (void)cudaGetLastError();
       flush();
-      ce = tnx_launch_qr_coop(dq, dqs, (int)qslots.size(), maxc, w, qstat, st);
+      ce = tnx_launch_qr_coop(dq, dqs, (int)qslots.size(), maxc, w, stat, st);
     }
     if (ce == cudaSuccess) {
-      CUDA_CHECK(tnx_launch_qr_gather_r(dq, ngr, maxc, st));
+      CUDA_CHECK(tnx_launch_qr_gather_r(dq, ngr, maxc, stat, st));
       // the sweeps run on R: vectors of c entries
       if (jw)
         CUDA_CHECK(tnx_launch_jacobi_block(dj, hj.data(), ngr, djs, (int)jslots.size(), MAX_SWEEPS, 1e-13, jmet,
-                                           (unsigned*)(jmet + (size_t)ngr * MAX_SWEEPS), jstat, jstat + 1, st));
+                                           (unsigned*)(jmet + (size_t)ngr * MAX_SWEEPS), stat, stat + 1, st));
       else
         CUDA_CHECK(tnx_launch_jacobi_coop(dr, dslots, (int)slots.size(), maxcp, maxc, MAX_SWEEPS, 1e-13, w + 2,
-                                          w + MAX_SWEEPS + 2, jstat, jstat + 1, st));
-      CUDA_CHECK(tnx_launch_qr_apply(dq, dvecs, (int)vecs.size(), maxr, st));
-      int hs[4] = {0, 0, 0, 0};
-      CUDA_CHECK(cudaMemcpyAsync(hs, qstat, 4, cudaMemcpyDeviceToHost, st));
-      CUDA_CHECK(cudaMemcpyAsync(hs + 2, jstat, 8, cudaMemcpyDeviceToHost, st));
+                                          w + MAX_SWEEPS + 2, stat, stat + 1, st));
+      CUDA_CHECK(tnx_launch_qr_apply(dq, dvecs, (int)vecs.size(), maxr, stat, st));
+      int hs[2] = {0, 0};
+      CUDA_CHECK(cudaMemcpyAsync(hs, stat, 8, cudaMemcpyDeviceToHost, st));
       CUDA_CHECK(cudaStreamSynchronize(st));
-      if (hs[0] != 0 || hs[2] != 0) fail(TNX_ERR_TIMEOUT, "SVD: a grid barrier of the QR or the Jacobi sweeps timed out");
-      sweeps = hs[3];
+      if (hs[0] != 0) fail(TNX_ERR_TIMEOUT, "SVD: a grid barrier of the QR or the Jacobi sweeps timed out");
+      sweeps = hs[1];
       for (int i = 0; i < ngr; ++i) hg[i].X = hq[i].Xf;   // the extraction reads sigma_p u_p from Xf
       done = via_qr = true;
     } else if (ce == cudaErrorNotSupported || ce == cudaErrorCooperativeLaunchTooLarge) {
