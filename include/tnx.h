@@ -360,6 +360,8 @@ tnx_status tnx_server_submit(tnx_server* s, tnx_network* net, const char* vec_sl
 /* Blocks until request id finishes (timeout_ms < 0: no limit; TNX_ERR_TIMEOUT
  * if it runs out) and returns its status; eval / matvecs (Lanczos) and the
  * latency from submission to completion in milliseconds (any may be NULL).
+ * A request whose own kernels gave up a bounded wait fails with TNX_ERR_TIMEOUT
+ * as well, and tnx_last_error names the site of the wait.
  * Each id can be waited for once. */
 tnx_status tnx_server_wait(tnx_server* s, int64_t id, int timeout_ms, double* eval, int* matvecs, double* latency_ms);
 /* Completed requests, evictions, bytes currently resident, peak resident bytes. */

@@ -97,7 +97,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase, int32_t
   while (!mbar_try(bar, phase)) {
     if (*abort_flag) return false;
     if (clock64() - t0 > WAIT_LIMIT) {
-      atomicExch(status, code);
+      *(volatile int32_t*)status = code;   // host memory (any of the codes will do)
       *abort_flag = 1;
       return false;
     }

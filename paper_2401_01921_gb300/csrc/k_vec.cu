@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(LT, 2) lanczos_step_kernel(LanczosDev L, int j
   // a wait that ran out: the solve stops, with an eigenvalue that is not a number
   auto give_up = [&](int code) {
     if (tid == 0) {
-      atomicExch(status, code);
+      *(volatile int32_t*)status = code;   // host memory (any of the codes will do)
       L.alpha[j] = __longlong_as_double(0x7FF8000000000000ll);
       L.state[0] = j + 1;
       L.state[1] = 1;

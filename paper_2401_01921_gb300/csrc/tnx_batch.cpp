@@ -59,6 +59,10 @@ struct tnx_batch {
   TaskList fin;
   int split_grid = 0;         // CTAs of the split GEMMs (autotune); 0: each step's schedule
   std::unique_ptr<GraphRec> graph;
+  StatusWord* status = nullptr;   // bounded waits of the batch's kernels report here
+  ~tnx_batch() {
+    if (ctx) ctx->status_release(status);
+  }
 
   template <class T>
   T* upload(const std::vector<T>& v) {
@@ -126,7 +130,7 @@ void enqueue_batch(tnx_batch& B, cudaStream_t st) {
         CUDA_CHECK(tnx_launch_tf32_rows(s.jobs.d, s.jobs.items, s.jobs.nitems, B.d_slots, st));
       }
       ProfScope ps(c, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
-      CUDA_CHECK(tnx_launch_gemm_tf32(s.dSG, s.dST, s.nst, B.d_slots, c->d_status, st,
+      CUDA_CHECK(tnx_launch_gemm_tf32(s.dSG, s.dST, s.nst, B.d_slots, &B.status->code, st,
                                       B.split_grid ? B.split_grid : s.grid, 64));
     } else {
       if (s.jobs.n) {
@@ -135,7 +139,7 @@ void enqueue_batch(tnx_batch& B, cudaStream_t st) {
         CUDA_CHECK(tnx_launch_slices(s.jobs.d, s.jobs.items, s.jobs.nitems, B.nslice, B.beta, f16, B.d_slots, st, 1));
       }
       ProfScope ps(c, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
-      CUDA_CHECK(tnx_launch_gemm_split(s.dSG, s.dST, s.nst, B.nslice, B.beta, f16, B.d_slots, c->d_status, st,
+      CUDA_CHECK(tnx_launch_gemm_split(s.dSG, s.dST, s.nst, B.nslice, B.beta, f16, B.d_slots, &B.status->code, st,
                                        B.split_grid ? B.split_grid : s.grid, 64, s.kmax <= 160 ? 2 : 0));
     }
   }
@@ -168,6 +172,7 @@ extern "C" tnx_status tnx_batch_create(tnx_ctx* ctx, int n, tnx_network* const* 
     if (!ctx || n < 1 || !nets || !out) fail(TNX_ERR_ARG, "bad batch arguments");
     std::unique_ptr<tnx_batch> B(new tnx_batch());
     B->ctx = ctx;
+    B->status = ctx->status_lease();
     int slots = 0;
     for (int i = 0; i < n; ++i) {
       if (!nets[i] || nets[i]->ctx != ctx) fail(TNX_ERR_ARG, "every network must belong to the context");

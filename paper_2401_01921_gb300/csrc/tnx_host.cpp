@@ -199,10 +199,9 @@ extern "C" tnx_status tnx_ctx_create(int device, void* stream, tnx_alloc_fn allo
   }
   tnx_status s = tnx_guard(c, [&] {
     c->scratch = new DevBuf(c, 64 * 1024);
-    c->d_status = (int32_t*)((char*)c->scratch->p + 63 * 1024);
-    CUDA_CHECK(cudaMemsetAsync(c->d_status, 0, 64, c->stream));
     c->pinned = nullptr;
     CUDA_CHECK(cudaMallocHost(&c->pinned, 4096));
+    c->status_release(c->status_lease());   // the first block of status words
   });
   if (s != TNX_OK) {
     delete c;
@@ -220,20 +219,55 @@ extern "C" tnx_status tnx_ctx_destroy(tnx_ctx* ctx) {
   delete ctx->scratch;
   if (ctx->pinned) cudaFreeHost(ctx->pinned);
   cudaStreamSynchronize(ctx->stream);
+  for (StatusWord* b : ctx->status_blocks) cudaFreeHost(b);
   delete ctx;
   return TNX_OK;
 }
 
-void check_device_status(tnx_ctx* ctx) {
-  int32_t* h = (int32_t*)ctx->pinned + 512;
-  CUDA_CHECK(cudaMemcpyAsync(h, ctx->d_status, 4, cudaMemcpyDeviceToHost, ctx->stream));
-  CUDA_CHECK(cudaStreamSynchronize(ctx->stream));
-  if (*h != 0) {
-    const int code = *h;
-    CUDA_CHECK(cudaMemsetAsync(ctx->d_status, 0, 4, ctx->stream));
-    CUDA_CHECK(cudaStreamSynchronize(ctx->stream));
-    fail(TNX_ERR_TIMEOUT, "a bounded device wait ran out (site " + std::to_string(code) + ")");
+StatusWord* tnx_ctx::status_lease() {
+  std::lock_guard<std::mutex> lock(status_mu);
+  if (status_free.empty()) {
+    StatusWord* b = nullptr;
+    CUDA_CHECK(cudaMallocHost((void**)&b, kStatusBlock * sizeof(StatusWord)));
+    status_blocks.push_back(b);
+    for (int i = kStatusBlock - 1; i >= 0; --i) status_free.push_back(new (b + i) StatusWord{0, {0}});
   }
+  StatusWord* w = status_free.back();
+  status_free.pop_back();
+  return w;
+}
+
+// An unread code stays in the word: check_device_status looks at free words too.
+void tnx_ctx::status_release(StatusWord* w) {
+  if (!w) return;
+  std::lock_guard<std::mutex> lock(status_mu);
+  w->served.store(0);
+  status_free.push_back(w);
+}
+
+int tnx_status_take(StatusWord* w) {
+  volatile int32_t* p = &w->code;
+  const int code = *p;
+  if (code != 0) *p = 0;
+  return code;
+}
+
+std::string tnx_status_message(int code) {
+  return "a bounded device wait ran out (site " + std::to_string(code) + ")";
+}
+
+void check_device_status(tnx_ctx* ctx) {
+  int code = 0;
+  {
+    std::lock_guard<std::mutex> lock(ctx->status_mu);
+    for (StatusWord* b : ctx->status_blocks)
+      for (int i = 0; i < tnx_ctx::kStatusBlock; ++i)
+        if (b[i].served.load() == 0) {
+          const int c = tnx_status_take(b + i);
+          if (c != 0) code = c;
+        }
+  }
+  if (code != 0) fail(TNX_ERR_TIMEOUT, tnx_status_message(code));
 }
 
 extern "C" tnx_status tnx_sync(tnx_ctx* ctx) {

@@ -1,9 +1,11 @@
 // Host-only internal declarations (C++).
 #pragma once
 
+#include <atomic>
 #include <functional>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -30,6 +32,15 @@ struct ProfRec {
   double work;
 };
 
+// Status word of the bounded waits in the kernels of one network or batch (0: none ran
+// out), in pinned host memory: kernels write it when a wait runs out and never read it,
+// so the host needs no copy to see it behind a synchronisation.  Words of their own keep
+// a served request's failure apart from that of any other work of the context.
+struct StatusWord {
+  int32_t code;                // written by the device
+  std::atomic<int32_t> served; // a server answers for it (a request is in flight)
+};
+
 struct tnx_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -39,7 +50,12 @@ struct tnx_ctx {
   std::string err;
   DevBuf* scratch = nullptr;   // small device scratch (norm partials)
   void* pinned = nullptr;      // small pinned host buffer
-  int32_t* d_status = nullptr; // device status word written by bounded waits (0 = ok)
+  std::mutex status_mu;
+  std::vector<StatusWord*> status_blocks;   // pinned blocks of kStatusBlock words
+  std::vector<StatusWord*> status_free;
+  static constexpr int kStatusBlock = 256;
+  StatusWord* status_lease();
+  void status_release(StatusWord* w);
   bool use_graphs = true;      // capture applies / Lanczos solves in CUDA graphs (needs a non-default stream)
   // profiler (CUDA events around kernel classes)
   uint32_t prof = 0;                 // bit c set: kernel class c is timed
@@ -116,8 +132,12 @@ struct tnx_tensor {
 tnx_status tnx_guard(tnx_ctx* ctx, const std::function<void()>& f);
 // add the timings of events recorded inside a graph (after the graph ran)
 void prof_accumulate(tnx_ctx* ctx, const std::vector<ProfRec>& recs);
-// after a stream sync: fail with TNX_ERR_TIMEOUT if a device wait ran out (and clear it)
+// after a stream sync: fail with TNX_ERR_TIMEOUT if a device wait ran out (and clear it);
+// the words that a server answers for are left alone
 void check_device_status(tnx_ctx* ctx);
+// The code of a word after the work that may write it has finished, and clears it.
+int tnx_status_take(StatusWord* w);
+std::string tnx_status_message(int code);
 void check_contractible(const BondD& a, const BondD& b, const std::string& label);
 void enumerate_blocks(const std::vector<BondD>& bonds, std::vector<int32_t>& qn, int64_t& nblk);
 tnx_tensor* make_tensor(tnx_ctx* ctx, const std::vector<BondD>& bonds);

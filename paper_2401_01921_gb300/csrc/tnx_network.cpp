@@ -1745,7 +1745,7 @@ std::unique_ptr<Plan> build_plan(tnx_network* net, const std::string& key, const
     }
     p->out_slot = p->new_slot(nullptr, ne);
   }
-  p->d_status = (int32_t*)p->alloc_zero(64);
+  p->d_status = &net->status->code;
   if (p->nin > 64) fail(TNX_ERR_UNSUPPORTED, "at most 64 tensors per network");
   std::function<uint64_t(int)> leaves = [&](int node) -> uint64_t {
     const TreeNode& n = net->tree[node];
@@ -1981,6 +1981,7 @@ extern "C" tnx_status tnx_network_create(tnx_ctx* ctx, const char* spec, tnx_net
     if (!ctx || !spec || !out) fail(TNX_ERR_ARG, "null argument");
     std::unique_ptr<tnx_network> net(new tnx_network());
     net->ctx = ctx;
+    net->status = ctx->status_lease();
     std::string text(spec), line, order;
     bool have_tout = false;
     size_t p0 = 0;
@@ -2194,7 +2195,9 @@ struct LanczosCache {
   int64_t vs_nitems = 0;
 };
 
-tnx_network::~tnx_network() = default;
+tnx_network::~tnx_network() {
+  if (ctx) ctx->status_release(status);
+}
 
 namespace {
 // Bytes of the Lanczos workspace buffers, in allocation order: V, w, alpha,
@@ -2441,7 +2444,7 @@ void tnx_lanczos_enqueue(tnx_network* net, int slot, tnx_tensor* v0, int nsteps,
       // (j+1)n + 2n for the update
       ProfScope ps(ctx, st, TNX_KC_VECTOR, 8.0 * (double)n * 8);
       CUDA_CHECK(tnx_launch_lanczos_step(L, j, p->d_slots + slot, st, vcopy == nullptr,
-                                         p->prec == TNX_PREC_F32 || p->prec == TNX_PREC_TF32, ctx->d_status));
+                                         p->prec == TNX_PREC_F32 || p->prec == TNX_PREC_TF32, p->d_status));
       if (vslice) {
         // v_{j+1} and the next apply's slices of the vector operand in one pass over w
         const VecSrc vs{(const int64_t*)lc->vs_rowtab->p, L.w, L.V + (int64_t)(j + 1) * n,
@@ -2511,6 +2514,8 @@ size_t tnx_network_resident_bytes(tnx_network* net) {
     for (auto& d : net->lanczos->bufs) b += d->bytes;
   return b;
 }
+
+int32_t* tnx_network_status(tnx_network* net) { return &net->status->code; }
 
 // Frees the plan and the Lanczos workspace (rebuilt on the next use).  The
 // caller guarantees nothing of this network is in flight.

@@ -136,7 +136,7 @@ struct Plan {
   int prec = TNX_PREC_F64;
   int nslice = 6, beta = 7;
   bool narrow_tiles = true;       // from the network (false in a batch: one split tile width, MPO steps always fused)
-  int32_t* d_status = nullptr;
+  int32_t* d_status = nullptr;    // the network's (StatusWord)
   std::string key;
   std::string order;
   ~Plan() = default;
@@ -226,6 +226,7 @@ struct tnx_network {
   size_t sized_bytes = 0;
   std::unique_ptr<Plan> plan;
   std::unique_ptr<struct LanczosCache> lanczos;
+  StatusWord* status = nullptr;    // bounded waits of this network's kernels report here
   ~tnx_network();
 };
 
@@ -269,3 +270,5 @@ size_t tnx_lanczos_workspace_bytes(int64_t n, int nsteps);
 // Bytes of the network's current Lanczos workspace (0 if none).
 size_t tnx_network_lanczos_bytes(tnx_network* net);
 void tnx_network_evict(tnx_network* net);
+// Where the bounded waits of the network's kernels report (host memory).
+int32_t* tnx_network_status(tnx_network* net);

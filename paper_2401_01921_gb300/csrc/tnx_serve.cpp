@@ -179,6 +179,9 @@ void worker_loop(tnx_server* S) {
         cudaGetLastError();
         r.status = TNX_ERR_CUDA;
         r.err = cudaGetErrorString(q);
+      } else if (const int code = tnx_status_take(r.net->status)) {
+        r.status = TNX_ERR_TIMEOUT;
+        r.err = tnx_status_message(code);
       } else {
         r.status = 0;
         if (r.kind == TNX_REQ_LANCZOS) {
@@ -186,6 +189,7 @@ void worker_loop(tnx_server* S) {
           r.matvecs = ((int32_t*)(S->pinned + 2 * k + 1))[0];
         }
       }
+      r.net->status->served.store(0);
       S->busy.erase(r.net);
       S->slot_req[k] = -1;
       S->completed++;
@@ -247,10 +251,12 @@ void worker_loop(tnx_server* S) {
         S->queue.erase(it);
         lock.unlock();
         std::string err;
+        r.net->status->served.store(1);
         const int code = start(S, r, k, err);
         lock.lock();
         account(S, r.net);
         if (code != TNX_OK) {
+          r.net->status->served.store(0);
           S->busy.erase(r.net);
           S->slot_req[k] = -1;
           finish_failed(S, r, code, err);
@@ -297,6 +303,8 @@ extern "C" tnx_status tnx_server_destroy(tnx_server* S) {
     cudaStreamSynchronize(st);
     cudaStreamDestroy(st);
   }
+  // what nobody waits for any more is the next tnx_sync's to report
+  for (auto& kv : S->busy) kv.first->status->served.store(0);
   for (auto& kv : S->reqs)
     if (kv.second.done) cudaEventDestroy(kv.second.done);
   if (S->pinned) cudaFreeHost(S->pinned);

@@ -257,7 +257,7 @@ void tnx_enqueue_split(Plan& p, StepPlan& s, cudaStream_t st, bool needA, bool n
       CUDA_CHECK(tnx_launch_tf32_rows(J->d, J->items, J->nitems, p.d_slots, st));
     }
     ProfScope ps(p.ctx, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
-    CUDA_CHECK(tnx_launch_gemm_tf32(s.dSG, s.dST, s.nstiles, p.d_slots, p.ctx->d_status, st, s.split_grid,
+    CUDA_CHECK(tnx_launch_gemm_tf32(s.dSG, s.dST, s.nstiles, p.d_slots, p.d_status, st, s.split_grid,
                                     s.split_tn, s.split_fold ? 1 : 0));
     return;
   }
@@ -267,6 +267,6 @@ void tnx_enqueue_split(Plan& p, StepPlan& s, cudaStream_t st, bool needA, bool n
     CUDA_CHECK(tnx_launch_slices(J->d, J->items, J->nitems, p.nslice, p.beta, f16, p.d_slots, st, balance ? 1 : 0));
   }
   ProfScope ps(p.ctx, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
-  CUDA_CHECK(tnx_launch_gemm_split(s.dSG, s.dST, s.nstiles, p.nslice, p.beta, f16, p.d_slots, p.ctx->d_status, st,
+  CUDA_CHECK(tnx_launch_gemm_split(s.dSG, s.dST, s.nstiles, p.nslice, p.beta, f16, p.d_slots, p.d_status, st,
                                    s.split_grid, s.split_tn, s.split_fold ? 1 : s.split_kmax <= 160 ? 2 : 0));
 }
