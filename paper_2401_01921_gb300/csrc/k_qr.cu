@@ -93,7 +93,13 @@ __global__ void __launch_bounds__(32 * QW) qr_block_kernel(const SvdQr* __restri
           const bool flat = S.below[best] == 0.0;
           S.mine.beta = flat ? x0 : (x0 >= 0.0 ? -n : n);
           S.mine.u0 = flat ? 1.0 : x0 + (x0 >= 0.0 ? n : -n);
-          S.mine.kappa = flat ? 0.0 : 1.0 / fma(fabs(x0), n, m);
+          const double d = fma(fabs(x0), n, m);   // at most 2 m
+          double kappa = 1.0 / d;
+          // half of it where d overflows; a norm that does leaves nothing finite behind it
+          // (0 would leave the column as it is)
+          if (!is_finite(d))
+            kappa = is_finite(m) ? 0.5 / fma(0.5 * fabs(x0), n, 0.5 * m) : __longlong_as_double(0x7FF8000000000000ll);
+          S.mine.kappa = flat ? 0.0 : kappa;
         }
       } else if (lane == 0) {
         S.mine.idx = -1;

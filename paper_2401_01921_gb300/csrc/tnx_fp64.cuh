@@ -40,14 +40,18 @@ __device__ __forceinline__ long long warp_sum_scaled(double x, int& k) {
   return warp_sum_int(scaled_int(x, k));
 }
 
-// x * 2^-k for a normal or zero x (0 when the result is not normal)
+// x * 2^-k for a normal or zero x (0 below the normal range, an infinity above it)
 __device__ __forceinline__ double shift_down(double x, int k) {
   const int hi = __double2hiint(x), e = expo(hi) - k;
-  if (expo(hi) == 0 || e <= 0 || e >= 2047) return 0.0;
+  if (expo(hi) == 0 || e <= 0) return 0.0;
+  if (e >= 2047) return __hiloint2double((hi & 0x80000000) | 0x7FF00000, 0);
   return __hiloint2double((hi & 0x800FFFFF) | (e << 20), __double2loint(x));
 }
 
-// Sum of a double over the warp, in every lane (NaN when a value is not finite).
+__device__ __forceinline__ bool is_finite(double x) { return expo(__double2hiint(x)) != 2047; }
+
+// Sum of a double over the warp, in every lane (NaN when a value is not finite, an infinity
+// when the sum of finite values is not; subnormal values count as zero).
 __device__ __forceinline__ double warp_sum_double(double x) {
   int k;
   const long long v = warp_sum_scaled(x, k);
