@@ -226,7 +226,10 @@ struct FlatSpace {
     FlatHist out;
     if (a.empty() || b.empty()) return out;
     const int64_t lo = a.front().first + b.front().first, hi = a.back().first + b.back().first;
-    if (hi - lo < (int64_t)1 << 22) {
+    // an array over the range of keys while it has at most 32 entries per product: clearing
+    // and reading one takes some 2 ns, an insertion into the map 50 to 100.  (Charges
+    // in steps of 20000: 187 ms for the order search of the H_eff with the array, 1.3 with the map.)
+    if (hi - lo < (int64_t)1 << 22 && hi - lo < 32 * (int64_t)(a.size() * b.size())) {
       std::vector<double> v((size_t)(hi - lo + 1), 0.0);
       for (const auto& x : a)
         for (const auto& y : b) v[(size_t)(x.first + y.first - lo)] += x.second * y.second;
