@@ -259,11 +259,21 @@ Hist leg_hist(const BondD& b) {
 void sparse_optimal_tree(tnx_network* net) {
   const int n = (int)net->ts.size();
   if (n > 12) fail(TNX_ERR_UNSUPPORTED, "the block-sparse order search supports at most 12 tensors");
+  // Tensors of different symmetries are refused where they meet (build_step); their
+  // search counts dimensions alone, as charges of different kinds do not add.
   SymInfo sy;
-  const BondD& b0 = net->ts[0].t->bonds[0];
-  sy.kinds = b0.kinds;
-  sy.zn = b0.zn;
-  const int nsym = b0.nsym;
+  const BondD* b0 = nullptr;
+  bool mixed = false;
+  for (auto& t : net->ts)
+    for (auto& b : t.t->bonds) {
+      if (!b0) b0 = &b;
+      mixed = mixed || !b.same_syms(*b0);
+    }
+  if (b0 && !mixed) {
+    sy.kinds = b0->kinds;
+    sy.zn = b0->zn;
+  }
+  const int nsym = (int)sy.kinds.size();
   // label -> (tensor, bond) of each occurrence
   std::map<std::string, std::vector<std::pair<int, const BondD*>>> occ;
   for (int i = 0; i < n; ++i) {
@@ -335,6 +345,13 @@ void sparse_optimal_tree(tnx_network* net) {
     for (int l : open[a]) (std::find(open[b].begin(), open[b].end(), l) != open[b].end() ? k : fa).push_back(l);
     for (int l : open[b])
       if (std::find(open[a].begin(), open[a].end(), l) == open[a].end()) fb.push_back(l);
+    if (mixed) {
+      double h[3] = {1.0, 1.0, 1.0};
+      for (int l : fa) h[0] *= (double)bond_in(l, a).dim;
+      for (int l : k) h[1] *= (double)bond_in(l, a).dim;
+      for (int l : fb) h[2] *= (double)bond_in(l, b).dim;
+      return 2.0 * h[0] * h[1] * h[2];
+    }
     double c = 0.0;
     if (space.ok) {
       const FlatHist &ha = flat_of(fa, a), &hk = flat_of(k, a), &hb = flat_of(fb, b);

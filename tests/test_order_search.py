@@ -1,5 +1,6 @@
 """CPU: the block-sparse order search of the library on host data alone (a small program around its source):
-charges in wide steps give the order that charges in steps of one give, and cost no array over their range."""
+charges in wide steps give the order that charges in steps of one give, and cost no array over their range;
+tensors whose symmetries differ get an order (their contraction is refused later)."""
 import os
 import subprocess
 
@@ -29,9 +30,11 @@ static BondD bond(int dir, int nsym, int nsec, int step, int deg) {
   return b;
 }
 
-// argv: symmetries, step between charges, sectors of the virtual bonds; prints the order and the shortest time in ms
+// argv: symmetries, step between charges, sectors of the virtual bonds, symmetries of tensor 0 (if others);
+// prints the order and the shortest time in ms
 int main(int argc, char** argv) {
-  const int nsym = atoi(argv[1]), step = atoi(argv[2]), nsec = atoi(argv[3]);
+  const int nsym_all = atoi(argv[1]), step = atoi(argv[2]), nsec = atoi(argv[3]);
+  const int nsym_0 = argc > 4 ? atoi(argv[4]) : nsym_all;
   const char* name[5] = {"L", "psi", "W1", "W2", "R"};
   const char* labels[5] = {"a,w0,ap", "a,s1,s2,b", "w0,s1p,s1,w1", "w1,s2p,s2,w2", "b,w2,bp"};
   double best = 1e30;
@@ -44,6 +47,7 @@ int main(int argc, char** argv) {
       t.name = name[i];
       t.labels = split_labels(labels[i]);
       t.t = new tnx_tensor();
+      const int nsym = i ? nsym_all : nsym_0;
       for (const std::string& l : t.labels) {
         const bool chi = l[0] == 'a' || l[0] == 'b';
         t.t->bonds.push_back(bond(seen[l]++ ? TNX_BD_OUT : TNX_BD_IN, nsym, !nsym ? 1 : chi ? nsec : l[0] == 'w' ? 3 : 2,
@@ -73,9 +77,8 @@ def search(tmp_path_factory):
                     f"-I{build.INCLUDE}", f"-I{build.CSRC}", *build.ARCH, f"-L{os.path.dirname(lib)}", "-l:libtnx.so",
                     "-Xlinker", f"-rpath={os.path.dirname(lib)}"], check=True, capture_output=True)
 
-    def run(nsym, step, nsec):
-        order, ms = subprocess.run([exe, str(nsym), str(step), str(nsec)], check=True, capture_output=True,
-                                   text=True).stdout.split()
+    def run(*args):
+        order, ms = subprocess.run([exe, *map(str, args)], check=True, capture_output=True, text=True).stdout.split()
         return order, float(ms)
     return run
 
@@ -87,3 +90,10 @@ def test_wide_charges(search, nsym, step, nsec):
     ref, ref_ms = search(nsym, 1, nsec)
     assert order == ref
     assert ms <= 20 * ref_ms + 5.0   # an array over the range took 100 to 270 times as long for one charge
+
+
+@pytest.mark.parametrize("nsym,nsym0", [(1, 0), (0, 1), (2, 1), (1, 2)])
+def test_tensors_of_different_symmetries(search, nsym, nsym0):
+    """Such a network is refused when it is launched; the search before that has to survive it."""
+    order, _ = search(nsym, 1, 8, nsym0)
+    assert sorted(order.replace("(", "").replace(")", "").split(",")) == ["L", "R", "W1", "W2", "psi"]
