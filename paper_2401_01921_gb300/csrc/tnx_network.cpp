@@ -260,7 +260,8 @@ void sparse_optimal_tree(tnx_network* net) {
   const int n = (int)net->ts.size();
   if (n > 12) fail(TNX_ERR_UNSUPPORTED, "the block-sparse order search supports at most 12 tensors");
   // Tensors of different symmetries are refused where they meet (build_step); their
-  // search counts dimensions alone, as charges of different kinds do not add.
+  // search counts dimensions alone, as charges of different kinds do not add.  Plain tensors
+  // need no histograms either.
   SymInfo sy;
   const BondD* b0 = nullptr;
   bool mixed = false;
@@ -345,7 +346,7 @@ void sparse_optimal_tree(tnx_network* net) {
     for (int l : open[a]) (std::find(open[b].begin(), open[b].end(), l) != open[b].end() ? k : fa).push_back(l);
     for (int l : open[b])
       if (std::find(open[a].begin(), open[a].end(), l) == open[a].end()) fb.push_back(l);
-    if (mixed) {
+    if (mixed || nsym == 0) {
       double h[3] = {1.0, 1.0, 1.0};
       for (int l : fa) h[0] *= (double)bond_in(l, a).dim;
       for (int l : k) h[1] *= (double)bond_in(l, a).dim;
