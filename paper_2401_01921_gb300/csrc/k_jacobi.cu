@@ -522,6 +522,8 @@ int tnx_jacobi_block_width(int c) {
   return w;
 }
 
+bool tnx_jacobi_block_fits(int64_t nslots, int nsm) { return nslots <= (int64_t)TNX_JB_MAXSLOTS * nsm; }
+
 cudaError_t tnx_launch_jacobi_block(const JbGroup* groups, const JbGroup* host_groups, int ngroups, const int2* slots,
                                     int nslots, int max_sweeps, double tol, int* met, unsigned* cnt, int* status,
                                     int* sweeps_out, cudaStream_t st) {
@@ -548,7 +550,7 @@ cudaError_t tnx_launch_jacobi_block(const JbGroup* groups, const JbGroup* host_g
   // one slot per SM: shared memory that keeps a second CTA off (two on one SM
   // would share its FP64 units while others idle)
   if (nslots <= nsm && smem < kSmemMax / 2 + 1024) smem = kSmemMax / 2 + 1024;
-  if ((nslots + grid - 1) / grid > TNX_JB_MAXSLOTS) return cudaErrorNotSupported;
+  if ((nslots + grid - 1) / grid > TNX_JB_MAXSLOTS) return cudaErrorInvalidValue;   // tnx_jacobi_block_fits
   float tol2 = (float)(tol * tol);
   void* args[] = {(void*)&groups, (void*)&slots, (void*)&nslots, (void*)&max_sweeps, (void*)&tol2,
                   (void*)&met,    (void*)&cnt,   (void*)&status, (void*)&sweeps_out};

@@ -360,6 +360,9 @@ struct JbGroup {
   int32_t c, ld, nb, wmax;
 };
 #define TNX_JB_MAXSLOTS 1024   // slots per CTA at most
+// Whether so many slots can run (at least one CTA per SM does); the caller takes
+// jacobi_coop_kernel for more, whatever the blocks' width.
+bool tnx_jacobi_block_fits(int64_t nslots, int nsm);
 // Vectors per column block for a block of c vectors (8 at most; 0: too long for
 // shared memory, the sweeps then run on jacobi_coop_kernel).
 int tnx_jacobi_block_width(int c);

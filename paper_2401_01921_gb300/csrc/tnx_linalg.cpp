@@ -199,8 +199,17 @@ void tnx_svd_run(tnx_tensor* t, int rowrank, int64_t keepdim, double err, const 
   int64_t nC = 0, nC2 = 0, nCR = 0;
   for (Group* G : groups) maxc = std::max(maxc, G->c);
   // the sweeps on column blocks in shared memory (k_jacobi.cu) want even row
-  // strides; a block too large for them keeps the rows of jacobi_coop_kernel
-  const int jw = tnx_jacobi_block_width(maxc);
+  // strides; a block too large for them keeps the rows of jacobi_coop_kernel, and so do
+  // more blocks than their CTAs can keep track of
+  int jw = tnx_jacobi_block_width(maxc);
+  if (jw) {
+    int64_t n = 0;
+    for (Group* G : groups)
+      if (const int w = tnx_jacobi_block_width(G->c)) n += (G->c + 2 * w - 1) / (2 * w);
+    int nsm = 0;
+    CUDA_CHECK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+    if (!tnx_jacobi_block_fits(n, nsm)) jw = 0;
+  }
   auto row_stride = [&](const Group* G) { return jw ? G->c + (G->c & 1) : G->c; };
   for (Group* G : groups) {
     nC += (G->c + 31) / 32 * 32;
