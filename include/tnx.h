@@ -331,7 +331,8 @@ tnx_status tnx_batch_launch_into(tnx_batch* b, tnx_tensor* const* outs);
 tnx_status tnx_batch_flops(tnx_batch* b, double* flops);
 /* Times the split-GEMM launch schedules (one CTA per tile; persistent grids of
  * 152, 304, 456 CTAs) on this batch (writing into outs) and keeps the fastest;
- * *choice (may be NULL) gets the grid size (0 = one CTA per tile). */
+ * *choice (may be NULL) gets the grid size (0 = one CTA per tile).  Without it a
+ * batch runs on 152 CTAs, its tiles dealt to them by their work. */
 tnx_status tnx_batch_autotune(tnx_batch* b, tnx_tensor* const* outs, int* choice);
 
 /* ---------------------------------------------------------------- serving */

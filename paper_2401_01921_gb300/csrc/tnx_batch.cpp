@@ -1,9 +1,9 @@
 // Batched contraction: many networks with the same blueprint and contraction
 // tree run as one sequence of launches (one relayout launch and one grouped
 // GEMM launch per pairwise step for all instances together), captured in one
-// CUDA graph.  The split GEMM's launch schedule (one CTA per tile, or a
-// persistent grid of 1x / 2x / 3x the SM count over a longest-K-first tile
-// list) is picked by timing each candidate on the batch itself.
+// CUDA graph.  The split GEMMs run on the least-loaded schedule of tnx_split_schedule;
+// tnx_batch_autotune times it against one CTA per tile and persistent grids of 2x and
+// 3x the SM count over the longest-K-first tile list, and keeps the fastest.
 //
 // Each instance keeps its own plan (tables, packed operands, intermediates);
 // the batch only merges the task tables, shifting every slot index by the
@@ -33,8 +33,10 @@ struct BStep {
   int64_t nki = 0;
   bool kx_cluster = false;
   SplitGroup* dSG = nullptr;
-  GemmTile* dST = nullptr;
+  GemmTile* dST = nullptr;      // scheduled for `grid` CTAs, holes included
   int nst = 0;
+  GemmTile* dSL = nullptr;      // the same tiles, longest K first
+  int nsl = 0;
   int kmax = 0;                 // largest K of the merged split groups
   int grid = 0;                 // CTAs that dST is scheduled for
   double flops = 0, flops_skinny = 0;
@@ -44,6 +46,8 @@ struct BStep {
   FusedCol* dFC = nullptr;
   int nft = 0, frows = 0, fkp = 0, fnp = 0;
 };
+
+static constexpr int BATCH_SCHEDULE = 152;   // the grid that the schedules are made for
 
 struct tnx_batch {
   tnx_ctx* ctx = nullptr;
@@ -57,7 +61,9 @@ struct tnx_batch {
   double** d_slots = nullptr;
   std::vector<BStep> steps;
   TaskList fin;
-  int split_grid = 0;         // CTAs of the split GEMMs (autotune); 0: each step's schedule
+  // the split GEMMs' launch: BATCH_SCHEDULE each step's own schedule, 0 one CTA per tile of
+  // the list, else so many CTAs over the list
+  int split_grid = BATCH_SCHEDULE;
   std::unique_ptr<GraphRec> graph;
   StatusWord* status = nullptr;   // bounded waits of the batch's kernels report here
   ~tnx_batch() {
@@ -73,6 +79,22 @@ struct tnx_batch {
     return (T*)bufs.back()->p;
   }
 };
+
+// Tiles and CTAs of a step's split GEMM under a choice of split_grid.
+struct SplitShape {
+  const GemmTile* tiles;
+  int n, grid;
+};
+static SplitShape split_shape(const BStep& s, int choice) {
+  return choice == BATCH_SCHEDULE ? SplitShape{s.dST, s.nst, s.grid} : SplitShape{s.dSL, s.nsl, choice};
+}
+
+// What a choice of the autotuning launches in a step (tiles, holes included, and CTAs).
+void tnx_batch_split_shape(const tnx_batch* b, int step, int choice, int* tiles, int* grid) {
+  const SplitShape x = split_shape(b->steps[step], choice);
+  *tiles = x.n;
+  *grid = x.grid;
+}
 
 namespace {
 
@@ -130,8 +152,8 @@ void enqueue_batch(tnx_batch& B, cudaStream_t st) {
         CUDA_CHECK(tnx_launch_tf32_rows(s.jobs.d, s.jobs.items, s.jobs.nitems, B.d_slots, st));
       }
       ProfScope ps(c, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
-      CUDA_CHECK(tnx_launch_gemm_tf32(s.dSG, s.dST, s.nst, B.d_slots, &B.status->code, st,
-                                      B.split_grid ? B.split_grid : s.grid, 64));
+      const SplitShape x = split_shape(s, B.split_grid);
+      CUDA_CHECK(tnx_launch_gemm_tf32(s.dSG, x.tiles, x.n, B.d_slots, &B.status->code, st, x.grid, 64));
     } else {
       if (s.jobs.n) {
         ProfScope ps(c, st, TNX_KC_SLICE, (double)s.jobs.elems * (16.0 + 2.0 * B.nslice));
@@ -139,8 +161,9 @@ void enqueue_batch(tnx_batch& B, cudaStream_t st) {
         CUDA_CHECK(tnx_launch_slices(s.jobs.d, s.jobs.items, s.jobs.nitems, B.nslice, B.beta, f16, B.d_slots, st, 1));
       }
       ProfScope ps(c, st, TNX_KC_GEMM, s.flops - s.flops_skinny);
-      CUDA_CHECK(tnx_launch_gemm_split(s.dSG, s.dST, s.nst, B.nslice, B.beta, f16, B.d_slots, &B.status->code, st,
-                                       B.split_grid ? B.split_grid : s.grid, 64, s.kmax <= 160 ? 2 : 0));
+      const SplitShape x = split_shape(s, B.split_grid);
+      CUDA_CHECK(tnx_launch_gemm_split(s.dSG, x.tiles, x.n, B.nslice, B.beta, f16, B.d_slots, &B.status->code, st, x.grid,
+                                       64, s.kmax <= 160 ? 2 : 0));
     }
   }
   ProfScope ps(c, st, TNX_KC_FINAL, 16.0 * (double)B.fin.total);
@@ -310,6 +333,8 @@ extern "C" tnx_status tnx_batch_create(tnx_ctx* ctx, int n, tnx_network* const* 
         const std::vector<GemmTile> sched = tnx_split_schedule(st, sg, B->prec == TNX_PREC_TF32 ? 16 : 32, bs.grid);
         bs.dST = B->upload(sched);
         bs.nst = (int)sched.size();
+        bs.dSL = B->upload(st);
+        bs.nsl = (int)st.size();
         for (const GemmTile& t : st) bs.kmax = std::max(bs.kmax, (int)sg[t.group].K);
       }
     }
@@ -371,9 +396,9 @@ extern "C" tnx_status tnx_batch_autotune(tnx_batch* b, tnx_tensor* const* outs, 
     tnx_ctx* c = b->ctx;
     const uint32_t prof = c->prof;
     c->prof = 0;
-    const int cands[] = {0, 152, 304, 456};
+    const int cands[] = {BATCH_SCHEDULE, 0, 304, 456};
     float best = 1e30f;
-    int pick = 0;
+    int pick = BATCH_SCHEDULE;
     cudaEvent_t e0, e1;
     CUDA_CHECK(cudaEventCreate(&e0));
     CUDA_CHECK(cudaEventCreate(&e1));
