@@ -44,7 +44,8 @@
 // Waits: a slot's round needs slots of its block's previous round only, and every
 // CTA runs its slots round by round, so with all CTAs resident (a cooperative
 // launch) each wait ends; all are bounded (about a second of clock) all the
-// same, and on expiry *status is set and every CTA leaves.
+// same, and on expiry *status is set, every CTA leaves, and the kernels behind touch
+// nothing.
 #include "tnx_fp64.cuh"
 #include "tnx_internal.h"
 
@@ -511,10 +512,13 @@ constexpr size_t kSmemMax = 226 * 1024;   // the 227 KB limit less the static sh
 }  // namespace
 
 // Vectors per column block: 8, or as many of 4, 2, 1 as fit shared memory (8 up to
-// c = 839).  8 against 4 in an SVD of Heisenberg wavefunctions: 3.3 against 3.4 ms at
-// bond dimension 200 (blocks of up to 83 vectors, SMs to spare: 4 spreads the FP64
-// work over twice the SMs but makes twice the trips through L2), 21.7 against 23.3 ms
-// at 1024 (up to 294 vectors; 4 for the largest blocks only).
+// c = 896, 4 up to 1792, 2 up to 3584, 1 up to 7168).  8 against 4 in an SVD of
+// Heisenberg wavefunctions: 3.3 against 3.4 ms at bond dimension 200 (blocks of up to 83
+// vectors, SMs to spare: 4 spreads the FP64 work over twice the SMs but makes twice the
+// trips through L2), 21.7 against 23.3 ms at 1024 (up to 294 vectors; 4 for the largest
+// blocks only).  The narrow widths against jacobi_coop_kernel, SVD of one dense c x c
+// block, ms: 1700 (4) 496 | 1057, 1900 (2) 1090 | 1366, 2600 (2) 2604 | 5045, 3400 (2)
+// 5282 | 10021, 3700 (1) 14000 | 14869.
 int tnx_jacobi_block_width(int c) {
   if (c < 2) return 0;
   int w = W;

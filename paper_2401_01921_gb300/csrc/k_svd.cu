@@ -25,7 +25,8 @@
 // Blocks of 16 or more vectors go through a column-pivoted Householder QR
 // first and the sweeps run on the rows of its triangular factor (see the QR
 // preconditioning section below), done by the kernels of k_qr.cu and k_jacobi.cu
-// (qr_coop_kernel, jacobi_coop_kernel when a block is too long for them); the output has the same form.
+// (qr_coop_kernel, jacobi_coop_kernel when a block is too long or the blocks are too many for
+// them); the output has the same form.
 // All arithmetic is FP64.  Block reductions use a fixed order (deterministic).
 #include "tnx_fp64.cuh"
 #include "tnx_internal.h"

@@ -478,7 +478,8 @@ __global__ void __launch_bounds__(LT, 2) lanczos_step_kernel(LanczosDev L, int j
   const double* vj = L.V + (int64_t)j * L.n;
   const double* vp = L.V + (int64_t)(j > 0 ? j - 1 : 0) * L.n;
   double* part = L.partial;   // [nb] alpha (later the pass's norms), [nb] norms, [nb][j + 1] dots
-  // a wait that ran out: the solve stops, with an eigenvalue that is not a number
+  // a wait that ran out: the solve stops, with an eigenvalue that is not a number, and the
+  // call that waits for it fails (the status word of its network)
   auto give_up = [&](int code) {
     if (tid == 0) {
       *(volatile int32_t*)status = code;   // host memory (any of the codes will do)

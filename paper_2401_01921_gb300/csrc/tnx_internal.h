@@ -355,7 +355,7 @@ struct JbGroup {
   double* X;
   double* J;
   double* D;   // [c][4]: the factor of vector v (its rows of X and J count times it; 1 at first), its
-               // reciprocal, |x_v|^2, unused
+               // reciprocal, |x_v|^2 as carried and as last summed
   unsigned* ver;   // [nb]: rounds that each column block has been through, zeroed by the caller
   int32_t c, ld, nb, wmax;
 };
@@ -446,7 +446,8 @@ cudaError_t tnx_launch_lanczos_set_input(double** slot_ptr, const LanczosDev& L,
 // normalize = false leaves out v_{j+1} = w / beta_{j+1} (1 / beta_{j+1} is in
 // scratch[3 * nmax + 3]) for the caller to fuse with its next relayout;
 // always_pass: a Gram-Schmidt pass in every step (an operator far from symmetric);
-// *status receives 41..44 when a wait among the step's CTAs ran out (the solve stops)
+// *status (which may lie in host memory: it is only written) receives 41..44 when a wait
+// among the step's CTAs ran out (the solve stops)
 cudaError_t tnx_launch_lanczos_step(const LanczosDev& L, int j, double** next_slot, cudaStream_t st, bool normalize,
                                     bool always_pass, int32_t* status);
 cudaError_t tnx_launch_lanczos_finish(const LanczosDev& L, double* evec, cudaStream_t st);

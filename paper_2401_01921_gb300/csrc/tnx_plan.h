@@ -244,7 +244,8 @@ std::vector<int2> tnx_tf32_schedule(std::vector<SliceJob>& jobs);
 // the groups listed, a launch's tile edge or width chosen for all of them
 int tnx_f64_edge(const std::vector<GemmGroup>& groups, const std::vector<int>& which);
 std::vector<GemmTile> tnx_gemm_tiles(const std::vector<GemmGroup>& groups, const std::vector<int>& which, int edge);
-// runs of fused-step tiles from entries that hold whole bands; run gets the most tiles in one
+// fused-step tiles from entries that hold whole bands; lane_rows: the kernel that takes them
+// (tnx_launch_fused_skinny)
 std::vector<FusedTile> tnx_fused_tiles(const std::vector<FusedTile>& bands, int& lane_rows);
 // tke: K values of a tile; grid: the CTAs that walk the returned list (tnx_split.cpp)
 std::vector<GemmTile> tnx_split_schedule(const std::vector<GemmTile>& tiles, const std::vector<SplitGroup>& sg, int tke,

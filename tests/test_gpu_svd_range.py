@@ -1,11 +1,12 @@
 """GPU: the SVD of blocks whose squared norms lie at or beyond the end of the FP64 range, and of blocks with
-an infinity or a NaN: a singular value is right or not finite, and other charge blocks are untouched."""
+an infinity or a NaN: a singular value is right or not finite, and other charge blocks are untouched; and
+columns at the length that the QR's shared memory ends at."""
 import numpy as np
 import pytest
 
 import paper_2401_01921_gb300 as tnx
 from oracle.symtensor import IN, OUT, Bond as OB, BlockTensor
-from test_gpu_linalg import SYM, ctx, to_lib  # noqa: F401 (ctx is a fixture)
+from test_gpu_linalg import SYM, _check_svd, ctx, to_lib  # noqa: F401 (ctx is a fixture)
 from test_gpu_svd_blocks import _plain
 
 pytestmark = pytest.mark.gpu
@@ -59,3 +60,13 @@ def test_an_entry_that_is_no_number_stays_in_its_block(ctx, value):  # noqa: F81
     for s, q in ((got[0], (0, 0)), (got[2], (2, 2))):
         ref = np.linalg.svd(T.blocks[q], compute_uv=False)
         assert np.max(np.abs(s - ref)) <= 1e-12 * ref[0]
+
+
+# a slot of the QR holds nine columns, padded to 32 entries: 9 * 8 * 3200 bytes and its few words of state
+# fit 226 KB, 9 * 8 * 3232 do not (the step-by-step QR takes them)
+@pytest.mark.parametrize("rows", [3169, 3200, 3201])
+def test_longest_columns_in_shared_memory(ctx, rows):  # noqa: F811
+    holds = tnx.lib()._Z20tnx_qr_block_columnsi
+    assert holds(rows) == (8 if rows <= 3200 else 0)
+    rng = np.random.default_rng(rows)
+    _check_svd(ctx, _plain(rng.standard_normal((rows, 20)) * 10.0 ** (-4.0 * np.arange(20) / 20)), 1)
