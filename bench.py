@@ -53,11 +53,11 @@ SINGLE_THREAD_ENV = {"OPENBLAS_NUM_THREADS": "1", "OMP_NUM_THREADS": "1", "MKL_N
 # roofline.traffic only while the kernel source is unchanged, else null.
 SPLIT_TRAFFIC = {
     "heisenberg_u1_chi512_d2_D5_lanczos20":
-        (9305600, "profiles/split_gemm_heisenberg_u1_chi512.md",
-         "1edccaadeb9ebab7b4ab4b062a986006f94f024ad0ed51f81a11861a747bc22f"),
+        (9320576, "profiles/split_gemm_heisenberg_u1_chi512.md",
+         "c004a39dbb2a3be8fdbbc08f355ec2673bdcfa35037953ec66818ab98bdfa9fc"),
     "heisenberg_u1_chi2048_d2_D5_sectorscaled_lanczos20":
-        (90162944, "profiles/split_gemm_heisenberg_u1_chi2048.md",
-         "3881178b94e7b3c07d3657f48af6a1640532fa838379ab8ed0827a232525ae31"),
+        (90473088, "profiles/split_gemm_heisenberg_u1_chi2048.md",
+         "c004a39dbb2a3be8fdbbc08f355ec2673bdcfa35037953ec66818ab98bdfa9fc"),
 }
 
 
