@@ -201,7 +201,7 @@ extern "C" tnx_status tnx_ctx_create(int device, void* stream, tnx_alloc_fn allo
     c->scratch = new DevBuf(c, 64 * 1024);
     c->pinned = nullptr;
     CUDA_CHECK(cudaMallocHost(&c->pinned, 4096));
-    c->status_release(c->status_lease());   // the first block of status words
+    c->status_own = c->status_lease();
   });
   if (s != TNX_OK) {
     delete c;
@@ -237,10 +237,11 @@ StatusWord* tnx_ctx::status_lease() {
   return w;
 }
 
-// An unread code stays in the word: check_device_status looks at free words too.
+// An unread code goes to the context's own word: the next holder of this one starts clean.
 void tnx_ctx::status_release(StatusWord* w) {
   if (!w) return;
   std::lock_guard<std::mutex> lock(status_mu);
+  if (const int code = tnx_status_take(w)) status_own->code = code;
   w->served.store(0);
   status_free.push_back(w);
 }

@@ -53,6 +53,7 @@ struct tnx_ctx {
   std::mutex status_mu;
   std::vector<StatusWord*> status_blocks;   // pinned blocks of kStatusBlock words
   std::vector<StatusWord*> status_free;
+  StatusWord* status_own = nullptr;         // codes that their network or batch left unread
   static constexpr int kStatusBlock = 256;
   StatusWord* status_lease();
   void status_release(StatusWord* w);

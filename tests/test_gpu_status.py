@@ -49,9 +49,15 @@ def test_a_direct_call_reports_and_clears(ctx):  # noqa: F811
         ctx.sync()
         assert tnx.lanczos(net, "psi", T["psi"], 10) == alone
     # a network destroyed with an unread code leaves it to the next synchronisation
+    # ... not to the network that is created next
     _expire(net, 42)
     del net, call, e
     gc.collect()
-    with pytest.raises(tnx.TnxError):
+    net, T, B = lib_heff(ctx, I.heisenberg_workload(64, 10), symmetric=True)
+    srv = tnx.Server(ctx, max_slots=1)
+    assert srv.wait(srv.submit(net, "psi", T["psi"], tnx.REQ_LANCZOS, 10), 60000)[:2] == alone
+    srv.close()
+    with pytest.raises(tnx.TnxError) as e:
         ctx.sync()
+    assert "site 42" in str(e.value)
     ctx.sync()
