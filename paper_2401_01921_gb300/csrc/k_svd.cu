@@ -37,6 +37,14 @@ using tnx_fp64::warp_sum_double;
 
 constexpr int JT = 256;   // threads per pair
 
+// A product of two squared norms far from both ends of the FP64 range: squares of dot
+// products can be compared with it.  Outside (vectors beyond 1e72 or below 1e-72 in length)
+// both sides would overflow or vanish and every pair would count as orthogonal.
+__device__ __forceinline__ bool mid_range(double ab) {
+  const int e = (__double2hiint(ab) >> 20) & 0x7FF;
+  return e > 64 && e < 1984;
+}
+
 __device__ __forceinline__ double block_sum3(double& a, double& b, double& c, double* sh) {
   // three sums at once over the CTA, fixed order; results broadcast in a, b, c
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -99,7 +107,7 @@ __global__ void __launch_bounds__(JT) jacobi_round_kernel(const SvdGroup* __rest
     if (threadIdx.x == 0) {
       int skip = 1;
       if (a > 0.0 && b > 0.0) {
-        const double off = fabs(c) / sqrt(a * b);
+        const double ab = a * b, off = mid_range(ab) ? fabs(c) / sqrt(ab) : fabs(c) / sqrt(a) / sqrt(b);
         atomicMax(maxoff, (unsigned long long)__double_as_longlong(off));
         if (off > 1e-15) {
           skip = 0;
@@ -242,13 +250,20 @@ __device__ __forceinline__ void jacobi_pair(const SvdGroup& g, int p, int q, int
   // squared relative off-diagonal; the same tests as |gamma| / sqrt(alpha beta)
   // against 1e-15 and tol, with one FP64 division instead of a root and two
   const double ab = a * b, c2 = c * c;
-  off_w = fmax(off_w, c2 / ab);
-  if (c2 <= 1e-30 * ab) return;
+  const bool mid = mid_range(ab);
+  if (mid) {
+    off_w = fmax(off_w, c2 / ab);
+    if (c2 <= 1e-30 * ab) return;
+  } else {
+    const double o = c / sqrt(a) / sqrt(b);
+    off_w = fmax(off_w, o * o);
+    if (!(o * o > 1e-30)) return;
+  }
   // t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)) with zeta = d / (2 gamma), d = beta - alpha,
   // multiplied through by 2 |gamma|: one root, one division and one reciprocal root
   const double d = b - a;
   double t;
-  if (fabs(d) < 1e150 && fabs(c) < 1e150) {
+  if (mid && fabs(d) < 1e150 && fabs(c) < 1e150) {
     t = 2.0 * c / (d + copysign(sqrt(fma(d, d, 4.0 * c2)), d));
   } else {   // squares out of range: the quotient form
     const double zeta = d / (2.0 * c), az = fabs(zeta);

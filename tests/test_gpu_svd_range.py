@@ -70,3 +70,16 @@ def test_longest_columns_in_shared_memory(ctx, rows):  # noqa: F811
     assert holds(rows) == (8 if rows <= 3200 else 0)
     rng = np.random.default_rng(rows)
     _check_svd(ctx, _plain(rng.standard_normal((rows, 20)) * 10.0 ** (-4.0 * np.arange(20) / 20)), 1)
+
+
+# blocks of fewer than 16 vectors: no QR, the sweeps run on the block itself
+@pytest.mark.parametrize("scale", [1e-140, 1e-75, 1e-70, 1e70, 1e75, 1e140])
+def test_small_blocks_far_from_one(ctx, scale):  # noqa: F811
+    rng = np.random.default_rng(14)
+    secs, secs2 = [((0,), 9), ((1,), 2), ((2,), 15)], [((0,), 12), ((1,), 3), ((2,), 4)]
+    T = BlockTensor([OB.make(IN, secs, SYM), OB.make(OUT, secs2, SYM)])
+    for q in T.keys():
+        T.blocks[q] = rng.standard_normal(T.block_shape(q)) * scale
+    for s, q in zip(_values(ctx, T), sorted(T.keys())):
+        ref = np.linalg.svd(T.blocks[q], compute_uv=False)
+        assert np.max(np.abs(s - ref)) <= 1e-13 * ref[0]
